@@ -523,8 +523,8 @@ lsq_status lsq_features(const double* A, int64_t m, int64_t n, int64_t lda, uint
 /* MLP in FP32 on the device.  forward: logits (batch x 4) for X (batch x d,
  * row-major).  backward: gradient of the mean softmax cross-entropy against
  * labels (0 FP8-e4m3, 1 BF16, 2 FP32, 3 FP64) in the parameter packing, and
- * the loss (device float, may be NULL); sums over the batch run in sample
- * order (deterministic).  adam: one Adam step (step counts from 1). */
+ * the loss (device float, may be NULL); sums over the batch run over chunks
+ * of 32 samples and then over the chunks, in a fixed order (deterministic).  adam: one Adam step (step counts from 1). */
 lsq_status lsq_mlp_forward(const float* params, int32_t d, int32_t batch, const float* X, float* logits,
                            void* stream);
 size_t lsq_mlp_backward_workspace_size(int32_t d, int32_t batch);

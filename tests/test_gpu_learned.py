@@ -38,6 +38,21 @@ def test_mlp_forward_and_gradient_match_oracle():
     assert np.linalg.norm(g - go) <= 1e-4 * np.linalg.norm(go)
 
 
+@pytest.mark.parametrize("d,B", [(1, 1), (10, 31), (10, 32), (10, 33), (10, 4096), (70, 100)])
+def test_mlp_gradient_chunk_edges(d, B):
+    """The gradient's chunks of 32 samples and any feature count against the
+    oracle: an FP32 sum of B terms over 64-term dot products, so 1e-4 of the
+    gradient's norm (a few hundred FP32 roundings)."""
+    rng = np.random.default_rng(100 * d + B)
+    p = (rng.standard_normal(O.mlp_param_count(d)) * 0.2).astype(np.float32)
+    X = rng.standard_normal((B, d)).astype(np.float32)
+    y = rng.integers(0, 4, B).astype(np.int32)
+    g, loss = lsq.mlp_backward(torch.from_numpy(p).cuda(), torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda())
+    lo_loss, go = O.mlp_backward(p.astype(np.float64), X.astype(np.float64), y)
+    assert abs(float(to_np(loss)[0]) - lo_loss) <= 1e-5 * max(1.0, lo_loss)
+    assert np.linalg.norm(to_np(g).astype(np.float64) - go) <= 1e-4 * np.linalg.norm(go)
+
+
 def test_features_match_oracle():
     for (m, n, kap) in [(3000, 50, 1e3), (2048, 128, 1e8), (700, 20, 10.0)]:
         pr = P.make_problem(m, n, kap, 0.0, 5)
