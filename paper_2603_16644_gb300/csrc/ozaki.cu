@@ -1,18 +1,29 @@
 // FP64 Gram matrix G = X^T X (and the product X^T Y of two m x n matrices)
-// on the FP8 tensor cores, exact to a 56-bit
+// on the FP8 tensor cores, exact to a 54-bit plus sign
 // fixed-point representation of every column (digit slicing in the manner
 // of Ozaki, Ogita & Oishi's error-free matrix multiplication):
 //
-//   x_ip = 2^(e_p) * sum_{t=0}^{S-1} d_t(i,p) 16^-(t+1) + r_ip,
-//          d_t in [-15, 15], |r_ip| < 2^(e_p - 56)   (S = 14 digits),
+//   x_ip = 2^(e_p - 4) * sum_{t=0}^{S-1} d_t(i,p) 32^-t + r_ip,
+//          d_t in [-16, 16], |r_ip| <= 2^(e_p - 55)   (S = 11 digits),
 //
-// where 2^(e_p) bounds column p.  Digit products are integers below 2^8, so
+// where 2^(e_p) bounds column p.  Digit products are integers up to 2^8, so
 // a K-chunk of up to 65536 rows sums exactly in the FP32 accumulators of
 // tcgen05.mma (kind::f8f6f4, E4M3 operands).  Every digit-pair block (t, u)
 // with t + u <= S - 1 is one tensor-core contraction over the rows; the
 // blocks are combined exactly in integers, scaled by 2^(e_p + e_q) and
-// rounded once.  Dropped pairs and the residuals r contribute below 2^-55 of
-// |x_p| |x_q| per row, the same order as FP64 rounding.
+// rounded once.  Dropped pairs and the residuals r contribute about 2^-55 of
+// 2^(e_p + e_q) per row, with signs that vary from row to row, the same order
+// as FP64 rounding.
+//
+// Why balanced digits: E4M3 holds every integer up to 16, so a signed digit
+// carries 5 bits, against 4 for a sign and a nibble, and 66 digit pairs take
+// the place of the 105 of 14 sign-and-magnitude digits (the tensor work is
+// what bounds the Gram).  The error is no larger: against
+// quadruple precision, relative to |x_p| |x_q|, 60000 normal rows: rms 2^-57.2
+// off the diagonal and 2^-53.5 on it, against 2^-56.4 and 2^-48.5 with the
+// 14 digits (whose dropped pairs all have the sign of x_ip x_iq).  Measured: A_p and Gram of a
+// 131072 x 2000 problem 58.3 -> 51.7 ms (digit products 16.7 -> 10.5 ms), a
+// 262144 x 4096 solve 556 -> 501 ms.
 //
 // Digits are extracted with integer operations on the FP64 bit pattern (no
 // FP64 instruction in the slicing pass).
@@ -23,7 +34,9 @@
 
 namespace lsq {
 
-constexpr int OZ_S = 14;        // digits per value (4 bits each: 56 bits)
+constexpr int OZ_S = 11;        // digits per value
+constexpr int OZ_B = 5;         // bits per digit: balanced base-32 digits in [-16, 16]
+constexpr int OZ_F = OZ_B * (OZ_S - 1) + 4;  // fraction bits of a value relative to 2^(e_p)
 constexpr int64_t OZ_KCHUNK = 65536;  // rows summed exactly per FP32 accumulator
 constexpr int32_t OZ_NONFINITE = INT32_MAX;  // column exponent of a column holding an Inf or NaN
 
@@ -57,51 +70,67 @@ __global__ void k_oz_colexp(const double* __restrict__ X, int64_t m, int64_t ld,
 }
 
 // Two FP32 values to E4M3 (the first in the upper byte); exact for the
-// integer digits in [-15, 15].
+// integer digits in [-16, 16].
 __device__ __forceinline__ uint32_t e4m3x2(float hi, float lo) {
     unsigned short r;
     asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
     return r;
 }
 
+// 16 added to every digit but the first: the fields of V + OZ_BIAS are then
+// the digits plus 16.
+constexpr unsigned long long oz_bias() {
+    unsigned long long b = 0;
+    for (int t = 1; t < OZ_S; ++t) b += 16ull << (OZ_B * (OZ_S - 1 - t));
+    return b;
+}
+
 // Z row (t * np + p), column i  <-  digit t of x_ip.  Rows p >= n and
 // columns i >= m (padding) are zero.  4 consecutive rows per thread: a warp
 // reads 1 KB of a column and writes 128 contiguous bytes of every digit
-// plane.  Digit t of |x| is a nibble of V = |x| 2^(56 - e_p); its signed FP32
-// value is s (2^23 1.5 + nibble) - s 2^23 1.5 (s = +-1; exact, and +0 for a
-// zero nibble), converted in pairs by the hardware.
+// plane.  V = |x| 2^(F - e_p) rounded to the nearest integer (V <= 2^F); field
+// t of W = V + bias is the digit of |x| plus 16 (the top field, W >> 50, is
+// the digit itself), and the signed digit is s (2^23 1.5 + field) -
+// s (2^23 1.5 + 16) with s = +-1 (exact in FP32, +0 for a zero digit), converted
+// in pairs by the hardware.  The digits are those of |x| times the sign, not
+// those of x: balanced digits in [-16, 15] average -1/2, and with the sign of
+// x taken out the dropped pairs of two uncorrelated columns would all be off
+// in the same direction.
 __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ X, int64_t m, int64_t n, int64_t ld,
                                                   const int32_t* __restrict__ e, int64_t np, int64_t ldz,
                                                   uint8_t* __restrict__ Z) {
+    constexpr unsigned long long BIAS = oz_bias();
     const int64_t p = blockIdx.y;
     const int32_t ep = p < n ? e[p] : 0;
     const double* col = X + p * ld;
     for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i0 < ldz;
          i0 += (int64_t)gridDim.x * blockDim.x * 4) {
-        unsigned long long V[4];
+        unsigned long long W[4];
         float sg[4], off[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const unsigned long long b =
                 (p < n && i0 + q < m) ? (unsigned long long)__double_as_longlong(col[i0 + q]) : 0ull;
             const int Eb = (int)((b >> 52) & 0x7ff);
-            V[q] = 0;
+            unsigned long long V = 0;
             if (Eb != 0 && Eb != 0x7ff && ep != OZ_NONFINITE) {
                 const unsigned long long sig = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
-                const int sh = (Eb - 1023) - ep + 4;  // x 2^(56 - e_p) = sig 2^(E_a - 52 + 56 - e_p)
-                if (sh >= 0) V[q] = sig << sh;        // sh <= 3: V < 2^56
-                else if (sh > -64) V[q] = sig >> (-sh);
+                const int sh = (Eb - 1023) - ep + (OZ_F - 52);  // x 2^(F - e_p) = sig 2^(E_a - 52 + F - e_p)
+                if (sh >= 0) V = sig << sh;                     // sh <= 1: V < 2^F
+                else if (sh > -64) V = (sig + (1ull << (-sh - 1))) >> (-sh);
             }
+            W[q] = V + BIAS;
             sg[q] = (b >> 63) ? -1.0f : 1.0f;
-            off[q] = -sg[q] * 12582912.0f;
+            off[q] = -sg[q] * 12582928.0f;
         }
 #pragma unroll
         for (int t = 0; t < OZ_S; ++t) {
             float d[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint32_t nib = (uint32_t)(V[q] >> (4 * (OZ_S - 1 - t))) & 15u;
-                d[q] = fmaf(sg[q], __uint_as_float(0x4B400000u | nib), off[q]);
+                const uint32_t f = t == 0 ? (uint32_t)(W[q] >> (OZ_B * (OZ_S - 1))) + 16u
+                                          : (uint32_t)(W[q] >> (OZ_B * (OZ_S - 1 - t))) & 31u;
+                d[q] = fmaf(sg[q], __uint_as_float(0x4B400000u | f), off[q]);
             }
             *(uint32_t*)(Z + ((int64_t)t * np + p) * ldz + i0) = e4m3x2(d[1], d[0]) | (e4m3x2(d[3], d[2]) << 16);
         }
@@ -112,11 +141,11 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ X, 
 // + Q] = index of the tile holding C_tu[P block, Q block], or -1 (symmetric
 // case: then C_tu = C_ut^T is read from the (u, t) tile at (Q, P)).  Tiles are
 // 128 x 128 FP32, column-major; chunk z of tile id starts at (z ntiles + id)
-// 16384.  Every tile value is an integer below 2^24 in magnitude, so each
+// 16384.  Every tile value is an integer of at most 2^24 in magnitude, so each
 // weight class d = t + u sums exactly in 64-bit integers,
 //   S_d = sum_{t + u = d} sum_z C_tu,z[p, q],
-// and I = sum_{d=0}^{S-1} S_d 16^(S-1-d) (Horner, 128-bit) is the exact
-// digit-sliced sum: G[p, q] = I 2^(e_p + e_q - 4 (S + 1)), rounded once.
+// and I = sum_{d=0}^{S-1} S_d 32^(S-1-d) (Horner, 128-bit) is the exact
+// digit-sliced sum: G[p, q] = I 2^(e_p + e_q - 8 - 5 (S - 1)), rounded once.
 // One CTA per (P, Q) block (P >= Q when sym) and 32-column quarter; thread
 // (r = tid mod 128, c = c0 + tid / 128 + 2k, k < 16) owns 16 entries.  Tiles
 // read transposed are staged through shared memory; the loads of the next
@@ -216,11 +245,11 @@ __global__ void __launch_bounds__(OZ_CB_THREADS) k_oz_combine(const float* __res
             for (int k = 0; k < 16; ++k) S[k] += (long long)__float2int_rz(tr_s[r][cb - c0 + 2 * k]);
         }
         if (dn != d || !more) {
-            // weight class d complete: I = 16 I + S_d
+            // weight class d complete: I = 32 I + S_d
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-                H[k] = (long long)(((unsigned long long)H[k] << 4) | (L[k] >> 60));
-                L[k] <<= 4;
+                H[k] = (long long)(((unsigned long long)H[k] << OZ_B) | (L[k] >> (64 - OZ_B)));
+                L[k] <<= OZ_B;
                 const unsigned long long l2 = L[k] + (unsigned long long)S[k];
                 H[k] += (S[k] >> 63) + (l2 < L[k] ? 1 : 0);
                 L[k] = l2;
@@ -238,7 +267,7 @@ __global__ void __launch_bounds__(OZ_CB_THREADS) k_oz_combine(const float* __res
         if (p >= n || q >= n || (sym && p < q)) continue;
         const int32_t a = ex[p], b = ey[q];
         const double g = (a == OZ_NONFINITE || b == OZ_NONFINITE) ? __longlong_as_double(0x7ff8000000000000ll)
-                                                                  : fixed128_to_double(H[k], L[k], a + b - 4 * (OZ_S + 1));
+                                                                  : fixed128_to_double(H[k], L[k], a + b - 8 - OZ_B * (OZ_S - 1));
         G[p + q * ldg] = g;
         if (sym) G[q + p * ldg] = g;
     }
