@@ -214,6 +214,34 @@ def test_lu_solve(n):
     assert np.linalg.norm(to_np(x) - x_o) / np.linalg.norm(x_o) <= 8 * n * U64 * kH
 
 
+@pytest.mark.parametrize("n", [31, 32, 65, 129, 257, 520, 1030, 2100])
+def test_lu_panel_rows_per_cluster(n):
+    """The panel's cluster sizes (1 to 16 CTAs), rows per CTA and ragged last
+    panels: the oracle's pivots, and factors within the bound of test_lu_solve;
+    duplicate magnitudes in a column take the first largest pivot."""
+    rng = np.random.default_rng(300 + n)
+    H = rng.standard_normal((n, n)) + np.diag(np.full(n, 0.5))
+    H[:, 0] = np.where(rng.random(n) < 0.5, -2.0, 2.0)  # ties in the first column
+    c = rng.standard_normal(n)
+    LU_o, piv_o, info_o = O.lu(H)
+    x, F, piv, info = lsq.factor_solve(dev_colmajor(H), torch.from_numpy(c).cuda(), hpne=True)
+    assert int(to_np(info)[0]) == 0 == info_o
+    np.testing.assert_array_equal(to_np(piv), piv_o)
+    kH = O.kappa(H)
+    assert np.linalg.norm(to_np(F) - LU_o) / np.linalg.norm(LU_o) <= 8 * n * U64 * kH
+
+
+@pytest.mark.parametrize("n", [1, 40, 300])
+def test_lu_zero_pivot_reported(n):
+    """A zero column breaks down at its own index on both sides."""
+    rng = np.random.default_rng(n)
+    H = rng.standard_normal((n, n))
+    H[:, n // 2] = 0.0
+    _, _, info_o = O.lu(H)
+    _, _, _, info = lsq.factor_solve(dev_colmajor(H), torch.ones(n, dtype=torch.float64).cuda(), hpne=True)
+    assert int(to_np(info)[0]) == info_o == n // 2 + 1
+
+
 def test_solve_wait_timeout_reports_and_recovers():
     """Fault injected on the host side (no GPU fault): with the test-only wait
     bound of the triangular solves cut to 1 ns, the blocks that find their
