@@ -40,7 +40,10 @@ constexpr int OT_BM = 128, OT_BN = 64;      // output tile (rows x columns)
 constexpr int OT_BK = 64;                   // K per stage: 64 BF16 = 128 bytes
 constexpr int OT_XST = 6;                   // stages of X digit tiles
 constexpr int OT_KMAX = 512;                // exact FP32 group sums up to this K
-constexpr int OT_KMAX3 = 1024;              // the same with three X digits (at most 3 pairs per group)
+// With three X digits (at most 3 pairs per group) the FP32 sums would be exact
+// up to K = 1024; the 64-bit sums of k_ot_update2, K 2^53 (1 + 2/128 + ...) in
+// magnitude, bound K to 1003: 15 slabs of 64.
+constexpr int OT_KMAX3 = 960;
 constexpr int OT_NB = 32;                   // diagonal block solved by substitution
 constexpr int OT_THREADS = 608;             // warp 0 TMA, warps 1-2 MMA, warps 3-18 epilogue
 constexpr int OT_XTILE = OT_BM * 128;       // bytes of one X digit tile
@@ -660,6 +663,386 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------
+// The same update by pairs of CTAs (cta_group::2): 256 x 128 output tiles, the
+// form of the updates with enough tiles to fill the chip.
+//
+// What bounded the 128 x 64 tiles: shared-memory bandwidth.  With all 8 group
+// accumulators in TMEM a tile can be no wider than 64 columns, and a 128 x 64
+// x 16 MMA reads 6 KB of operands (48 cycles of shared memory) for 32 cycles
+// of tensor work, the TMA's writes on top: 0.55 of the tensor peak at best,
+// 1.03 PFLOP/s measured.  Here a pair of CTAs owns 256 x 128 outputs, each CTA
+// holding 128 rows of X and half of the Y columns in shared memory (6 KB per
+// 64 cycles), and the groups are formed two at a time: four passes over K, pass
+// p accumulating groups 2p and 2p + 1 in one half of TMEM (2 x 128 columns)
+// while the epilogue drains the other half.  A pass walks the digit tiles in a
+// zigzag: stage t holds X digit t and Y digit (2p + 1) - t; X digit t meets Y
+// digit 2p + 1 - t (group 2p + 1) and Y digit 2p - t of the next stage (group
+// 2p), so that every tile loaded is used by two products (52 bytes a cycle and
+// SM from L2).  Two warps issue, one per accumulator (one warp alone took ~98
+// cycles per MMA of 64).  The epilogue keeps the exact sum as one 64-bit integer
+// per output over the passes, sum_{d<=5} S_d 128^(5-d) and then 6 more bits, and
+// the last 8 bits of the 71 packed four to a register: all of TMEM is read
+// before the conversion to FP64 starts, which then overlaps the next tile's
+// first passes (converting while the last half of TMEM was held cost 78 of 210
+// thousand cycles a tile).  Rounded once: the same bits as the 128 x 64 form.
+// Measured, 131072 x 512 x 1488: 83 thousand cycles for each 128 x 64 tile of one
+// SM before, 100 thousand for the 128 x 128 of one here (74 of them tensor
+// work).  A_p and Gram of a 131072 x 2000 problem 51.7 -> 44.9 ms, its FP64
+// Gaussian sketch 54.8 -> 44.8 ms, a 262144 x 4096 solve 501 -> 441 ms.
+// ---------------------------------------------------------------------------
+constexpr int O2_BM = 256, O2_BN = 128;       // output tile of the CTA pair
+constexpr int O2_ST = 8;                      // ring stages
+constexpr int O2_XB = 128 * 128, O2_YB = 64 * 128;  // bytes of an X / Y digit tile in one CTA
+constexpr int O2_STAGE = O2_XB + O2_YB;
+constexpr int O2_EPI_WARPS = 16;
+constexpr int O2_EC = 32;  // columns per epilogue warp
+constexpr int O2_THREADS = 32 * (4 + O2_EPI_WARPS);  // warp 0 TMA, warps 1-2 MMA, warp 3 idle, warps 4-19 epilogue
+// Registers: 640 threads launch with 96 each; the first warpgroup keeps 32 and
+// the epilogue's four take 112 (128 * 32 + 512 * 112 = 640 * 96), so that the 32
+// sums of a thread (72 registers) stay in registers: with 200 KB of shared
+// memory in use the L1 that is left cannot hold spills.  16 warps and not 8
+// with twice the columns: the conversion is a chain of integer operations, and
+// 8 warps left it bound by their latency.
+constexpr int O2_REG_LO = 32, O2_REG_HI = 112;
+
+// 2^s (256 S + low) for |S| < 2^63, 0 <= low < 256, rounded once to
+// nearest-even.  The magnitude is normalised to 64 bits (top bit set, the bits
+// below it in `sticky`), the significand rounded off its upper 53, and added to
+// the exponent field, so that a carry moves to the next binade by itself.
+// Results outside the normal range (rare) are scaled by exact powers of two
+// (inlined: a call would spill the sums held in registers; the FP64 pipe takes
+// 16 cycles an instruction and SM, so that running these products for every
+// value and selecting cost three times the conversion).
+__device__ __forceinline__ double o2_pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
+
+__device__ __forceinline__ double o2_fixed_to_double(long long S, unsigned low, int s) {
+    const bool neg = S < 0;
+    // magnitude: -(256 S + low) = 256 (~S) + (256 - low)
+    unsigned lo = neg ? 256u - low : low;  // 1 .. 256 when negative
+    unsigned long long hi = (unsigned long long)(neg ? ~S : S) + (lo >> 8);
+    lo &= 255u;
+    const bool small = hi == 0;  // below 2^8: 256 times as large a unit
+    hi = small ? (unsigned long long)lo : hi;
+    lo = small ? 0u : lo;
+    const int z = __clzll((long long)hi);  // 64 only when the value is 0
+    const unsigned long long n = (hi << (z & 63)) | ((((unsigned long long)lo << 56) >> 1) >> ((63 - z) & 63));
+    const bool sticky = z < 8 && (lo & ((1u << (8 - z)) - 1u)) != 0;
+    const unsigned rem = (unsigned)n & 0x7ffu;
+    unsigned long long mant = n >> 11;
+    mant += (rem > 0x400u || (rem == 0x400u && (sticky || (mant & 1ull)))) ? 1ull : 0ull;
+    const int E = 71 - z + s + 1023 - (small ? 8 : 0);  // exponent field of a magnitude in [2^(71-z), 2^(72-z))
+    const unsigned long long sgn = neg ? 0x8000000000000000ull : 0ull;
+    double r = __longlong_as_double((long long)((((unsigned long long)(unsigned)(E - 1) << 52) + mant) | sgn));
+    if ((unsigned)(E - 1) >= 2045u) {
+        r = __longlong_as_double((long long)(((1022ull << 52) + mant) | sgn));
+        int e = E - 1023;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int k = max(-1000, min(1000, e));
+            asm volatile("mul.rn.f64 %0, %0, %1;" : "+d"(r) : "d"(o2_pow2(k)));  // volatile: not run speculatively
+            e -= k;
+        }
+    }
+    return hi == 0 ? 0.0 : r;
+}
+
+// Stages of pass p: X digits t < XD with a partner, and the Y digit that only
+// group 2p needs when the X digits end before it.
+__host__ __device__ constexpr int o2_stages(int XD, int p) { return 2 * p + 1 < XD ? 2 * p + 2 : XD + 1 < 2 * p + 2 ? XD + 1 : 2 * p + 2; }
+
+// Tile t -> (first row, first column), as ot_tile_coords.
+template <bool GROUPED>
+__device__ __forceinline__ void o2_tile_coords(int t, int ntj, int nti, int64_t& i0, int64_t& j0) {
+    constexpr int GM = OT_GM * OT_BM / O2_BM;
+    if (!GROUPED) {
+        i0 = (int64_t)(t / ntj) * O2_BM;
+        j0 = (int64_t)(t % ntj) * O2_BN;
+        return;
+    }
+    const int per = GM * ntj;
+    const int first = (t / per) * GM;
+    const int gs = min(nti - first, GM);
+    const int w = t % per;
+    i0 = (int64_t)(first + w % gs) * O2_BM;
+    j0 = (int64_t)(w / gs) * O2_BN;
+}
+
+template <int XD>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(O2_THREADS, 1)
+    k_ot_update2(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, int64_t m,
+                 int64_t N, int64_t K, const int32_t* __restrict__ Ex, const int32_t* __restrict__ Ey,
+                 const double* Cin, int64_t ldi, double* Cout, int64_t ldo, int32_t* __restrict__ err, int ntj,
+                 int ntiles) {
+    extern __shared__ unsigned char o2_raw[];
+    uint8_t* base = (uint8_t*)(((uintptr_t)o2_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = (uint64_t*)(base + O2_ST * O2_STAGE);  // leader CTA: both CTAs' copies of a stage have landed
+    uint64_t* empty = full + O2_ST;    // each CTA: the MMAs have read a stage
+    uint64_t* accf = empty + O2_ST;    // each CTA: a pass's sums are complete (2 TMEM halves)
+    uint64_t* tfree = accf + 2;        // leader CTA: both CTAs' epilogues have read a half
+    uint64_t* mdone = tfree + 2;       // leader CTA: every MMA has completed
+    uint32_t* tslot = (uint32_t*)(mdone + 1);
+    volatile int* bad = (volatile int*)(tslot + 1);
+    int* cnt = (int*)(tslot + 2);      // leader CTA: stages issued, consumed by issuers 0 and 1
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
+    const int nslab = (int)((K + OT_BK - 1) / OT_BK);
+    const int ntl = ntiles > pair ? (ntiles - pair + npairs - 1) / npairs : 0;
+    const int nti = ntiles / ntj;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < O2_ST; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 2);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&accf[s], 2);
+            mbar_init(&tfree[s], 2 * O2_EPI_WARPS);
+        }
+        mbar_init(mdone, 2);
+        *bad = 0;
+        cnt[0] = cnt[1] = cnt[2] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) tmem_alloc2(tslot, 512);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    cluster_sync_all();  // barriers of both CTAs initialised, TMEM of both allocated
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tslot;
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(O2_REG_LO));
+        if (warp == 0 && lane == 0) {
+            // producer (both CTAs): its own rows of X and its own half of the Y
+            // columns, signalled to the leader's barrier
+            int q = 0;
+            for (int i = 0; i < ntl && !*bad; ++i) {
+                int64_t i0, j0;
+                o2_tile_coords<XD == 3>(pair + i * npairs, ntj, nti, i0, j0);
+                for (int p = 0; p < 4 && !*bad; ++p) {
+                    const int ns = o2_stages(XD, p), g1 = 2 * p + 1;
+                    for (int s = 0; s < nslab && !*bad; ++s) {
+                        for (int t = 0; t < ns; ++t, ++q) {
+                            const int st = q & (O2_ST - 1);
+                            if (q >= O2_ST && !mbar_wait(&empty[st], (uint32_t)(((q / O2_ST) - 1) & 1))) {
+                                *bad = 1;
+                                break;
+                            }
+                            uint8_t* sx = base + st * O2_STAGE;
+                            const uint32_t fb = mapa_u32(smem_u32(&full[st]), 0);
+                            if (rank == 0) {
+                                mbar_expect_tx(&full[st], 2u * (uint32_t)(t < XD ? O2_STAGE : O2_YB));
+                                cnt[0] = q + 1;
+                            }
+                            if (t < XD) tma_load_3d_cg2(sx, &tmX, fb, s * OT_BK, (int)i0 + 128 * (int)rank, t);
+                            tma_load_3d_cg2(sx + O2_XB, &tmY, fb, s * OT_BK, (int)j0 + 64 * (int)rank, g1 - t);
+                        }
+                    }
+                }
+            }
+        } else if ((warp == 1 || warp == 2) && rank == 0) {
+            // MMA issuers (leader CTA): issuer 1 group 2p + 1 (X digit t with the Y
+            // digit of its stage), issuer 0 group 2p (with the Y digit of the next
+            // stage).  Each warp runs in convergence, lane 0 issues (see
+            // k_ot_update); the 4 K steps of one pair go back to back into one
+            // accumulator.  Both commit every stage and pass.
+            const uint32_t lead = lane == 0 ? 1u : 0u;
+            constexpr uint32_t idesc = umma_idesc(1u, O2_BM, O2_BN);
+            const uint64_t d0 = umma_desc(smem_u32(base));
+            int q = 0, ab = 0;
+            auto pass = [&](auto pc, auto issc) -> bool {
+                constexpr int p = decltype(pc)::value;
+                constexpr int ISS = decltype(issc)::value;
+                constexpr int ns = o2_stages(XD, p);
+                const int buf = ab & 1;
+                if (ab >= 2 && !__all_sync(0xffffffffu, mbar_wait(&tfree[buf], (uint32_t)(((ab >> 1) - 1) & 1)))) return false;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t acc = tmem + (uint32_t)((buf * 2 + ISS) * O2_BN);
+                for (int s = 0; s < nslab; ++s, q += ns) {
+                    // 16-wide K steps past K (zero digits) are not issued
+                    const int64_t krem = K - (int64_t)s * OT_BK;
+                    const uint32_t lk[4] = {lead, krem > 16 ? lead : 0u, krem > 32 ? lead : 0u, krem > 48 ? lead : 0u};
+#pragma unroll
+                    for (int t = 0; t < ns; ++t) {
+                        // issuer 0 needs the stage after t (stage 0 with it at first)
+                        const int w = ISS ? t : t + 1;
+                        if (!ISS && t == 0 &&
+                            !__all_sync(0xffffffffu, mbar_wait(&full[q & (O2_ST - 1)], (uint32_t)((q / O2_ST) & 1))))
+                            return false;
+                        if (w < ns) {
+                            const int qw = q + w;
+                            if (!__all_sync(0xffffffffu, mbar_wait(&full[qw & (O2_ST - 1)], (uint32_t)((qw / O2_ST) & 1))))
+                                return false;
+                            if (lead) cnt[1 + ISS] = qw + 1;
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            if (t < XD) {
+                                const uint64_t ad = d0 + (uint64_t)(((q + t) & (O2_ST - 1)) * (O2_STAGE >> 4));
+                                const uint64_t bd = d0 + (uint64_t)(((qw & (O2_ST - 1)) * O2_STAGE + O2_XB) >> 4);
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)
+                                    umma_f16_cg2_w(acc, ad + 2 * kk, bd + 2 * kk, idesc, (s | t | kk) != 0 ? 1u : 0u, lk[kk]);
+                            }
+                        }
+                        umma_commit_cg2_w(&empty[(q + t) & (O2_ST - 1)], lead);
+                    }
+                }
+                umma_commit_cg2_w(&accf[buf], lead);
+                ++ab;
+                return true;
+            };
+            auto issue = [&](auto issc) {
+                for (int i = 0; i < ntl; ++i) {
+                    if (__shfl_sync(0xffffffffu, *bad, 0)) break;
+                    if (!(pass(std::integral_constant<int, 0>(), issc) && pass(std::integral_constant<int, 1>(), issc) &&
+                          pass(std::integral_constant<int, 2>(), issc) && pass(std::integral_constant<int, 3>(), issc))) {
+                        *bad = 1;
+                        break;
+                    }
+                }
+            };
+            if (warp == 1) issue(std::integral_constant<int, 0>());
+            else issue(std::integral_constant<int, 1>());
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(O2_REG_HI));
+        // epilogue (both CTAs): TMEM lane quadrant warp % 4, 32 of the 128 columns
+        const int quad = warp & 3, cq = (warp - 4) >> 2;
+        const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(cq * O2_EC);
+        const uint32_t tf0 = mapa_u32(smem_u32(&tfree[0]), 0), tf1 = mapa_u32(smem_u32(&tfree[1]), 0);
+        int eb = 0;
+        bool ok = true;
+        for (int i = 0; i < ntl && ok; ++i) {
+            int64_t i0, j0;
+            o2_tile_coords<XD == 3>(pair + i * npairs, ntj, nti, i0, j0);
+            const int64_t row = i0 + 128 * (int)rank + quad * 32 + lane;
+            const int64_t c0 = j0 + cq * O2_EC;
+            const int nrem = row < m ? (int)min64(O2_EC, N - c0) : 0;  // this row's columns
+#pragma unroll 1
+            for (int j = 0; j < nrem; ++j)  // this tile's C_in entries into L2 while its MMAs run
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(Cin + row + (c0 + j) * ldi));
+            __syncwarp();
+            const int32_t ex = row < m ? Ex[row] : 0;
+            const int32_t eyl = c0 + lane < N ? Ey[c0 + lane] : 0;  // lane's column; read by shuffles
+            long long st[O2_EC];
+            auto half_ready = [&]() -> bool {
+                const bool w = mbar_wait(&accf[eb & 1], (uint32_t)((eb >> 1) & 1));
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (!w) *bad = 1;
+                return __all_sync(0xffffffffu, w && !*bad);
+            };
+            auto release = [&]() {
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster((eb & 1) ? tf1 : tf0);
+                ++eb;
+            };
+            uint32_t low[O2_EC / 4];  // bits 0-7 of four outputs each
+#pragma unroll
+            for (int c = 0; c < O2_EC; ++c) st[c] = 0;
+            // groups 2p and 2p + 1 of 8 columns
+            auto drain8 = [&](uint32_t tb, int h, auto use) {
+                uint32_t va[8], vb[8];
+                tmem_ld8_nowait(tb + 8 * h, va);
+                tmem_ld8_nowait(tb + O2_BN + 8 * h, vb);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    use(8 * h + j, (long long)__float2int_rn(__uint_as_float(va[j])) * 128 +
+                                       (long long)__float2int_rn(__uint_as_float(vb[j])));
+            };
+#pragma unroll 1
+            for (int p = 0; p < 3; ++p) {
+                if (!half_ready()) ok = false;
+                if (!ok) break;
+                const uint32_t tb = tq + (uint32_t)((eb & 1) * 2 * O2_BN);
+#pragma unroll
+                for (int h = 0; h < O2_EC / 8; ++h)
+                    drain8(tb, h, [&](int c, long long v) { st[c] = st[c] * 16384 + v; });
+                release();
+            }
+            if (!ok || !half_ready()) {
+                ok = false;
+                break;
+            }
+            {
+                // 2^14 x + v = 2^8 (2^6 x + floor(v / 2^8)) + the low 8 bits of v
+                const uint32_t tb = tq + (uint32_t)((eb & 1) * 2 * O2_BN);
+#pragma unroll
+                for (int h = 0; h < O2_EC / 8; ++h)
+                    drain8(tb, h, [&](int c, long long v) {
+                        st[c] = st[c] * 64 + (v >> 8);
+                        const uint32_t l8 = (uint32_t)v & 255u;
+                        low[c >> 2] = (c & 3) ? low[c >> 2] | (l8 << (8 * (c & 3))) : l8;
+                    });
+                // formed here and not where they are used (the compiler would keep
+                // the raw sums of all columns until then, twice the registers)
+#pragma unroll
+                for (int c = 0; c < O2_EC; ++c) asm volatile("" : "+l"(st[c]));
+#pragma unroll
+                for (int c = 0; c < O2_EC / 4; ++c) asm volatile("" : "+r"(low[c]));
+                release();
+            }
+            // 4 columns at a time, the next 4 entries of C_in loaded meanwhile
+            const double* ci = Cin + row + c0 * ldi;
+            double* co = Cout + row + c0 * ldo;
+            double cur[4], nxt[4];
+            auto load_c = [&](int g, double (&c)[4]) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    c[j] = 4 * g + j < nrem ? *ci : 0.0;
+                    ci += ldi;
+                }
+            };
+            load_c(0, cur);
+            // rolled, the sums moved down four registers an iteration: unrolled,
+            // the 16 warps run through more straight-line code than the
+            // instruction caches hold (47 against 24 thousand cycles a tile)
+#pragma unroll 1
+            for (int g = 0; g < O2_EC / 4; ++g) {
+                load_c(g + 1, nxt);  // (nrem <= 32: none past the last group)
+                double val[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int32_t ey = __shfl_sync(0xffffffffu, eyl, 4 * g + j);
+                    val[j] = o2_fixed_to_double(st[j], (low[0] >> (8 * j)) & 255u, ex + ey - 61);
+                    if (ex == OT_NONFINITE || ey == OT_NONFINITE) val[j] = __longlong_as_double(0x7ff8000000000000ll);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (4 * g + j < nrem) *co = cur[j] - val[j];
+                    co += ldo;
+                    cur[j] = nxt[j];
+                }
+#pragma unroll
+                for (int c = 0; c + 4 < O2_EC; ++c) st[c] = st[c + 4];
+#pragma unroll
+                for (int w = 0; w + 1 < O2_EC / 4; ++w) low[w] = low[w + 1];
+            }
+        }
+    }
+    if ((warp == 1 || warp == 2) && rank == 0) umma_commit_cg2_local_w(mdone, lane == 0 ? 1u : 0u);  // every MMA issued has completed
+    __syncthreads();
+    if (*bad) {
+        if (threadIdx.x == 0) {
+            set_info_once(err, -2);
+            if (rank == 0) {
+                // wait (bounded) for copies issued but never consumed, then the MMAs
+                for (int q = min(cnt[1], cnt[2]); q < cnt[0]; ++q) mbar_wait(&full[q & (O2_ST - 1)], (uint32_t)((q / O2_ST) & 1));
+                mbar_wait(mdone, 0);
+            }
+        }
+        __syncthreads();
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    cluster_sync_all();  // neither CTA leaves while the other reads its shared memory or signals its barriers
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tmem_dealloc2(tmem, 512);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Diagonal block: Ap[i, 0:nc] = src[i, 0:nc] R_jj^{-1} (R_jj upper, nc <= NB)
 // by substitution, one thread per row.  Each x_j is scaled by the reciprocal
 // of R[j, j] (one rounding more than a division).
@@ -803,6 +1186,20 @@ lsq_status ot_gauss_digits(uint64_t seed, int64_t s, int64_t j0, int64_t kc, int
     return LSQ_OK;
 }
 
+// Which form of the update: cycles of the busiest SM, from the rounds of
+// tiles each form needs and the cycles of a tile as measured, the larger of its
+// products (72 cycles per 16-wide K step of one digit pair for a 128 x 64 tile,
+// 87 for the 128 x 128 that a CTA of a pair does) and its epilogue (35 and 42
+// thousand).  The pairs win wherever their tiles fill the chip; few rows or
+// columns (N <= 64 above all) stay with the small tiles.
+static bool o2_faster(int ntiles, int ntiles2, int64_t K, int sms) {
+    if (sms < 2) return false;
+    const double steps = 36.0 * (double)ceil_div(K, 16);
+    const double c1 = (double)ceil_div(ntiles, sms) * std::max(72.0 * steps, 35000.0);
+    const double c2 = (double)ceil_div(ntiles2, sms / 2) * std::max(87.0 * steps, 42000.0);
+    return c2 < c1;
+}
+
 // C_out = C_in - X Y (M x N; X: M x K column-major, ld ldx; Y: entry (k, j)
 // at Y[k sk + j sj]) with FP64 accuracy on the tensor cores; K <= 512.
 // C_in may equal C_out (same ld).  xmode: 0 slice X here; 1 slice X with the
@@ -813,7 +1210,7 @@ lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t
                           int nbk, int x_digits) {
     if (M <= 0 || N <= 0 || K <= 0) return LSQ_OK;
     // exact group sums: at most 8 pairs of digits (|d_t d_u| <= 2^12) per
-    // group over K <= 512, or 3 pairs over K <= 1024 with three X digits
+    // group over K <= 512, or 3 pairs over K <= OT_KMAX3 with three X digits
     if (K > (x_digits == 3 ? OT_KMAX3 : OT_KMAX) || !ws || ws_bytes < ot_update_ws_bytes(M, N, K) ||
         (x_digits != 3 && x_digits != OT_DIG))
         return LSQ_ERR_ARG;
@@ -862,14 +1259,25 @@ lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t
     LSQ_LAUNCH_CHECK();
     CUtensorMap tx, ty;
     if (!ot_map(&tx, U.Zx, U.Kp, U.mp, OT_BM) || !ot_map(&ty, U.Zy, U.Kp, U.Np, OT_BN)) return LSQ_ERR_CUDA;
-    const size_t smem = ot_update_smem();
-    auto kern = x_digits == 3 ? k_ot_update<3> : k_ot_update<OT_DIG>;
-    LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int ntj = (int)(U.Np / OT_BN), ntiles = (int)(ntj * (U.mp / OT_BM));
-    const int grid = std::min(ntiles, device_sm_count());
     const int stage = x_digits == 3 ? ST_K_UPDATE3 : ST_K_UPDATE;
-    stage_mark(stage, true, st);
-    kern<<<grid, OT_THREADS, smem, st>>>(tx, ty, M, N, K, U.Ex, U.Ey, Cin, ldi, Cout, ldo, err, ntj, ntiles);
+    const int sms = device_sm_count();
+    const int ntj = (int)(U.Np / OT_BN), ntiles = (int)(ntj * (U.mp / OT_BM));
+    const int ntj2 = (int)ceil_div(U.Np, O2_BN), ntiles2 = (int)(ntj2 * ceil_div(U.mp, O2_BM));
+    if (o2_faster(ntiles, ntiles2, K, sms)) {
+        const size_t smem = 1024 + (size_t)O2_ST * O2_STAGE + 512;
+        auto kern = x_digits == 3 ? k_ot_update2<3> : k_ot_update2<OT_DIG>;
+        LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const int grid = 2 * std::min(ntiles2, sms / 2);
+        stage_mark(stage, true, st);
+        kern<<<grid, O2_THREADS, smem, st>>>(tx, ty, M, N, K, U.Ex, U.Ey, Cin, ldi, Cout, ldo, err, ntj2, ntiles2);
+    } else {
+        const size_t smem = ot_update_smem();
+        auto kern = x_digits == 3 ? k_ot_update<3> : k_ot_update<OT_DIG>;
+        LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const int grid = std::min(ntiles, sms);
+        stage_mark(stage, true, st);
+        kern<<<grid, OT_THREADS, smem, st>>>(tx, ty, M, N, K, U.Ex, U.Ey, Cin, ldi, Cout, ldo, err, ntj, ntiles);
+    }
     LSQ_LAUNCH_CHECK();
     // tensor-core work: the digit pairs actually issued
     const double pairs = x_digits == 3 ? 21.0 : 36.0;

@@ -129,3 +129,37 @@ def test_nonfinite_rows_propagate():
     ok = np.ones(400, bool)
     ok[[17, 200]] = False
     assert np.isfinite(Ap[ok]).all()
+
+
+@pytest.mark.parametrize("m,n", [(19457, 700), (40001, 333), (20000, 1029), (65536, 416)])
+def test_pair_tiles_give_the_small_tiles_bits(m, n):
+    """A row of A_p depends on that row alone, and both forms of the update sum
+    the same digit products exactly and round once: rows of a solve large
+    enough for the 256 x 128 tiles of CTA pairs are bit-identical to the same
+    rows solved among few (128 x 64 tiles).  First and last rows, tile edges
+    and a sample, rows and columns not multiples of the tiles."""
+    rng = np.random.default_rng(m + n)
+    A = rng.standard_normal((m, n)) * np.exp2(rng.uniform(-20, 20, m))[:, None]
+    R = np.triu(rng.standard_normal((n, n))) * 0.3
+    R[np.arange(n), np.arange(n)] = 1.0 + rng.random(n)
+    R *= np.exp2(rng.uniform(-4, 4, n))[None, :]
+    rows = np.unique(np.concatenate([np.arange(3), [127, 128, 255, 256, 257], rng.integers(0, m, 150),
+                                     np.arange(m - 130, m)]))
+    full, info = lsq.trsm_tc(dev_colmajor(np.asfortranarray(A)), dev_colmajor(R))
+    assert int(to_np(info)[0]) == 0
+    part, info = lsq.trsm_tc(dev_colmajor(np.asfortranarray(A[rows])), dev_colmajor(R))
+    assert int(to_np(info)[0]) == 0
+    np.testing.assert_array_equal(to_np(full)[rows], to_np(part))
+
+
+@pytest.mark.parametrize("m,n,s", [(6000, 1030, 4870), (3500, 1500, 3001), (5200, 2100, 5000)])
+def test_fp64_gaussian_sketch_pair_tiles_give_the_small_tiles_bits(m, n, s):
+    """The same for the three-digit products of an FP64 Gaussian sketch: a
+    column of A_s depends on that column of A alone."""
+    rng = np.random.default_rng(m + n + s)
+    A = rng.standard_normal((m, n)) * np.exp2(rng.uniform(-20, 20, n))[None, :]
+    opts = lsq.make_opts(kind=lsq.GAUSSIAN, s=s, seed=5, sketch_prec=lsq.FP64)
+    cols = np.unique(np.concatenate([[0, 1, 63, 64, 127, 128], rng.integers(0, n, 20), [n - 1]]))
+    full, _, _ = lsq.sketch(dev_colmajor(np.asfortranarray(A)), opts)
+    part, _, _ = lsq.sketch(dev_colmajor(np.asfortranarray(A[:, cols])), opts)
+    np.testing.assert_array_equal(to_np(full)[:, cols], to_np(part))
