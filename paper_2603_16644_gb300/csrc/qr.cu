@@ -210,6 +210,50 @@ __device__ __forceinline__ T tree_sum(const T* x, int stride) {
     return v[0];
 }
 
+// FP64 reciprocal square root and reciprocal for the Householder scalars: an
+// FP32 estimate (about 23 bits; operands and estimates moved between FP64 and
+// FP32 on the bit patterns, the exponent split off so that any normal FP64
+// operand works) refined in FP64, by one third-order step (sqrt) and by two
+// Newton steps (reciprocal).  A few units in the last place, 4 to 5 dependent
+// FP64 operations each, where the library's correctly rounded sqrt and division
+// cost ~650 cycles apiece on this GPU and formed a chain of four per column.
+// Subnormal, infinite and NaN operands take the library functions.
+__device__ __forceinline__ bool qr_normal(double d) {
+    const int e = (int)(((unsigned long long)__double_as_longlong(d) >> 52) & 0x7ff);
+    return e != 0 && e != 0x7ff;
+}
+
+// 1 / sqrt(d), d > 0
+__device__ __forceinline__ double qr_rsqrt(double d) {
+    if (!qr_normal(d)) return 1.0 / sqrt(d);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    const int e2 = ((int)(b >> 52) - 1023) & ~1;                           // d = m 2^e2, m in [1, 4)
+    const unsigned long long mb = b - ((unsigned long long)(long long)e2 << 52);
+    const double m = __longlong_as_double((long long)mb);
+    const uint32_t fb = (uint32_t)((((mb >> 52) & 0x7ff) - 1023 + 127) << 23) | (uint32_t)((mb >> 29) & 0x7fffff);
+    const uint32_t yb = __float_as_uint(rsqrtf(__uint_as_float(fb)));
+    double y = __longlong_as_double((long long)(((unsigned long long)((yb >> 23) - 127 + 1023) << 52) |
+                                                ((unsigned long long)(yb & 0x7fffff) << 29)));
+    const double e = fma(-(m * y), y, 1.0);
+    y = fma(y * e, fma(0.375, e, 0.5), y);
+    return __longlong_as_double(__double_as_longlong(y) - ((long long)(e2 / 2) << 52));
+}
+
+// 1 / d, d > 0 and 1 / d normal
+__device__ __forceinline__ double qr_rcp(double d) {
+    if (!qr_normal(d)) return 1.0 / d;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    const int ed = (int)(b >> 52) - 1023;
+    const double m = __longlong_as_double((long long)((b & 0x000fffffffffffffull) | (1023ull << 52)));  // [1, 2)
+    const uint32_t fb = (127u << 23) | (uint32_t)((b >> 29) & 0x7fffff);
+    const uint32_t yb = __float_as_uint(__frcp_rn(__uint_as_float(fb)));
+    double y = __longlong_as_double((long long)(((unsigned long long)((yb >> 23) - 127 + 1023) << 52) |
+                                                ((unsigned long long)(yb & 0x7fffff) << 29)));
+    y = fma(fma(-m, y, 1.0), y, y);
+    y = fma(fma(-m, y, 1.0), y, y);
+    return ed < 1021 ? __longlong_as_double(__double_as_longlong(y) - ((long long)ed << 52)) : 1.0 / d;
+}
+
 // QCL: CTAs per cluster (16, non-portable, where the device allows it; else
 // 8).  Dynamic shared memory: the local panel (Rp x QNB) and, in the fused
 // form, the previous panel's reflector rows and the partial products behind it.
@@ -233,7 +277,7 @@ __global__ void __launch_bounds__(QCT)
     __shared__ __align__(16) T bcx[QCT / 32][QRC];  // per warp: x_{jj+1} below its diagonal
     __shared__ T rowbuf[QNB];                      // row jj of the panel (owning CTA)
     __shared__ T scal_sh[4];                       // FP64: mu, b, v1, 1 / v1 of the column (warp 0)
-    __shared__ T wc_sh[QNB];                       // FP64: w_c of the column (warp 0)
+    __shared__ T wc_sh[QNB], f_sh[QNB];            // FP64: w_c and w_c / v1 of the column (warp 0)
     __shared__ int scale_sh;
     const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -438,8 +482,55 @@ __global__ void __launch_bounds__(QCT)
     // CTA; after the cluster barrier every CTA forms the same Householder
     // scalars, w_c for each column and (rank 0) column jj - 1 of Y.
     struct Scal {
-        T mu, b, v1, rv1, wc;
+        T mu, b, v1, rv1, wc;  // R's diagonal entry, beta, v's leading entry before scaling, its reciprocal, w_c
+        T f;                   // FP64: w_c / v1
         bool scale;
+    };
+    // FP64: the sign of v1 is that of x1 (no cancellation, no case distinction;
+    // R's diagonal entry is then -sign(x1) mu, and k_qr_extract makes the
+    // diagonal positive by the signs of R's rows), and with mu = sqrt(x1^2 +
+    // sigma), |v1| = |x1| + mu:  sigma + v1^2 = 2 mu |v1|, so that beta =
+    // 2 v1^2 / (sigma + v1^2) = |v1| / mu needs 1/mu and 1/|v1| only.
+    auto scalars64 = [&](int jj, int buf, int owner) -> Scal {
+        Scal sc;
+        // lane > jj: d_c of this column; lane jj: sigma; lane < jj - 1: u_i^T u_{jj-1}
+        const T dsum = tree_sum<T, QCL>(&all_part[buf][0][lane], QNB);
+        const T sigma = __shfl_sync(0xffffffffu, dsum, jj);
+        const T x1 = all_row[buf][jj];
+        const T s2 = fma(x1, x1, sigma);
+        sc.scale = sigma != (T)0;
+        sc.mu = x1;
+        sc.b = (T)0;
+        sc.v1 = (T)1;
+        sc.rv1 = (T)1;
+        sc.wc = sc.f = (T)0;
+        if (sc.scale) {
+            const T y = (T)qr_rsqrt((double)s2);
+            T mu = s2 * y;
+            mu = fma((T)0.5 * y, fma(-mu, mu, s2), mu);  // to the last bit
+            const T av = fabs(x1) + mu;
+            const T r = (T)qr_rcp((double)av);
+            sc.v1 = x1 < (T)0 ? -av : av;
+            sc.rv1 = x1 < (T)0 ? -r : r;
+            sc.mu = x1 < (T)0 ? mu : -mu;
+            // tau = 2 / u^T u = 1 / (mu |v1|) and beta = |v1| / mu, each corrected
+            // once: their errors are common to all rows, so that they would
+            // show in R's where those of single entries average out
+            T tau = y * r;
+            tau = fma(fma(-(tau * mu), av, (T)1), tau, tau);
+            T bt = av * y;
+            bt = fma(fma(-bt, mu, av), y, bt);
+            sc.b = bt;
+            if (lane > jj && lane < nb) {
+                const T ac = all_row[buf][lane];
+                sc.f = tau * fma(sc.v1, ac, dsum);
+                sc.wc = bt * fma(dsum, sc.rv1, ac);
+            }
+        }
+        if (rank == 0 && warp == 0 && lane + 1 < jj) Ysm[lane][jj - 1] = dsum;
+        if (tid == 0) bsh[jj] = sc.b;  // identical in every CTA of the cluster
+        if (rank == owner && tid == 0) beta_out[k0 + jj] = sc.b;
+        return sc;
     };
     // The Householder scalars of column jj from the exchanged partials (the
     // same in every CTA) and, per lane c > jj, w_c.
@@ -492,7 +583,7 @@ __global__ void __launch_bounds__(QCT)
             // (every warp forming them kept the FP64 pipe 73 % busy on a panel
             // of few rows), and read by the other warps from shared memory.
             if (warp == 0) {
-                sc = scalars(jj, buf, owner);
+                sc = scalars64(jj, buf, owner);
                 if (lane == 0) {
                     scal_sh[0] = sc.mu;
                     scal_sh[1] = sc.b;
@@ -501,6 +592,7 @@ __global__ void __launch_bounds__(QCT)
                     scale_sh = sc.scale ? 1 : 0;
                 }
                 wc_sh[lane] = sc.wc;
+                f_sh[lane] = sc.f;
             }
             __syncthreads();
             sc.mu = scal_sh[0];
@@ -509,11 +601,13 @@ __global__ void __launch_bounds__(QCT)
             sc.rv1 = scal_sh[3];
             sc.scale = scale_sh != 0;
             sc.wc = wc_sh[lane];
+            sc.f = f_sh[lane];
             return sc;
         }
         return scalars(jj, buf, owner);
     };
     T acc;
+    T yscale = (T)1;  // scale of lane i's entry of Y's last column
     if (std::is_same<T, double>::value && chunk <= QRC) {
         // FP64: each thread keeps its column's QRC rows of this warp in
         // registers; per column every lane of a warp takes the raw column jj
@@ -522,10 +616,10 @@ __global__ void __launch_bounds__(QCT)
         // divergent single-lane phases, no shared-memory round trips).
         // Measured: the FP64 path 6.2 -> 23.5 solves/s; for FP32 the
         // shared-memory form below is faster (3.07 against 4.55 ms per solve).
-        // The loops run over QR = 8, 16 or 32 rows per lane, the fewest that
-        // hold the warp's rows: FP64 instructions issue at a small fraction of
-        // the FP32 rate on this GPU, so masked rows are not free (a 32-column
-        // panel of ~1000 rows took 0.53 ms with 32 rows per lane).
+        // The loops run over QR = 4, 8, ... 32 rows per lane, the fewest that hold
+        // the warp's rows: the FP64 pipe takes 16 cycles an instruction and SM, so
+        // masked rows are not free (a panel's column costs ~11 thousand cycles
+        // with 32 rows per lane, in update and dots alone).
         auto f64_cols = [&](auto qr_tag) {
             constexpr int QR = decltype(qr_tag)::value;
             T a[QR];
@@ -541,13 +635,24 @@ __global__ void __launch_bounds__(QCT)
                 return v;
             };
             // column c below row `row` on this warp's rows, from lane c
+            // The columns stay as they are in registers: with u = [v1; x] (not
+            // scaled to a unit leading entry) the update is a_c -= (w_c / v1) u and
+            // u_i^T u_j gives Y up to the scales 1 / v1, so that a column costs two
+            // FP64 operations per row and lane (three with v formed by every
+            // lane); lane c keeps its own 1 / v1 and R_cc and applies them at the
+            // end.
             T xn[QR];
+            T myscale = (T)1, myR = (T)0, rprev = (T)1;
             auto column_below = [&](int c, int row) {
 #pragma unroll
                 for (int q = 0; q < QR; ++q) {
                     const T x = __shfl_sync(0xffffffffu, a[q], c);
                     xn[q] = (q < nv && gr0 + q > row) ? x : (T)0;
                 }
+            };
+            // Y[i][j] = v_i^T v_j from u_i^T u_j (lane i; rank 0, warp 0)
+            auto scale_y = [&](int j) {
+                if (rank == 0 && warp == 0 && lane < j) Ysm[lane][j] *= myscale * rprev;
             };
             column_below(0, 0);
             if (0 >= gr0 && 0 < gr0 + nv) rowbuf[lane] = row_of(0);
@@ -559,41 +664,59 @@ __global__ void __launch_bounds__(QCT)
             }
             for (int jj = 0; jj < nb; ++jj) {
                 const Scal sc = exchange(jj, acc, rowbuf, 1);
-                // v_jj on this warp's rows: 0 above row jj, 1 on it, x / v1 below
-                T v[QR];
+                if (jj > 0) scale_y(jj - 1);
+                // u_jj on this warp's rows: 0 above row jj, v1 on it, x below
+                T u[QR];
 #pragma unroll
                 for (int q = 0; q < QR; ++q) {
                     const T x = __shfl_sync(0xffffffffu, a[q], jj);
                     const int gr = gr0 + q;
-                    v[q] = (gr < jj || q >= nv) ? (T)0 : (gr == jj ? (T)1 : (sc.scale ? x * sc.rv1 : x));
+                    u[q] = (gr < jj || q >= nv) ? (T)0 : (gr == jj ? sc.v1 : x);
                 }
-                // lane jj: its column becomes v (R diagonal mu on row jj); later
-                // columns: a_c -= w_c v
-                const bool own = lane == jj, upd = lane > jj && lane < nb && sc.b != (T)0;
+                if (lane == jj) {
+                    myscale = sc.rv1;
+                    myR = sc.mu;
+                }
+                rprev = sc.rv1;
+                // later columns: a_c -= w_c v = (w_c / v1) u
+                const bool upd = lane > jj && lane < nb && sc.b != (T)0;
+                const T f = sc.f;
+                if (upd) {
 #pragma unroll
-                for (int q = 0; q < QR; ++q) {
-                    const int gr = gr0 + q;
-                    const T ownv = (q < nv && gr > jj) ? v[q] : ((q < nv && gr == jj) ? sc.mu : a[q]);
-                    a[q] = own ? ownv : (upd ? fma(-sc.wc, v[q], a[q]) : a[q]);
+                    for (int q = 0; q < QR; ++q) a[q] = fma(-f, u[q], a[q]);
                 }
                 const int jn = jj + 1;
                 if (jn < nb) {
                     column_below(jn, jn);
                     if (jn >= gr0 && jn < gr0 + nv) rowbuf[lane] = row_of(jn);
                 }
-                // lanes c > jj: dots of column jj + 1; lanes i < jj: Y[i][jj]
+                // lanes c > jj: dots of column jj + 1; lanes i < jj: u_i^T u_jj
                 const bool ylane = lane < jj, dlane = lane >= jn && lane < nb && jn < nb;
                 T s4[4] = {(T)0, (T)0, (T)0, (T)0};
 #pragma unroll
-                for (int q = 0; q < QR; ++q) s4[q & 3] = fma(ylane ? v[q] : xn[q], a[q], s4[q & 3]);
+                for (int q = 0; q < QR; ++q) s4[q & 3] = fma(ylane ? u[q] : xn[q], a[q], s4[q & 3]);
                 acc = (ylane || dlane) ? (s4[0] + s4[1]) + (s4[2] + s4[3]) : (T)0;
+            }
+            yscale = myscale * rprev;  // of Y's last column, formed below
+            // R on and above the diagonal, v below it
+            if (lane < nb) {
+#pragma unroll
+                for (int q = 0; q < QR; ++q) {
+                    const int gr = gr0 + q;
+                    a[q] = gr > lane ? a[q] * myscale : (gr == lane ? myR : a[q]);
+                }
             }
 #pragma unroll
             for (int q = 0; q < QR; ++q)
                 if (q < nv) P[lane * Rp + g0 + q] = a[q];
         };
-        if (chunk <= 8) f64_cols(std::integral_constant<int, 8>{});
+        if (chunk <= 4) f64_cols(std::integral_constant<int, 4>{});
+        else if (chunk <= 8) f64_cols(std::integral_constant<int, 8>{});
+        else if (chunk <= 12) f64_cols(std::integral_constant<int, 12>{});
         else if (chunk <= 16) f64_cols(std::integral_constant<int, 16>{});
+        else if (chunk <= 20) f64_cols(std::integral_constant<int, 20>{});
+        else if (chunk <= 24) f64_cols(std::integral_constant<int, 24>{});
+        else if (chunk <= 28) f64_cols(std::integral_constant<int, 28>{});
         else f64_cols(std::integral_constant<int, QRC>{});
     } else if (chunk <= QRC) {
         // Each thread keeps its column's QRC rows of this warp in registers
@@ -756,7 +879,8 @@ __global__ void __launch_bounds__(QCT)
         *cluster.map_shared_rank(&all_part[nb & 1][rank][lane], 0) = t;
     }
     cluster.sync();
-    if (rank == 0 && warp == 0 && lane + 1 < nb) Ysm[lane][nb - 1] = tree_sum<T, QCL>(&all_part[nb & 1][0][lane], QNB);
+    if (rank == 0 && warp == 0 && lane + 1 < nb)
+        Ysm[lane][nb - 1] = tree_sum<T, QCL>(&all_part[nb & 1][0][lane], QNB) * yscale;
     // write R / v back to W and the explicit V (0 above, 1 on the diagonal)
     for (int c = 0; c < QNB; ++c)
         for (int i = tid; i < nloc; i += QCT) {
@@ -777,10 +901,11 @@ __global__ void __launch_bounds__(QCT)
             T trow[QNB];
 #pragma unroll
             for (int jj = 0; jj < QNB; ++jj) {
-                T t = (T)0;
+                T t4[4] = {(T)0, (T)0, (T)0, (T)0};  // 4 chains: the latency of 496 dependent FMAs is long in FP64
                 if (jj < nb)
 #pragma unroll
-                    for (int qq = 0; qq < jj; ++qq) t = fma(trow[qq], Ysm[qq][jj], t);
+                    for (int qq = 0; qq < jj; ++qq) t4[qq & 3] = fma(trow[qq], Ysm[qq][jj], t4[qq & 3]);
+                const T t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
                 const T bj = jj < nb ? bsh[jj] : (T)0;
                 trow[jj] = lane < jj ? -bj * t : (lane == jj ? bj : (T)0);
             }
@@ -989,7 +1114,9 @@ __global__ void k_qr_extract(const T* __restrict__ W, int64_t ld, int64_t n, con
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
         int64_t i = q % n, j = q / n;
         if (i <= j) {
+            // row i times the sign of its diagonal entry (FP64 panels leave either)
             double v = (double)W[i + j * ld];
+            if (W[i + i * ld] < (T)0) v = -v;
             Rs[i + j * ldr] = colexp ? ldexp(v, -colexp[j]) : v;
         }
     }

@@ -150,6 +150,44 @@ def test_precond_qr(qr_prec, s, n):
     assert np.linalg.norm(Ru.T @ Ru - As.T @ As) / np.linalg.norm(As) ** 2 <= 20 * s * u
 
 
+@pytest.mark.parametrize("s,n", [(40, 33), (400, 64), (700, 40), (1900, 40), (2500, 40), (3500, 70), (5000, 70),
+                                 (2100, 300)])
+def test_precond_qr_fp64_rows_per_lane(s, n):
+    """FP64 panels over every row count per lane (and more rows than the
+    registers hold), columns graded over 2^+-60 and of either sign, against
+    the oracle's R; both are columnwise backward stable, so every column of R
+    is within a modest multiple of n u kappa of the other's, relative to the
+    column (kappa of the matrix with its grading taken out)."""
+    rng = np.random.default_rng(7 * s + n)
+    B = rng.standard_normal((s, n))
+    B[0] += 3.0 * np.where(np.arange(n) % 2, 1.0, -1.0)
+    g = np.exp2(rng.integers(-60, 61, n))
+    As = np.asfortranarray(B * g[None, :])
+    R, info = lsq.precond_qr(dev_colmajor(As), None, O.FP64)
+    R = to_np(R)
+    assert int(to_np(info)[0]) == 0 and np.all(np.diag(R) > 0)
+    Ro = O.qr_r(As, O.FP64)
+    err = np.linalg.norm(R - Ro, axis=0) / np.linalg.norm(Ro, axis=0)
+    assert err.max() <= 20 * n * U64 * O.kappa(B), err.max()
+
+
+def test_precond_qr_fp64_triangular_input():
+    """Columns that are zero below the diagonal already (sigma = 0) with
+    diagonal entries of either sign: R is the input with its rows' signs
+    made positive, exactly, and a zero diagonal entry is a breakdown."""
+    n = 45
+    rng = np.random.default_rng(3)
+    A = np.zeros((200, n))
+    A[:n] = np.triu(rng.standard_normal((n, n)))
+    R, info = lsq.precond_qr(dev_colmajor(A), None, O.FP64)
+    assert int(to_np(info)[0]) == 0
+    sg = np.sign(np.diag(A[:n]))
+    np.testing.assert_array_equal(to_np(R), A[:n] * sg[:, None])
+    A[20, 20] = 0.0
+    _, info = lsq.precond_qr(dev_colmajor(A), None, O.FP64)
+    assert int(to_np(info)[0]) == 21
+
+
 def test_precond_qr_zero_column_reports_breakdown():
     s, n = 100, 10
     rng = np.random.default_rng(1)
