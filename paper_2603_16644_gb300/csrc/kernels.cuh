@@ -153,6 +153,13 @@ lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t
                           int64_t ldi, double* Cout, int64_t ldo, int64_t M, int64_t N, int64_t K, void* ws,
                           size_t ws_bytes, int32_t* err, cudaStream_t st, int xmode = 0,
                           const int32_t* Eblk = nullptr, int64_t b0 = 0, int nbk = 0, int x_digits = 8);
+// out (M x (N0 + N1), ld M) = -X [Y0 Y1], K of any length, M small (see
+// oz_trsm.cu); part and ws: the bytes of the two functions with N = N0 + N1.
+size_t ot_gemm_long_ws_bytes(int64_t M, int64_t N, int64_t K);
+size_t ot_gemm_long_part_bytes(int64_t M, int64_t N, int64_t K);
+lsq_status ot_gemm_long(const double* X, int64_t ldx, const double* Y0, int64_t ld0, int64_t N0, const double* Y1,
+                        int64_t ld1, int64_t N1, double* out, int64_t M, int64_t K, double* part, void* ws,
+                        size_t ws_bytes, int32_t* err, cudaStream_t st);
 // The negated Gaussian operator's columns j0 .. j0 + kc - 1 (rows 0 .. s - 1,
 // kc <= 960) written as the X digit planes of an update's scratch ws (the
 // scratch of ot_gemm_update with M = s, N, K = kc), for ot_gemm_update with

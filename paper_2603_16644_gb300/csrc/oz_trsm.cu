@@ -107,19 +107,21 @@ __device__ __forceinline__ uint32_t ot_digit_pair(unsigned long long W0, unsigne
 // TMA box lies inside the planes), with the row exponents from per-block
 // exponents (Eblk[b m + i] for blocks b0 .. b0+nbk-1, INT32_MIN for an
 // all-zero block): a 2-D grid, one thread per row and 64-wide range of K
-// (blockIdx.y), so that many loads are in flight.
+// (blockIdx.y), so that many loads are in flight.  zdiv ranges form a K chunk
+// with exponents of its own (Eblk + z m, Ex + z mp).
 __global__ void __launch_bounds__(128) k_ot_rowslice_e(const double* __restrict__ X, int64_t m, int64_t mp,
                                                        int64_t K, int64_t ld, int64_t Kp, int32_t* __restrict__ Ex,
                                                        uint16_t* __restrict__ Z, const int32_t* __restrict__ Eblk,
-                                                       int64_t b0, int nbk) {
+                                                       int64_t b0, int nbk, unsigned zdiv) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= mp) return;
+    const int64_t z = blockIdx.y / zdiv;
     int32_t eb = INT32_MIN;
     if (i < m)
-        for (int b = 0; b < nbk; ++b) eb = max(eb, Eblk[(b0 + b) * m + i]);
+        for (int b = 0; b < nbk; ++b) eb = max(eb, Eblk[(z + b0 + b) * m + i]);
     const int32_t E = eb == INT32_MIN ? 0 : eb;
     const int64_t kb = (int64_t)blockIdx.y * 64;
-    if (blockIdx.y == 0) Ex[i] = E;
+    if (blockIdx.y % zdiv == 0) Ex[z * mp + i] = E;
     const double* row = X + i;
     const int64_t Kr = i < m ? K : 0;
 #pragma unroll 1
@@ -145,9 +147,10 @@ __global__ void __launch_bounds__(128) k_ot_rowslice_e(const double* __restrict_
 }
 
 // Row maxima of |X| (bit patterns, the sign cleared; atomicMax orders them
-// like the values) over 64-wide K ranges, one thread per row; Mx zeroed.
+// like the values) over 64-wide K ranges, one thread per row; Mx zeroed.  zdiv
+// ranges form a K chunk with maxima of its own (Mx + z m).
 __global__ void __launch_bounds__(128) k_ot_rowmax2d(const double* __restrict__ X, int64_t m, int64_t K, int64_t ld,
-                                                     unsigned long long* __restrict__ Mx) {
+                                                     unsigned long long* __restrict__ Mx, unsigned zdiv) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     const int64_t k0 = (int64_t)blockIdx.y * 64, k1 = min64(K, k0 + 64);
@@ -156,7 +159,7 @@ __global__ void __launch_bounds__(128) k_ot_rowmax2d(const double* __restrict__ 
         const unsigned long long a = (unsigned long long)__double_as_longlong(X[i + k * ld]) & 0x7fffffffffffffffull;
         mx = a > mx ? a : mx;
     }
-    if (mx) atomicMax(&Mx[i], mx);
+    if (mx) atomicMax(&Mx[blockIdx.y / zdiv * m + i], mx);
 }
 
 // The rows' exponents in the per-block convention (INT32_MIN for a zero row).
@@ -281,15 +284,18 @@ __global__ void __launch_bounds__(128) k_ot_rowslice_s(const __grid_constant__ C
 
 // Columns of Y (K x N, entry (k, j) at Y[k sk + j sj]): Ey[j] and digit
 // planes Z[(u Np + j) Kp + k] (zero for columns N <= j < Np and for
-// K <= k < Kp).  One CTA per column.
+// K <= k < Kp).  One CTA per column and K chunk of kc (blockIdx.y), which has
+// an exponent of its own (Ey + z Np); the columns go to places j0 + j.
 __global__ void __launch_bounds__(128) k_ot_colslice(const double* __restrict__ Y, int64_t K, int64_t N, int64_t Np,
                                                      int64_t sk, int64_t sj, int64_t Kp, int32_t* __restrict__ Ey,
-                                                     uint16_t* __restrict__ Z) {
-    const int64_t j = blockIdx.x;
-    const double* col = Y + j * sj;
-    const int64_t Kr = j < N ? K : 0;
+                                                     uint16_t* __restrict__ Z, int64_t j0, int64_t kc) {
+    const int64_t j = j0 + blockIdx.x;
+    const double* col = Y + (int64_t)blockIdx.x * sj;
+    const int64_t k0 = (int64_t)blockIdx.y * kc;
+    const int64_t k1 = blockIdx.y + 1 == gridDim.y ? Kp : k0 + kc;
+    const int64_t Kr = blockIdx.x < N ? min64(K, k1) : 0;
     unsigned long long mx = 0;
-    for (int64_t k = threadIdx.x; k < Kr; k += blockDim.x) {
+    for (int64_t k = k0 + threadIdx.x; k < Kr; k += blockDim.x) {
         unsigned long long v = (unsigned long long)__double_as_longlong(col[k * sk]) & 0x7fffffffffffffffull;
         mx = v > mx ? v : mx;
     }
@@ -305,11 +311,11 @@ __global__ void __launch_bounds__(128) k_ot_colslice(const double* __restrict__ 
         unsigned long long t = 0;
         for (int q = 0; q < 4; ++q) t = w[q] > t ? w[q] : t;
         Es = ot_exp_of_max(t);
-        Ey[j] = Es;
+        Ey[blockIdx.y * Np + j] = Es;
     }
     __syncthreads();
     const int32_t E = Es;
-    for (int64_t k = threadIdx.x; k < Kp; k += blockDim.x) {
+    for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
         const unsigned long long W = ot_fields(k < Kr ? col[k * sk] : 0.0, E);
 #pragma unroll
         for (int u = 0; u < OT_DIG; ++u) Z[((int64_t)u * Np + j) * Kp + k] = (uint16_t)(ot_digit_f32(W, u) >> 16);
@@ -400,12 +406,16 @@ __device__ __forceinline__ void ot_tile_coords(int t, int ntj, int nti, int64_t&
 
 // XD: digits of X taken (8, or 3 when X's lower digits are known to vanish);
 // pairs (t, u) with t < XD and t + u <= 7.
+// kc < K (a multiple of OT_BK): K is taken in chunks of kc, each a set of tiles
+// of its own (tiles of chunk z after those of chunk z - 1) whose result -X Y
+// over the chunk goes to Cout + z zs (Cin NULL), with the exponents Ex + z zx
+// and Ey + z zy; K past the operands reads as zeros.
 template <int XD>
 __global__ void __launch_bounds__(OT_THREADS, 1)
     k_ot_update(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, int64_t m,
                 int64_t N, int64_t K, const int32_t* __restrict__ Ex, const int32_t* __restrict__ Ey,
                 const double* Cin, int64_t ldi, double* Cout, int64_t ldo, int32_t* __restrict__ err, int ntj,
-                int ntiles) {
+                int ntiles, int64_t kc, int64_t zs, int zt, int64_t zx, int64_t zy) {
     extern __shared__ unsigned char ot_raw[];
     uint8_t* base = (uint8_t*)(((uintptr_t)ot_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* sY = base;                                // 2 stages x 8 digit tiles
@@ -422,7 +432,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
     int* cnt = (int*)(tslot + 2);  // x issued, x consumed (issuer 0), y issued, y consumed (0), x / y consumed (1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nslab = (int)((K + OT_BK - 1) / OT_BK);
+    const int nslab = (int)((kc + OT_BK - 1) / OT_BK);
     const int ntl = ntiles > (int)blockIdx.x ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
 
     if (threadIdx.x == 0) {
@@ -452,10 +462,10 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
         // X tile 3 of the current one, or after its last), then the XD X digit
         // tiles
         const int total = ntl * nslab;  // slabs over all tiles of this CTA
-        auto slab_tile = [&](int g, int64_t& i0, int64_t& j0, int& s) {
+        auto slab_tile = [&](int g, int64_t& i0, int64_t& j0, int& kx) {
             const int tl = (int)blockIdx.x + (g / nslab) * (int)gridDim.x;
-            s = g % nslab;
-            ot_tile_coords<XD == 3>(tl, ntj, ntiles / ntj, i0, j0);
+            kx = (int)(tl / zt * kc) + g % nslab * OT_BK;  // zt: tiles of a chunk
+            ot_tile_coords<XD == 3>(tl % zt, ntj, zt / ntj, i0, j0);
         };
         auto load_y = [&](int g) -> bool {
             int64_t i0, j0;
@@ -465,7 +475,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
             if (g >= 2 && !mbar_wait(&yempty[ys], (uint32_t)(((g >> 1) - 1) & 1))) return false;
             mbar_expect_tx(&yfull[ys], OT_DIG * OT_YTILE);
             for (int u = 0; u < OT_DIG; ++u)
-                tma_load_3d(sY + (ys * OT_DIG + u) * OT_YTILE, &tmY, &yfull[ys], s * OT_BK, (int)j0, u);
+                tma_load_3d(sY + (ys * OT_DIG + u) * OT_YTILE, &tmY, &yfull[ys], s, (int)j0, u);
             cnt[2] = g + 1;
             return true;
         };
@@ -487,7 +497,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
                     break;
                 }
                 mbar_expect_tx(&xfull[xs], OT_XTILE);
-                tma_load_3d(sX + xs * OT_XTILE, &tmX, &xfull[xs], s * OT_BK, (int)i0, t);
+                tma_load_3d(sX + xs * OT_XTILE, &tmX, &xfull[xs], s, (int)i0, t);
                 cnt[0] = xq + 1;
             }
         }
@@ -528,7 +538,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
                     const uint64_t dy = dy0 + (uint64_t)(ys * (OT_DIG * OT_YTILE >> 4));
                     // 16-wide K steps past K (zero digits) are not issued: lane
                     // 0's issue predicate per step, set once per slab
-                    const int64_t krem = K - (int64_t)s * OT_BK;
+                    const int64_t krem = K - ((int)blockIdx.x + i * (int)gridDim.x) / zt * kc - (int64_t)s * OT_BK;
                     const uint32_t lk[4] = {lead, krem > 16 ? lead : 0u, krem > 32 ? lead : 0u, krem > 48 ? lead : 0u};
 #pragma unroll
                     for (int t = 0; t < XD; ++t) {
@@ -566,7 +576,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
         const int quad = warp & 3, cq = (warp - 3) >> 2;
         const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16);
         // drain W columns of the 8 group sums, release the TMEM, convert and store
-        auto epi = [&](auto Wc, int64_t row, int64_t c0) {
+        auto epi = [&](auto Wc, int64_t row, int64_t c0, int64_t z) {
             constexpr int W = decltype(Wc)::value;
             const uint32_t tl = tq + (uint32_t)(cq * W);
             long long hi[W], lo[W];
@@ -596,7 +606,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(tfree);
             if (row < m) {
-                const int32_t ex = Ex[row];
+                const int32_t ex = Ex[z * zx + row];
 #pragma unroll
                 for (int h = 0; h < W / 8; ++h) {
                     double cin[8];
@@ -604,8 +614,8 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const int64_t col = c0 + 8 * h + j;
-                        cin[j] = col < N ? Cin[row + col * ldi] : 0.0;
-                        ey[j] = col < N ? Ey[col] : 0;
+                        cin[j] = col < N && Cin ? Cin[row + col * ldi] : 0.0;
+                        ey[j] = col < N ? Ey[z * zy + col] : 0;
                     }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
@@ -616,7 +626,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
                                 val = __longlong_as_double(0x7ff8000000000000ll);
                             else
                                 val = ot_fixed_to_double(hi[8 * h + j], lo[8 * h + j], ex + ey[j] - 61);
-                            Cout[row + col * ldo] = cin[j] - val;
+                            Cout[z * zs + row + col * ldo] = cin[j] - val;
                         }
                     }
                 }
@@ -625,11 +635,11 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
         for (int i = 0; i < ntl; ++i) {
             const int tile = (int)blockIdx.x + i * (int)gridDim.x;
             int64_t i0, j0;
-            ot_tile_coords<XD == 3>(tile, ntj, ntiles / ntj, i0, j0);
+            ot_tile_coords<XD == 3>(tile % zt, ntj, zt / ntj, i0, j0);
             const int64_t row = i0 + quad * 32 + lane;
             const bool narrow = N - j0 <= 32;
             const int64_t c0 = j0 + cq * (narrow ? 8 : 16);
-            if (row < m) {  // this tile's C_in entries into L2 while its MMAs run
+            if (Cin && row < m) {  // this tile's C_in entries into L2 while its MMAs run
                 for (int j = 0; j < (narrow ? 8 : 16); ++j)
                     if (c0 + j < N) asm volatile("prefetch.global.L2 [%0];" ::"l"(Cin + row + (c0 + j) * ldi));
             }
@@ -637,8 +647,8 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (!ok) *bad = 1;
             if (!__all_sync(0xffffffffu, ok && !*bad)) break;
-            if (narrow) epi(std::integral_constant<int, 8>(), row, c0);
-            else epi(std::integral_constant<int, 16>(), row, c0);
+            if (narrow) epi(std::integral_constant<int, 8>(), row, c0, tile / zt);
+            else epi(std::integral_constant<int, 16>(), row, c0, tile / zt);
         }
     }
     if ((warp == 1 || warp == 2) && lane == 0) umma_commit(mdone);  // fires when every MMA issued has completed
@@ -1242,20 +1252,20 @@ lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t
             tzs, txs, X, M, U.mp, K, ldx, U.Ex, nullptr, 0, 0, err);
     } else if (xmode == 1) {
         k_ot_rowslice_e<<<dim3((unsigned)(U.mp / 128), (unsigned)(U.Kp / 64)), 128, 0, st>>>(
-            X, M, U.mp, K, ldx, U.Kp, U.Ex, U.Zx, Eblk, b0, nbk);
+            X, M, U.mp, K, ldx, U.Kp, U.Ex, U.Zx, Eblk, b0, nbk, 1u << 30);
     } else {
         // row maxima over a 2-D grid (rows x 64-wide K ranges), then the
         // slicing on the same grid: every SM has work even when M is small
         LSQ_CUDA_TRY(cudaMemsetAsync(U.Mx, 0, sizeof(unsigned long long) * (size_t)U.mp, st));
         const dim3 g2((unsigned)(U.mp / 128), (unsigned)(U.Kp / 64));
-        k_ot_rowmax2d<<<g2, 128, 0, st>>>(X, M, K, ldx, U.Mx);
+        k_ot_rowmax2d<<<g2, 128, 0, st>>>(X, M, K, ldx, U.Mx, 1u << 30);
         LSQ_LAUNCH_CHECK();
         k_ot_rowexp<<<(unsigned)ceil_div(M, 256), 256, 0, st>>>(U.Mx, M, U.Eb);
         LSQ_LAUNCH_CHECK();
-        k_ot_rowslice_e<<<g2, 128, 0, st>>>(X, M, U.mp, K, ldx, U.Kp, U.Ex, U.Zx, U.Eb, 0, 1);
+        k_ot_rowslice_e<<<g2, 128, 0, st>>>(X, M, U.mp, K, ldx, U.Kp, U.Ex, U.Zx, U.Eb, 0, 1, 1u << 30);
     }
     LSQ_LAUNCH_CHECK();
-    k_ot_colslice<<<(unsigned)U.Np, 128, 0, st>>>(Y, K, N, U.Np, sk, sj, U.Kp, U.Ey, U.Zy);
+    k_ot_colslice<<<(unsigned)U.Np, 128, 0, st>>>(Y, K, N, U.Np, sk, sj, U.Kp, U.Ey, U.Zy, 0, U.Kp);
     LSQ_LAUNCH_CHECK();
     CUtensorMap tx, ty;
     if (!ot_map(&tx, U.Zx, U.Kp, U.mp, OT_BM) || !ot_map(&ty, U.Zy, U.Kp, U.Np, OT_BN)) return LSQ_ERR_CUDA;
@@ -1276,12 +1286,91 @@ lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t
         LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         const int grid = std::min(ntiles, sms);
         stage_mark(stage, true, st);
-        kern<<<grid, OT_THREADS, smem, st>>>(tx, ty, M, N, K, U.Ex, U.Ey, Cin, ldi, Cout, ldo, err, ntj, ntiles);
+        kern<<<grid, OT_THREADS, smem, st>>>(tx, ty, M, N, K, U.Ex, U.Ey, Cin, ldi, Cout, ldo, err, ntj, ntiles,
+                                               K, 0, ntiles, 0, 0);
     }
     LSQ_LAUNCH_CHECK();
     // tensor-core work: the digit pairs actually issued
     const double pairs = x_digits == 3 ? 21.0 : 36.0;
     stage_mark(stage, false, st, pairs * 2.0 * (double)M * (double)N * (double)K);
+    return LSQ_OK;
+}
+
+// out (M x (N0 + N1), ld M) = -X [Y0 Y1] for a long K (any length; X: M x K
+// column-major, ld ldx, M small; Y0, Y1: K x N0 and K x N1 column-major), FP64
+// accuracy: the operands are sliced in one pass (every K chunk of OT_KMAX with
+// row and column exponents of its own: over the whole K, a reflector's unit
+// entry would set the scale of all its rows, 4.5e-14 against 1.4e-14 of error
+// in R), the chunks run as tiles of one launch into `part` (chunks x M (N0 + N1)) and are
+// summed in chunk order.  Chunk after chunk through ot_gemm_update (five
+// launches each, two row tiles of outputs at a time) left most of the chip
+// idle: the products of one 256-column block of a 4000 x 2000 QR took about
+// 0.9 ms; in one launch the whole QR went from 32.4 to 25.0 ms.
+__global__ void __launch_bounds__(256) k_ot_ksum(const double* __restrict__ part, int64_t count, int chunks,
+                                                 double* __restrict__ out) {
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < count; q += (int64_t)gridDim.x * blockDim.x) {
+        double s = part[q];
+        for (int z = 1; z < chunks; ++z) s += part[(int64_t)z * count + q];
+        out[q] = s;
+    }
+}
+
+size_t ot_gemm_long_ws_bytes(int64_t M, int64_t N, int64_t K) {
+    const size_t chunks = (size_t)ceil_div(K, OT_KMAX);
+    return ot_update_ws_bytes(M, N, K) + align_up(16 * chunks * (size_t)ot_pad(M, OT_BM), 256) +
+           align_up(4 * chunks * (size_t)ot_pad(N, OT_BN), 256);
+}
+
+size_t ot_gemm_long_part_bytes(int64_t M, int64_t N, int64_t K) {
+    return align_up(sizeof(double) * (size_t)M * N * ceil_div(K, OT_KMAX), 256);
+}
+
+lsq_status ot_gemm_long(const double* X, int64_t ldx, const double* Y0, int64_t ld0, int64_t N0, const double* Y1,
+                        int64_t ld1, int64_t N1, double* out, int64_t M, int64_t K, double* part, void* ws,
+                        size_t ws_bytes, int32_t* err, cudaStream_t st) {
+    const int64_t N = N0 + N1;
+    if (M <= 0 || N <= 0 || K <= 0) return LSQ_OK;
+    if (!ws || ws_bytes < ot_gemm_long_ws_bytes(M, N, K)) return LSQ_ERR_ARG;
+    const int chunks = (int)ceil_div(K, OT_KMAX);
+    const int64_t kc = chunks == 1 ? K : OT_KMAX;
+    OtUpd U = ot_upd_ptrs(ws, M, N, K);
+    // the exponents and row maxima of every chunk, behind the planes of one update
+    char* e = (char*)(((uintptr_t)ws + 255) & ~(uintptr_t)255) + ot_update_ws_bytes(M, N, K) - 256;
+    U.Mx = (unsigned long long*)e;
+    U.Ex = (int32_t*)(U.Mx + chunks * U.mp);
+    U.Eb = U.Ex + chunks * U.mp;
+    U.Ey = U.Eb + chunks * U.mp;
+    LSQ_CUDA_TRY(cudaMemsetAsync(U.Mx, 0, sizeof(unsigned long long) * (size_t)(chunks * U.mp), st));
+    const dim3 g2((unsigned)(U.mp / 128), (unsigned)(U.Kp / 64));
+    k_ot_rowmax2d<<<g2, 128, 0, st>>>(X, M, K, ldx, U.Mx, OT_KMAX / 64);
+    LSQ_LAUNCH_CHECK();
+    k_ot_rowexp<<<(unsigned)ceil_div(chunks * M, 256), 256, 0, st>>>(U.Mx, chunks * M, U.Eb);
+    LSQ_LAUNCH_CHECK();
+    k_ot_rowslice_e<<<g2, 128, 0, st>>>(X, M, U.mp, K, ldx, U.Kp, U.Ex, U.Zx, U.Eb, 0, 1, OT_KMAX / 64);
+    LSQ_LAUNCH_CHECK();
+    if (N0 > 0) {
+        k_ot_colslice<<<dim3((unsigned)N0, (unsigned)chunks), 128, 0, st>>>(Y0, K, N0, U.Np, 1, ld0, U.Kp, U.Ey, U.Zy,
+                                                                            0, kc);
+        LSQ_LAUNCH_CHECK();
+    }
+    k_ot_colslice<<<dim3((unsigned)(U.Np - N0), (unsigned)chunks), 128, 0, st>>>(Y1, K, N1, U.Np, 1, ld1, U.Kp, U.Ey,
+                                                                                U.Zy, N0, kc);
+    LSQ_LAUNCH_CHECK();
+    CUtensorMap tx, ty;
+    if (!ot_map(&tx, U.Zx, U.Kp, U.mp, OT_BM) || !ot_map(&ty, U.Zy, U.Kp, U.Np, OT_BN)) return LSQ_ERR_CUDA;
+    const size_t smem = ot_update_smem();
+    LSQ_CUDA_TRY(cudaFuncSetAttribute(k_ot_update<OT_DIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int ntj = (int)(U.Np / OT_BN), zt = (int)(ntj * (U.mp / OT_BM));
+    double* dst = chunks == 1 ? out : part;
+    stage_mark(ST_K_UPDATE, true, st);
+    k_ot_update<OT_DIG><<<std::min(chunks * zt, device_sm_count()), OT_THREADS, smem, st>>>(
+        tx, ty, M, N, K, U.Ex, U.Ey, nullptr, 0, dst, M, err, ntj, chunks * zt, kc, M * N, zt, U.mp, U.Np);
+    LSQ_LAUNCH_CHECK();
+    stage_mark(ST_K_UPDATE, false, st, 36.0 * 2.0 * (double)M * (double)N * (double)K);
+    if (chunks > 1) {
+        k_ot_ksum<<<(unsigned)std::min<int64_t>(ceil_div(M * N, 256), 4096), 256, 0, st>>>(part, M * N, chunks, out);
+        LSQ_LAUNCH_CHECK();
+    }
     return LSQ_OK;
 }
 

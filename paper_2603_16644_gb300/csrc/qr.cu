@@ -1482,19 +1482,18 @@ static QrStreams* qr_streams() {
 // rank-32 updates as above (restricted to the block); then the block's
 // reflectors H_1 ... H_b = I - V T V^T update every later column at once,
 //   W = V^T C,  X = T^T W,  C <- C - V X,
-// each an FP64-accurate digit-sliced product (csrc/oz_trsm.cu; K chunks of
-// at most 512).  T is formed from S = T^{-1} = striu(V^T V) + diag(1/beta)
-// (Puglisi 1992; Joffrain et al. 2006: the triangular factor of the compact
-// WY form is the inverse of that matrix), column by column with the betas
-// as factors (a zero beta, H = I, gives a zero row and column of T).
+// each an FP64-accurate digit-sliced product (csrc/oz_trsm.cu).  T is formed
+// from S = T^{-1} = striu(V^T V) + diag(1/beta) (Puglisi 1992; Joffrain et al.
+// 2006: the triangular factor of the compact WY form is the inverse of that
+// matrix) and the panels' own T factors, the inverses of its diagonal blocks (a
+// zero beta, H = I, gives a zero row and column of T).
 // ---------------------------------------------------------------------------
 constexpr int QTB = 256;  // columns per block of the tensor-core form
-constexpr int QTK = 512;  // K chunk of one digit-sliced product
 
 static bool qr_tc_blocked(int es, int64_t n) { return es == 8 && n > QTB && fp64_emulation_enabled() && ot_trsm_supported(); }
 
 struct QrTcLayout {
-    size_t vx, vt, g, tt, wn, xp, err, ot, ot_bytes, total;
+    size_t vx, vt, gw, part, tt, tp, xp, err, ot, ot_bytes, total;
 };
 
 static QrTcLayout qr_tc_layout(int64_t s, int64_t n) {
@@ -1503,12 +1502,14 @@ static QrTcLayout qr_tc_layout(int64_t s, int64_t n) {
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
     L.vx = take(sizeof(double) * (size_t)s * QTB);
     L.vt = take(sizeof(double) * (size_t)s * QTB);
-    L.g = take(sizeof(double) * QTB * QTB);
+    L.gw = take(sizeof(double) * QTB * (size_t)n);  // -V^T [V C] (V and C: at most n columns)
+    L.part = take(ot_gemm_long_part_bytes(QTB, n, s));
     L.tt = take(sizeof(double) * QTB * QTB);
-    L.wn = take(sizeof(double) * QTB * (size_t)n);
+    L.tp = take(sizeof(double) * QNB * QTB);  // the T factors of the block's panels
     L.xp = take(sizeof(double) * QTB * (size_t)n);
     L.err = take(sizeof(int32_t));
-    L.ot_bytes = ot_update_ws_bytes(std::max<int64_t>(s, QTB), std::max<int64_t>(n, QTB), QTK);
+    L.ot_bytes = std::max(ot_gemm_long_ws_bytes(QTB, n, s),
+                          ot_update_ws_bytes(std::max<int64_t>(s, QTB), std::max<int64_t>(n, QTB), QTB));
     L.ot = take(L.ot_bytes);
     L.total = off;
     return L;
@@ -1528,23 +1529,38 @@ __global__ void k_qr_vblock(const double* __restrict__ W, int64_t ld, int64_t j0
     }
 }
 
-// T^T (ld nb) from Gn = -V^T V and the betas: column j of T by back
-// substitution, t_j = beta_j, t_i = -beta_i sum_{i < p <= j} S[i][p] t_p with
-// S[i][p] = (V^T V)[i][p]; one warp per column, the sums over lanes in a
-// fixed order.
-__global__ void __launch_bounds__(32) k_qr_tinv(const double* __restrict__ Gn, const double* __restrict__ beta,
-                                                 int nb, double* __restrict__ Tt) {
+// T^T (ld nb) of the block from Gn = -V^T V (ld nb) and the T factors of its
+// panels (Tp: panel q's 32 x 32 T at Tp + 1024 q, column-major, zero below the
+// diagonal and past its columns).  With S = T^{-1} = striu(V^T V) + diag(1/beta),
+// column j of T by back substitution over 32-row blocks,
+//   t_I = -T_II sum_{J > I} S[I, J] t_J,   t_J(j) = T_JJ[:, j] in j's own block:
+// the diagonal blocks of S are inverted already (the panels' T), so that a block
+// takes two matrix-vector products and no chain of 32 steps (one warp per
+// column walking its 256 rows one by one took 232 us).  One warp
+// per column, lane = row of the block.
+__global__ void __launch_bounds__(32) k_qr_tblock(const double* __restrict__ Gn, const double* __restrict__ Tp, int nb,
+                                                   double* __restrict__ Tt) {
     __shared__ double t[QTB];
-    const int j = blockIdx.x, lane = threadIdx.x;
-    for (int i = lane; i < nb; i += 32) t[i] = 0.0;
+    __shared__ double rhs[QNB];
+    const int j = blockIdx.x, lane = threadIdx.x, jb = j / QNB;
+    t[jb * QNB + lane] = Tp[1024 * jb + lane + (j % QNB) * QNB];
+    for (int I = jb + 1; I * QNB < nb; ++I) t[I * QNB + lane] = 0.0;
     __syncwarp();
-    if (lane == 0) t[j] = beta[j];
-    __syncwarp();
-    for (int i = j - 1; i >= 0; --i) {
-        double acc = 0.0;
-        for (int p = i + 1 + lane; p <= j; p += 32) acc = fma(-Gn[i + (int64_t)p * nb], t[p], acc);
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) t[i] = -beta[i] * acc;
+    for (int I = jb - 1; I >= 0; --I) {
+        const int i = I * QNB + lane;  // only the last block can be ragged, and I is not it
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        const int p1 = min(nb, (jb + 1) * QNB);
+        int p = (I + 1) * QNB;
+        for (; p + 4 <= p1; p += 4)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] = fma(-Gn[i + (int64_t)(p + q) * nb], t[p + q], s[q]);
+        for (; p < p1; ++p) s[0] = fma(-Gn[i + (int64_t)p * nb], t[p], s[0]);
+        rhs[lane] = (s[0] + s[1]) + (s[2] + s[3]);
+        __syncwarp();
+        double w[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < QNB; ++q) w[q & 3] = fma(Tp[1024 * I + lane + q * QNB], rhs[q], w[q & 3]);
+        t[i] = -((w[0] + w[1]) + (w[2] + w[3]));
         __syncwarp();
     }
     for (int i = lane; i < nb; i += 32) Tt[j + (int64_t)i * nb] = t[i];
@@ -1556,15 +1572,15 @@ __global__ void k_qr_err_to_info(const int32_t* __restrict__ err, int32_t* __res
 
 // C (rows x nt, ld s) <- (I - V T^T V^T) C for the block of nb reflectors
 // stored in W's columns j0 .. j0 + nb - 1 (C: W's rows j0.., columns j0 + nb..).
-static lsq_status qr_tc_trailing(double* W, int64_t s, int64_t j0, int nb, int64_t n, const double* beta, char* base,
-                                 const QrTcLayout& L, cudaStream_t st) {
+static lsq_status qr_tc_trailing(double* W, int64_t s, int64_t j0, int nb, int64_t n, char* base, const QrTcLayout& L,
+                                 cudaStream_t st) {
     const int64_t rows = s - j0, nt = n - j0 - nb;
     if (nt <= 0) return LSQ_OK;
     double* Vx = (double*)(base + L.vx);
     double* Vt = (double*)(base + L.vt);
-    double* Gn = (double*)(base + L.g);
+    double* Gn = (double*)(base + L.gw);
+    double* Wn = Gn + (int64_t)nb * nb;
     double* Tt = (double*)(base + L.tt);
-    double* Wn = (double*)(base + L.wn);
     double* Xp = (double*)(base + L.xp);
     int32_t* err = (int32_t*)(base + L.err);
     char* ows = base + L.ot;
@@ -1573,19 +1589,11 @@ static lsq_status qr_tc_trailing(double* W, int64_t s, int64_t j0, int nb, int64
     k_qr_vblock<<<(unsigned)std::min<int64_t>(ceil_div(rows * nb, 256), 8192), 256, 0, st>>>(W, s, j0, rows, nb, Vx,
                                                                                               Vt);
     LSQ_LAUNCH_CHECK();
-    // Gn = -V^T V and Wn = -V^T C, accumulated over K chunks of the rows
-    LSQ_CUDA_TRY(cudaMemsetAsync(Gn, 0, sizeof(double) * nb * nb, st));
-    LSQ_CUDA_TRY(cudaMemsetAsync(Wn, 0, sizeof(double) * nb * (size_t)nt, st));
-    for (int64_t k = 0; k < rows; k += QTK) {
-        const int64_t kc = std::min<int64_t>(QTK, rows - k);
-        if ((r = ot_gemm_update(Vt + k * nb, nb, Vx + k, 1, rows, Gn, nb, Gn, nb, nb, nb, kc, ows, L.ot_bytes, err,
-                                st)) != LSQ_OK)
-            return r;
-        if ((r = ot_gemm_update(Vt + k * nb, nb, C + k, 1, s, Wn, nb, Wn, nb, nb, nt, kc, ows, L.ot_bytes, err, st)) !=
-            LSQ_OK)
-            return r;
-    }
-    k_qr_tinv<<<(unsigned)nb, 32, 0, st>>>(Gn, beta + j0, nb, Tt);
+    // [Gn Wn] = -V^T [V C]
+    if ((r = ot_gemm_long(Vt, nb, Vx, rows, nb, C, s, nt, Gn, nb, rows, (double*)(base + L.part), ows, L.ot_bytes, err,
+                          st)) != LSQ_OK)
+        return r;
+    k_qr_tblock<<<(unsigned)nb, 32, 0, st>>>(Gn, (const double*)(base + L.tp), nb, Tt);
     LSQ_LAUNCH_CHECK();
     // Xp = 0 - T^T Wn = T^T (V^T C)
     LSQ_CUDA_TRY(cudaMemsetAsync(Xp, 0, sizeof(double) * nb * (size_t)nt, st));
@@ -1624,7 +1632,7 @@ static lsq_status qr_blocked_f64(double* W, double* beta, int64_t s, int64_t n, 
             const int b = k & 1;
             const int nb = (int)std::min<int64_t>(QNB, j1 - k0);
             const int64_t rows = s - k0;
-            double* Tm = (double*)(base + L.tm[b]);
+            double* Tm = (double*)(tcb + TL.tp) + 1024 * ((k0 - j0) / QNB);
             double* V = (double*)(base + L.v[b]);
             if (qcl > 0) {
                 const size_t clsm = qr_cluster_smem<double>(rows, qcl, qc.fused);
@@ -1656,7 +1664,7 @@ static lsq_status qr_blocked_f64(double* W, double* beta, int64_t s, int64_t n, 
             ldvprev = rows;
         }
         // the block's reflectors on every later column
-        r = qr_tc_trailing(W, s, j0, (int)(j1 - j0), n, beta, tcb, TL, st);
+        r = qr_tc_trailing(W, s, j0, (int)(j1 - j0), n, tcb, TL, st);
     }
     if (r != LSQ_OK) return r;
     k_qr_extract<double><<<(unsigned)std::min<int64_t>(ceil_div(n * n, 256), 4096), 256, 0, st>>>(W, s, n, colexp, Rs,
