@@ -325,48 +325,45 @@ __global__ void __launch_bounds__(128) k_ot_colslice(const double* __restrict__ 
 // ---------------------------------------------------------------------------
 // Update C_out = C_in - X Y over 128 x 64 tiles (C_in may equal C_out).
 // ---------------------------------------------------------------------------
-// Results outside the normal range (rare): scaled in FP64.  Not inlined, so
-// that the FP64 instructions of this path are never executed speculatively.
-__device__ __noinline__ double ot_fixed_to_double_slow(long long hi, long long lo, int s) {
-    return ldexp(fma((double)hi, 268435456.0, (double)lo), s);
-}
+// 2^s (256 S + low) for |S| < 2^63, 0 <= low < 256, rounded once to
+// nearest-even.  The magnitude is normalised to 64 bits (top bit set, the bits
+// below it in `sticky`), the significand rounded off its upper 53, and added to
+// the exponent field, so that a carry moves to the next binade by itself.
+// Results outside the normal range (rare) are scaled by exact powers of two
+// (inlined: a call would spill the sums held in registers; the FP64 pipe takes
+// 16 cycles an instruction and SM, so that running these products for every
+// value and selecting cost three times the conversion).
+__device__ __forceinline__ double ot_pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
 
-// 2^s (hi 2^28 + lo) for |hi|, |lo| < 2^47, rounded once to nearest-even:
-// the exact integer (below 2^76) is normalised with integer operations and
-// the scale goes into the exponent field (no FP64 instruction on the common
-// path).  Straight-line code (selects), so that the compiler interleaves
-// independent conversions; the epilogue's throughput is bound by these
-// integer operations when K is small.
-__device__ __forceinline__ double ot_fixed_to_double(long long hi, long long lo, int s) {
-    unsigned long long L = (unsigned long long)hi << 28;
-    long long H = hi >> 36;
-    const unsigned long long L2 = L + (unsigned long long)lo;
-    H += (lo >> 63) + (L2 < L ? 1 : 0);
-    L = L2;
-    // magnitude: two's-complement negation of (H:L) when negative (H < 2^11)
-    const unsigned long long sgn = (unsigned long long)(H >> 63);
-    const unsigned long long neg = sgn & 1ull;
-    const unsigned long long uL = (L ^ sgn) + neg;
-    const unsigned long long uH = ((unsigned long long)H ^ sgn) + (neg & (uL == 0 ? 1ull : 0ull));
-    const bool zero = (uH | uL) == 0;
-    int p = uH ? 127 - __clzll((long long)uH) : 63 - __clzll((long long)uL);
-    const int shl = p <= 52 ? 52 - p : 0;  // 0 .. 52
-    const int shr = p > 52 ? p - 52 : 0;   // 0 .. 22
-    const unsigned long long small = uL << shl;
-    const unsigned long long big = (uL >> shr) | (shr ? (uH << ((64 - shr) & 63)) : 0ull);
-    unsigned long long mant = p > 52 ? big : small;
-    const unsigned long long rb = shr ? (uL >> ((shr - 1) & 63)) & 1ull : 0ull;
-    const bool sticky = shr > 1 ? (uL & ((1ull << ((shr - 1) & 63)) - 1ull)) != 0 : false;
-    mant += (rb && (sticky || (mant & 1ull))) ? 1ull : 0ull;
-    const bool carry = mant == (1ull << 53);
-    mant = carry ? mant >> 1 : mant;
-    p += carry ? 1 : 0;
-    const int E = p + s + 1023;
-    double r = __longlong_as_double((long long)((sgn & 0x8000000000000000ull) | ((unsigned long long)(E & 2047) << 52) |
-                                                (mant & 0x000fffffffffffffull)));
-    if (zero) r = 0.0;
-    if (!zero && (E <= 0 || E >= 2047)) r = ot_fixed_to_double_slow(hi, lo, s);
-    return r;
+__device__ __forceinline__ double ot_fixed_to_double(long long S, unsigned low, int s) {
+    const bool neg = S < 0;
+    // magnitude: -(256 S + low) = 256 (~S) + (256 - low)
+    unsigned lo = neg ? 256u - low : low;  // 1 .. 256 when negative
+    unsigned long long hi = (unsigned long long)(neg ? ~S : S) + (lo >> 8);
+    lo &= 255u;
+    const bool small = hi == 0;  // below 2^8: 256 times as large a unit
+    hi = small ? (unsigned long long)lo : hi;
+    lo = small ? 0u : lo;
+    const int z = __clzll((long long)hi);  // 64 only when the value is 0
+    const unsigned long long n = (hi << (z & 63)) | ((((unsigned long long)lo << 56) >> 1) >> ((63 - z) & 63));
+    const bool sticky = z < 8 && (lo & ((1u << (8 - z)) - 1u)) != 0;
+    const unsigned rem = (unsigned)n & 0x7ffu;
+    unsigned long long mant = n >> 11;
+    mant += (rem > 0x400u || (rem == 0x400u && (sticky || (mant & 1ull)))) ? 1ull : 0ull;
+    const int E = 71 - z + s + 1023 - (small ? 8 : 0);  // exponent field of a magnitude in [2^(71-z), 2^(72-z))
+    const unsigned long long sgn = neg ? 0x8000000000000000ull : 0ull;
+    double r = __longlong_as_double((long long)((((unsigned long long)(unsigned)(E - 1) << 52) + mant) | sgn));
+    if ((unsigned)(E - 1) >= 2045u) {
+        r = __longlong_as_double((long long)(((1022ull << 52) + mant) | sgn));
+        int e = E - 1023;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int k = max(-1000, min(1000, e));
+            asm volatile("mul.rn.f64 %0, %0, %1;" : "+d"(r) : "d"(ot_pow2(k)));  // volatile: not run speculatively
+            e -= k;
+        }
+    }
+    return hi == 0 ? 0.0 : r;
 }
 
 // Persistent: one CTA per SM walks the tiles (column tiles fastest, so that
@@ -579,7 +576,10 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
         auto epi = [&](auto Wc, int64_t row, int64_t c0, int64_t z) {
             constexpr int W = decltype(Wc)::value;
             const uint32_t tl = tq + (uint32_t)(cq * W);
-            long long hi[W], lo[W];
+            // I = sum_d S_d 128^(7 - d) as 256 st + low (see ot_fixed_to_double):
+            // sum_{d <= 5} S_d 128^(5 - d) below 2^57, then 6 bits and 8 more
+            long long st[W];
+            uint32_t low[W / 4];
 #pragma unroll
             for (int d = 0; d < OT_DIG; d += 2) {
                 uint32_t va[W], vb[W];
@@ -593,43 +593,51 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
                 tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < W; ++j) {
-                    const long long a = (long long)__float2int_rn(__uint_as_float(va[j]));
-                    const long long b = (long long)__float2int_rn(__uint_as_float(vb[j]));
-                    if (d == 0) hi[j] = a * 128 + b;
-                    else if (d == 2) hi[j] = (hi[j] * 128 + a) * 128 + b;
-                    else if (d == 4) lo[j] = a * 128 + b;
-                    else lo[j] = (lo[j] * 128 + a) * 128 + b;
+                    const long long v = (long long)__float2int_rn(__uint_as_float(va[j])) * 128 +
+                                        (long long)__float2int_rn(__uint_as_float(vb[j]));
+                    if (d == 0) st[j] = v;
+                    else if (d < 6) st[j] = st[j] * 16384 + v;
+                    else {
+                        st[j] = st[j] * 64 + (v >> 8);
+                        const uint32_t l8 = (uint32_t)v & 255u;
+                        low[j >> 2] = (j & 3) ? low[j >> 2] | (l8 << (8 * (j & 3))) : l8;
+                    }
                 }
             }
             // this tile's TMEM is read: the next tile's MMAs may start
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(tfree);
-            if (row < m) {
-                const int32_t ex = Ex[z * zx + row];
+            const int32_t ex = row < m ? Ex[z * zx + row] : 0;
+            const int nrem = row < m ? (int)min64(W, N - c0) : 0;
+            const int32_t eyl = lane < W && c0 + lane < N ? Ey[z * zy + c0 + lane] : 0;  // lane's column
+            const double* ci = Cin + row + c0 * ldi;
+            double* co = Cout + z * zs + row + c0 * ldo;
+            // rolled, the sums moved down four registers an iteration (see
+            // k_ot_update2: unrolled, this is bound by the instruction caches)
+#pragma unroll 1
+            for (int g = 0; g < W / 4; ++g) {
+                double cin[4], val[4];
 #pragma unroll
-                for (int h = 0; h < W / 8; ++h) {
-                    double cin[8];
-                    int32_t ey[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int64_t col = c0 + 8 * h + j;
-                        cin[j] = col < N && Cin ? Cin[row + col * ldi] : 0.0;
-                        ey[j] = col < N ? Ey[z * zy + col] : 0;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int64_t col = c0 + 8 * h + j;
-                        if (col < N) {
-                            double val;
-                            if (ex == OT_NONFINITE || ey[j] == OT_NONFINITE)
-                                val = __longlong_as_double(0x7ff8000000000000ll);
-                            else
-                                val = ot_fixed_to_double(hi[8 * h + j], lo[8 * h + j], ex + ey[j] - 61);
-                            Cout[z * zs + row + col * ldo] = cin[j] - val;
-                        }
-                    }
+                for (int j = 0; j < 4; ++j) {
+                    cin[j] = Cin && 4 * g + j < nrem ? *ci : 0.0;
+                    ci += ldi;
                 }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int32_t ey = __shfl_sync(0xffffffffu, eyl, 4 * g + j);
+                    val[j] = ot_fixed_to_double(st[j], (low[0] >> (8 * j)) & 255u, ex + ey - 61);
+                    if (ex == OT_NONFINITE || ey == OT_NONFINITE) val[j] = __longlong_as_double(0x7ff8000000000000ll);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (4 * g + j < nrem) *co = cin[j] - val[j];
+                    co += ldo;
+                }
+#pragma unroll
+                for (int c = 0; c + 4 < W; ++c) st[c] = st[c + 4];
+#pragma unroll
+                for (int w = 0; w + 1 < W / 4; ++w) low[w] = low[w + 1];
             }
         };
         for (int i = 0; i < ntl; ++i) {
@@ -714,47 +722,6 @@ constexpr int O2_THREADS = 32 * (4 + O2_EPI_WARPS);  // warp 0 TMA, warps 1-2 MM
 // with twice the columns: the conversion is a chain of integer operations, and
 // 8 warps left it bound by their latency.
 constexpr int O2_REG_LO = 32, O2_REG_HI = 112;
-
-// 2^s (256 S + low) for |S| < 2^63, 0 <= low < 256, rounded once to
-// nearest-even.  The magnitude is normalised to 64 bits (top bit set, the bits
-// below it in `sticky`), the significand rounded off its upper 53, and added to
-// the exponent field, so that a carry moves to the next binade by itself.
-// Results outside the normal range (rare) are scaled by exact powers of two
-// (inlined: a call would spill the sums held in registers; the FP64 pipe takes
-// 16 cycles an instruction and SM, so that running these products for every
-// value and selecting cost three times the conversion).
-__device__ __forceinline__ double o2_pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
-
-__device__ __forceinline__ double o2_fixed_to_double(long long S, unsigned low, int s) {
-    const bool neg = S < 0;
-    // magnitude: -(256 S + low) = 256 (~S) + (256 - low)
-    unsigned lo = neg ? 256u - low : low;  // 1 .. 256 when negative
-    unsigned long long hi = (unsigned long long)(neg ? ~S : S) + (lo >> 8);
-    lo &= 255u;
-    const bool small = hi == 0;  // below 2^8: 256 times as large a unit
-    hi = small ? (unsigned long long)lo : hi;
-    lo = small ? 0u : lo;
-    const int z = __clzll((long long)hi);  // 64 only when the value is 0
-    const unsigned long long n = (hi << (z & 63)) | ((((unsigned long long)lo << 56) >> 1) >> ((63 - z) & 63));
-    const bool sticky = z < 8 && (lo & ((1u << (8 - z)) - 1u)) != 0;
-    const unsigned rem = (unsigned)n & 0x7ffu;
-    unsigned long long mant = n >> 11;
-    mant += (rem > 0x400u || (rem == 0x400u && (sticky || (mant & 1ull)))) ? 1ull : 0ull;
-    const int E = 71 - z + s + 1023 - (small ? 8 : 0);  // exponent field of a magnitude in [2^(71-z), 2^(72-z))
-    const unsigned long long sgn = neg ? 0x8000000000000000ull : 0ull;
-    double r = __longlong_as_double((long long)((((unsigned long long)(unsigned)(E - 1) << 52) + mant) | sgn));
-    if ((unsigned)(E - 1) >= 2045u) {
-        r = __longlong_as_double((long long)(((1022ull << 52) + mant) | sgn));
-        int e = E - 1023;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const int k = max(-1000, min(1000, e));
-            asm volatile("mul.rn.f64 %0, %0, %1;" : "+d"(r) : "d"(o2_pow2(k)));  // volatile: not run speculatively
-            e -= k;
-        }
-    }
-    return hi == 0 ? 0.0 : r;
-}
 
 // Stages of pass p: X digits t < XD with a partner, and the Y digit that only
 // group 2p needs when the X digits end before it.
@@ -1015,7 +982,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(O2_THREADS, 1)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int32_t ey = __shfl_sync(0xffffffffu, eyl, 4 * g + j);
-                    val[j] = o2_fixed_to_double(st[j], (low[0] >> (8 * j)) & 255u, ex + ey - 61);
+                    val[j] = ot_fixed_to_double(st[j], (low[0] >> (8 * j)) & 255u, ex + ey - 61);
                     if (ex == OT_NONFINITE || ey == OT_NONFINITE) val[j] = __longlong_as_double(0x7ff8000000000000ll);
                 }
 #pragma unroll
