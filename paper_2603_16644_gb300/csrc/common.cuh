@@ -152,6 +152,16 @@ __device__ __forceinline__ uint32_t quant_bits(double x, int escale, int prec) {
     unsigned long long b = (unsigned long long)__double_as_longlong(x);
     uint32_t sign = (uint32_t)(b >> 63) << (tot - 1);
     int E = (int)((b >> 52) & 0x7ff);
+    // Normal results away from the overflow threshold (nearly all): round the
+    // significand to nearest-even on the FP64 pattern, a carry moving into the
+    // exponent field by itself, and rebias.
+    const int ef = E + escale - 1023 + bias;
+    if ((unsigned)(ef - 1) < (unsigned)(emax + bias - 1) && E != 0 && E != 0x7ff) {
+        const int dr = 52 - mb;
+        const unsigned long long mag = b & 0x7fffffffffffffffull;
+        const unsigned long long r = (mag + ((1ull << (dr - 1)) - 1ull) + ((mag >> dr) & 1ull)) >> dr;
+        return sign | ((uint32_t)r + ((uint32_t)(escale - 1023 + bias) << mb));
+    }
     unsigned long long mant = b & 0x000fffffffffffffull;
     const uint32_t inf_bits = ((1u << ebits) - 1u) << mb;
     const uint32_t sat_bits = prec == LSQ_FP8_E4M3 ? 0x7Eu : inf_bits;  // 448 for e4m3fn
