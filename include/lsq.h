@@ -448,9 +448,10 @@ size_t lsq_batched_workspace_size(int32_t hpne, int32_t count, const lsq_batch_p
  * $LSQ_BATCH_STREAMS, 1 to 64, read once per process; the workspace size
  * grows with it), heaviest first to the least-loaded stream, and the whole
  * fan-out is captured into one
- * CUDA graph launched on `stream`; the executable graph is cached and
- * replayed while the descriptors (pointers, shapes, options, workspace) stay
- * the same.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
+ * CUDA graph; the executable graph is cached and replayed on `stream` while
+ * the descriptors (pointers, shapes, options, workspace) stay the same.  A
+ * call with new descriptors enqueues the fan-out directly (forked from and
+ * joined to `stream`) and captures the graph while the GPU works.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
  * batched condition-estimate pass (the same fan-out, in a cached graph of
  * its own) and one readback of the chosen precisions (a stream
  * synchronisation).  Each problem's status goes to its own info.

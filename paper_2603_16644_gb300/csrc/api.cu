@@ -49,6 +49,11 @@ lsq_status reduce_partial(void* buf, int64_t count, int kind, cudaStream_t st) {
     int32_t r = g_reduce_fn(buf, count, kind, (void*)st, g_reduce_user);
     return r == LSQ_OK ? LSQ_OK : LSQ_ERR_CUDA;
 }
+bool reduce_hook_set() { return g_reduce_fn != nullptr; }
+bool profiling_on() {
+    std::lock_guard<std::mutex> lk(g_prof.mu);
+    return g_prof.on;
+}
 void note_cuda_error(cudaError_t e) { g_last_cuda_error.store((int)e); }
 
 void stage_mark(int stage, bool begin, cudaStream_t st, double work) {

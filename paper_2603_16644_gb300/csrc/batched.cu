@@ -3,9 +3,11 @@
 // The problems are spread over a fixed set of internal streams (heaviest
 // first, each to the least-loaded stream), and the whole fan-out -- every
 // kernel of every problem plus the fork/join events -- is captured into one
-// CUDA graph that is launched on the caller's stream.  The executable graph
-// is cached and replayed while the batch description is unchanged, so a
-// repeated batched call is one graph launch.  Problems asking for the AUTO
+// CUDA graph.  The executable graph is cached and replayed while the batch
+// description is unchanged, so a repeated batched call is one graph launch on
+// the caller's stream; a call with a new description enqueues the fan-out on
+// the internal streams and captures it while the GPU works.  Problems asking
+// for the AUTO
 // precision first get one batched condition-estimate pass (Sec. 6.1; on A^T A
 // for AUTO, on a sketch for AUTO_SKETCH) and a single readback of the chosen
 // precisions, because kernel selection in the captured graph needs them on
@@ -130,12 +132,51 @@ lsq_status check_problem(const lsq_batch_problem& p) {
 
 bool is_auto(int p) { return p == LSQ_AUTO || p == LSQ_AUTO_SKETCH; }
 
-// Capture a fan-out of per-problem work over the internal streams into one
-// graph (cached in `cache` under `key`) and launch it on st.  run(i, stream,
-// slot) enqueues problem i.  Every pass over the internal streams is such a
-// graph: while a stream is captured, no step of a problem forks onto the
-// library's shared look-ahead streams, so concurrent problems never share a
-// stream.  Caller holds g_batch.mu.
+// The fan-out on the internal streams, forked from and joined to `from` by
+// events: captured into a graph when `from` is being captured, else enqueued.
+template <typename F>
+lsq_status enqueue_fanout(cudaStream_t from, const std::vector<int>& order, const std::vector<int>& stream_of,
+                          char* slots, size_t slot_bytes, F run) {
+    lsq_status r = LSQ_OK;
+    if (cudaEventRecord(g_batch.fork, from) != cudaSuccess) return LSQ_ERR_CUDA;
+    for (int k = 0; k < n_streams() && r == LSQ_OK; ++k)
+        if (cudaStreamWaitEvent(g_batch.sub[k], g_batch.fork, 0) != cudaSuccess) r = LSQ_ERR_CUDA;
+    for (int i : order) {
+        if (r != LSQ_OK) break;
+        int k = stream_of[i];
+        r = run(i, g_batch.sub[k], slots + (size_t)k * slot_bytes);
+    }
+    // joined after a failure too: what was enqueued uses the caller's buffers
+    for (int k = 0; k < n_streams(); ++k)
+        if ((cudaEventRecord(g_batch.join[k], g_batch.sub[k]) != cudaSuccess ||
+             cudaStreamWaitEvent(from, g_batch.join[k], 0) != cudaSuccess) &&
+            r == LSQ_OK)
+            r = LSQ_ERR_CUDA;
+    return r;
+}
+
+// Whether a new fan-out is enqueued directly before it is captured: not when the
+// caller's own stream is being captured, nor while a reduction hook or the
+// stage timing would see every step twice.
+bool direct_ok(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cap == cudaStreamCaptureStatusNone && !reduce_hook_set() && !profiling_on();
+}
+
+// A fan-out of per-problem work over the internal streams, run(i, stream, slot)
+// enqueuing problem i: one graph (cached in `cache` under `key`) launched on st.
+// Under a new key the work is enqueued on the internal streams directly and
+// the graph captured while the GPU runs it: capturing and instantiating the
+// thousands of launches of 64 solves takes ~46 ms of host time, which the GPU
+// waited for (145 ms a pass over ever new batches of 64 uneven problems, 113
+// now; 99 ms when the same batch is repeated).  No step of a problem forks onto
+// the library's shared look-ahead streams here (FanoutScope; captured or
+// not), so concurrent problems never share a stream and both ways run the same
+// kernels.  Caller holds g_batch.mu.
 template <typename F>
 lsq_status capture_fanout(GraphCache& cache, const std::vector<int>& order, const std::vector<int>& stream_of,
                           char* slots, size_t slot_bytes, std::vector<unsigned char>& key, cudaStream_t st, F run) {
@@ -144,37 +185,35 @@ lsq_status capture_fanout(GraphCache& cache, const std::vector<int>& order, cons
         return LSQ_OK;
     }
     cache.drop();
+    FanoutScope scope;
+    const bool direct = direct_ok(st);
+    if (direct) {
+        lsq_status r = enqueue_fanout(st, order, stream_of, slots, slot_bytes, run);
+        if (r != LSQ_OK) return r;
+    }
     cudaGraph_t graph = nullptr;
     // Capture on an internal stream (the caller may use the legacy default
     // stream, which cannot be captured); the graph is then launched on st.
     cudaStream_t cs = g_batch.cap;
     LSQ_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
-    lsq_status cap = LSQ_OK;
-    if (cudaEventRecord(g_batch.fork, cs) != cudaSuccess) cap = LSQ_ERR_CUDA;
-    for (int k = 0; k < n_streams() && cap == LSQ_OK; ++k)
-        if (cudaStreamWaitEvent(g_batch.sub[k], g_batch.fork, 0) != cudaSuccess) cap = LSQ_ERR_CUDA;
-    for (int i : order) {
-        if (cap != LSQ_OK) break;
-        int k = stream_of[i];
-        cap = run(i, g_batch.sub[k], slots + (size_t)k * slot_bytes);
-    }
-    for (int k = 0; k < n_streams() && cap == LSQ_OK; ++k) {
-        if (cudaEventRecord(g_batch.join[k], g_batch.sub[k]) != cudaSuccess) cap = LSQ_ERR_CUDA;
-        else if (cudaStreamWaitEvent(cs, g_batch.join[k], 0) != cudaSuccess) cap = LSQ_ERR_CUDA;
-    }
+    const lsq_status cap = enqueue_fanout(cs, order, stream_of, slots, slot_bytes, run);
     cudaError_t ec = cudaStreamEndCapture(cs, &graph);
     if (cap != LSQ_OK || ec != cudaSuccess || !graph) {
         if (graph) cudaGraphDestroy(graph);
         cudaGetLastError();  // do not leave a capture error behind for the caller
+        if (direct) return LSQ_OK;  // the work is enqueued; the next call tries to capture it again
         return cap != LSQ_OK ? cap : LSQ_ERR_CUDA;
     }
     cudaGraphExec_t exec = nullptr;
     cudaError_t ei = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
-    if (ei != cudaSuccess) return LSQ_ERR_CUDA;
+    if (ei != cudaSuccess) {
+        cudaGetLastError();
+        return direct ? LSQ_OK : LSQ_ERR_CUDA;
+    }
     cache.exec = exec;
     cache.key.swap(key);
-    LSQ_CUDA_TRY(cudaGraphLaunch(cache.exec, st));
+    if (!direct) LSQ_CUDA_TRY(cudaGraphLaunch(cache.exec, st));
     return LSQ_OK;
 }
 

@@ -178,6 +178,25 @@ lsq_status hager_inv_norm1(const float* M, int64_t n, int64_t ld, bool upper, co
 // ||M||_1 (upper: of the upper triangle) into *out (device float).
 lsq_status launch_colnorm1_max(const float* M, int64_t n, int64_t ld, bool upper, float* out, cudaStream_t st);
 
+// Whether a reduction hook is registered / the stage timing is on (api.cu).
+bool reduce_hook_set();
+bool profiling_on();
+
+// While one lives, this thread's steps stay on the stream they are given (no
+// look-ahead on the library's shared streams): the batched fan-out, whose
+// problems run side by side.
+struct FanoutScope {
+    FanoutScope() { ++depth(); }
+    ~FanoutScope() { --depth(); }
+    static bool active() { return depth() > 0; }
+
+private:
+    static int& depth() {
+        static thread_local int d = 0;
+        return d;
+    }
+};
+
 // ---- qr.cu -------------------------------------------------------------------
 size_t qr_ws_bytes(int64_t s, int64_t n, int prec);
 lsq_status launch_precond_qr(const void* As, int64_t s, int64_t n, int64_t ldas, int as_prec, int qr_prec,

@@ -1704,11 +1704,12 @@ static lsq_status qr_run(const void* As, int64_t s, int64_t n, int64_t ldas, int
     // look-ahead: while panel k + 1 is factored (high-priority stream), the
     // wide part of panel k's trailing update runs on the low-priority stream;
     // the narrow part (the next panel's columns) goes first on the panel
-    // stream.  Not while the caller's stream is being captured into a graph
-    // (the batched solver), where concurrent problems must not share streams.
+    // stream.  Not while the caller's stream is being captured into a graph, nor
+    // in the batched solver, where concurrent problems must not share streams.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     LSQ_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-    QrStreams* qs = (cap == cudaStreamCaptureStatusNone && n > 2 * QNB) ? qr_streams() : nullptr;
+    QrStreams* qs =
+        (cap == cudaStreamCaptureStatusNone && !FanoutScope::active() && n > 2 * QNB) ? qr_streams() : nullptr;
     std::unique_lock<std::mutex> lk(g_qr_mu, std::defer_lock);
     cudaEvent_t ev_fork = nullptr, ev_p = nullptr, ev_w[2] = {nullptr, nullptr}, ev_join = nullptr;
     auto cleanup = [&]() {
