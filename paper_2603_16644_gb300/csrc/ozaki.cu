@@ -273,6 +273,78 @@ __global__ void __launch_bounds__(OZ_CB_THREADS) k_oz_combine(const float* __res
     }
 }
 
+// The same combination for few blocks (small n): 4 columns per CTA, two entries
+// per thread, the tiles of a weight class loaded four at a time (transposed ones
+// directly).  32 columns per CTA and one tile after the other left a single
+// block's sums to 4 CTAs that walked 66 tiles in a chain: 106 us for n = 100
+// (a 1000 x 100 solve went from 875 to 802 us with this and the tile list by warps).
+__global__ void __launch_bounds__(OZ_CB_THREADS) k_oz_combine_few(const float* __restrict__ T,
+                                                                  const int32_t* __restrict__ pair_tile,
+                                                                  int64_t ntiles, int chunks, int64_t n, int64_t nb,
+                                                                  const int32_t* __restrict__ ex,
+                                                                  const int32_t* __restrict__ ey, int sym,
+                                                                  double* __restrict__ G, int64_t ldg) {
+    const int c0 = (int)(blockIdx.x & 31) * 4;
+    const int64_t blk = blockIdx.x >> 5;
+    int64_t P, Q;
+    if (sym) {
+        P = 0;
+        while ((P + 1) * (P + 2) / 2 <= blk) ++P;
+        Q = blk - P * (P + 1) / 2;
+    } else {
+        P = blk % nb;
+        Q = blk / nb;
+    }
+    const int r = threadIdx.x & 127, cb = c0 + (threadIdx.x >> 7);  // columns cb, cb + 2
+    if (P * 128 + r >= n || Q * 128 + c0 >= n) return;
+    long long H[2] = {0, 0};
+    unsigned long long L[2] = {0, 0};
+    for (int d = 0; d < OZ_S; ++d) {
+        long long S[2] = {0, 0};
+        for (int z = 0; z < chunks; ++z)
+            for (int t0 = 0; t0 <= d; t0 += 4) {
+                float v[4][2];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    v[q][0] = v[q][1] = 0.f;
+                    if (t0 + q <= d) {
+                        bool tr;
+                        const int64_t base = oz_item_base(pair_tile, ntiles, nb, P, Q, d, t0 + q, z, tr);
+                        if (base >= 0) {
+                            const float* src = T + base + (tr ? r * 128 + cb : r + cb * 128);
+                            v[q][0] = src[0];
+                            v[q][1] = src[tr ? 2 : 256];
+                        }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    S[0] += (long long)__float2int_rz(v[q][0]);
+                    S[1] += (long long)__float2int_rz(v[q][1]);
+                }
+            }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            H[k] = (long long)(((unsigned long long)H[k] << OZ_B) | (L[k] >> (64 - OZ_B)));
+            L[k] <<= OZ_B;
+            const unsigned long long l2 = L[k] + (unsigned long long)S[k];
+            H[k] += (S[k] >> 63) + (l2 < L[k] ? 1 : 0);
+            L[k] = l2;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int64_t p = P * 128 + r, q = Q * 128 + cb + 2 * k;
+        if (q >= n || (sym && p < q)) continue;
+        const int32_t a = ex[p], b = ey[q];
+        const double g = (a == OZ_NONFINITE || b == OZ_NONFINITE)
+                             ? __longlong_as_double(0x7ff8000000000000ll)
+                             : fixed128_to_double(H[k], L[k], a + b - 8 - OZ_B * (OZ_S - 1));
+        G[p + q * ldg] = g;
+        if (sym) G[q + p * ldg] = g;
+    }
+}
+
 struct OzPlan {
     int64_t np, nb, ldz, ntiles, kchunk;
     int chunks;
@@ -322,8 +394,9 @@ size_t oz_gemm_tn_ws_bytes(int64_t m, int64_t n) { return oz_plan(m, n, false).t
 // so that a wave of 152 CTAs spans about OZ_GX X tiles and 152 / OZ_GX Y
 // tiles and both are shared through L2 while the wave moves along K (with
 // the Y tiles outer over all X tiles a wave read ~152 distinct X tiles).  One
-// CTA: each group's tiles are counted by one thread, prefix summed in group
-// order, and each group's range is filled by its thread.
+// CTA: each group's tiles are counted by one warp (lanes over the Y tiles), prefix
+// summed in group order, and each group's range is filled by its warp, the Y
+// tiles in order (one thread per group took 0.6 ms for n = 2000).
 constexpr int OZ_GX = 16;
 
 __device__ __forceinline__ bool oz_tile_valid(int t, int64_t P, int u, int64_t Qp, int sym) {
@@ -331,19 +404,28 @@ __device__ __forceinline__ bool oz_tile_valid(int t, int64_t P, int u, int64_t Q
     return !(sym && t == u && P < 2 * Qp);  // P >= 2 Qp when t == u
 }
 
-__global__ void k_oz_tiles(int64_t nb, int64_t np, int sym, int2* __restrict__ tiles, int32_t* __restrict__ map) {
+// Valid X tiles of group g with Y tile yj.
+__device__ __forceinline__ int oz_group_count(int64_t g, int64_t yj, int64_t nb, int64_t nq, int64_t nx, int sym) {
+    const int64_t x1 = min(nx, (g + 1) * OZ_GX);
+    int c = 0;
+    for (int64_t xi = g * OZ_GX; xi < x1; ++xi)
+        c += oz_tile_valid((int)(xi / nb), xi % nb, (int)(yj / nq), yj % nq, sym) ? 1 : 0;
+    return c;
+}
+
+__global__ void __launch_bounds__(1024) k_oz_tiles(int64_t nb, int64_t np, int sym, int2* __restrict__ tiles,
+                                                   int32_t* __restrict__ map) {
     extern __shared__ int32_t oz_cnt[];  // groups + 1
     const int64_t nq = (nb + 1) / 2;
     const int64_t nx = (int64_t)OZ_S * nb, ny = (int64_t)OZ_S * nq;
     const int64_t groups = (nx + OZ_GX - 1) / OZ_GX;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int64_t q = threadIdx.x; q < (int64_t)OZ_S * OZ_S * nb * nb; q += blockDim.x) map[q] = -1;
-    for (int64_t g = threadIdx.x; g < groups; g += blockDim.x) {
-        int32_t c = 0;
-        const int64_t x1 = min(nx, (g + 1) * OZ_GX);
-        for (int64_t yj = 0; yj < ny; ++yj)
-            for (int64_t xi = g * OZ_GX; xi < x1; ++xi)
-                c += oz_tile_valid((int)(xi / nb), xi % nb, (int)(yj / nq), yj % nq, sym) ? 1 : 0;
-        oz_cnt[g + 1] = c;
+    for (int64_t g = warp; g < groups; g += nw) {
+        int c = 0;
+        for (int64_t yj = lane; yj < ny; yj += 32) c += oz_group_count(g, yj, nb, nq, nx, sym);
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) oz_cnt[g + 1] = c;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -351,10 +433,20 @@ __global__ void k_oz_tiles(int64_t nb, int64_t np, int sym, int2* __restrict__ t
         for (int64_t g = 0; g < groups; ++g) oz_cnt[g + 1] += oz_cnt[g];
     }
     __syncthreads();
-    for (int64_t g = threadIdx.x; g < groups; g += blockDim.x) {
-        int32_t k = oz_cnt[g];
+    for (int64_t g = warp; g < groups; g += nw) {
+        int32_t k0 = oz_cnt[g];
         const int64_t x1 = min(nx, (g + 1) * OZ_GX);
-        for (int64_t yj = 0; yj < ny; ++yj) {
+        for (int64_t y0 = 0; y0 < ny; y0 += 32) {
+            const int64_t yj = y0 + lane;
+            const int c = yj < ny ? oz_group_count(g, yj, nb, nq, nx, sym) : 0;
+            int incl = c;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += o;
+            }
+            int32_t k = k0 + incl - c;
+            k0 += __shfl_sync(0xffffffffu, incl, 31);
+            if (yj >= ny) continue;
             const int u = (int)(yj / nq);
             const int64_t Qp = yj % nq;
             for (int64_t xi = g * OZ_GX; xi < x1; ++xi) {
@@ -391,7 +483,7 @@ static lsq_status oz_run(const double* X, int64_t ldx, const double* Y, int64_t 
     int32_t* ey = sym ? ex : (int32_t*)((char*)ex + eb);
     const size_t tsm = sizeof(int32_t) * (size_t)(ceil_div((int64_t)OZ_S * P.nb, OZ_GX) + 1);
     if (tsm > 48 * 1024) return LSQ_ERR_ARG;
-    k_oz_tiles<<<1, 256, tsm, st>>>(P.nb, P.np, sym ? 1 : 0, tiles, map);
+    k_oz_tiles<<<1, 1024, tsm, st>>>(P.nb, P.np, sym ? 1 : 0, tiles, map);
     LSQ_LAUNCH_CHECK();
     dim3 gs((unsigned)std::min<int64_t>(ceil_div(P.ldz, 256 * 4), 64), (unsigned)P.np);
     k_oz_colexp<<<(unsigned)n, 256, 0, st>>>(X, m, ldx, ex);
@@ -407,7 +499,13 @@ static lsq_status oz_run(const double* X, int64_t ldx, const double* Y, int64_t 
     lsq_status r = launch_tc_tiles_fp8(Zx, P.ldz, OZ_S * P.np, Zy, P.ldz, OZ_S * P.np, P.ldz, P.kchunk, tiles,
                                        P.ntiles / 2, T, err, st);
     if (r != LSQ_OK) return r;
-    const int64_t cblocks = (sym ? P.nb * (P.nb + 1) / 2 : P.nb * P.nb) * 4;
+    const int64_t blocks = sym ? P.nb * (P.nb + 1) / 2 : P.nb * P.nb, cblocks = 4 * blocks;
+    if (cblocks < device_sm_count()) {  // fewer than one CTA an SM at 32 columns each
+        k_oz_combine_few<<<(unsigned)(32 * blocks), OZ_CB_THREADS, 0, st>>>(T, map, P.ntiles, P.chunks, n, P.nb, ex, ey,
+                                                                           sym ? 1 : 0, G, ldg);
+        LSQ_LAUNCH_CHECK();
+        return LSQ_OK;
+    }
     k_oz_combine<<<(unsigned)cblocks, OZ_CB_THREADS, 0, st>>>(
         T, map, P.ntiles, P.chunks, n, P.nb, ex, ey, sym ? 1 : 0, G, ldg);
     LSQ_LAUNCH_CHECK();
