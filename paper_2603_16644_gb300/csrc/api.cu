@@ -341,7 +341,8 @@ SolveLayout solve_layout(int64_t m, int64_t n, const lsq_opts* o, int prec, int 
     L.err = q.take(sizeof(int32_t));
     L.tsync = q.take(sizeof(int32_t) * trsv_sync_ints(n));
     // shared by the tensor-core A_p (first) and the tensor-core Gram of PNE
-    L.oz_bytes = std::max(ot_trsm_ws_bytes(m, n), hpne ? oz_gemm_tn_ws_bytes(m, n) : oz_gram_ws_bytes(m, n));
+    L.oz_bytes = std::max({ot_trsm_ws_bytes(m, n), hpne ? oz_gemm_tn_ws_bytes(m, n) : oz_gram_ws_bytes(m, n),
+                           cholesky_ws_bytes(n)});
     L.oz = q.take(L.oz_bytes);
     L.est = o->sketch_prec == LSQ_AUTO_SKETCH ? q.take(est_layout(m, n, sms).total) : 0;
     if (method == M_HPNE_QR) {

@@ -152,7 +152,11 @@ size_t ot_update_ws_bytes(int64_t M, int64_t N, int64_t K);
 lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t sk, int64_t sj, const double* Cin,
                           int64_t ldi, double* Cout, int64_t ldo, int64_t M, int64_t N, int64_t K, void* ws,
                           size_t ws_bytes, int32_t* err, cudaStream_t st, int xmode = 0,
-                          const int32_t* Eblk = nullptr, int64_t b0 = 0, int nbk = 0, int x_digits = 8);
+                          const int32_t* Eblk = nullptr, int64_t b0 = 0, int nbk = 0, int x_digits = 8,
+                          bool lower = false);
+// C -= X X^T (X: M x K), at least the lower triangle of C.
+lsq_status ot_gemm_update_lower(const double* X, int64_t ld, double* C, int64_t ldc, int64_t M, int64_t K, void* ws,
+                                size_t ws_bytes, int32_t* err, cudaStream_t st);
 // out (M x (N0 + N1), ld M) = -X [Y0 Y1], K of any length, M small (see
 // oz_trsm.cu); part and ws: the bytes of the two functions with N = N0 + N1.
 size_t ot_gemm_long_ws_bytes(int64_t M, int64_t N, int64_t K);

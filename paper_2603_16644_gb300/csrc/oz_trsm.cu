@@ -386,8 +386,25 @@ constexpr int OT_EPI_WARPS = 16;
 // the column tiles fastest: a CTA then stays on one column tile, and the
 // banded order raised their traffic by 30 % at the same time.
 constexpr int OT_GM = 8;
+//
+// ntj = 0: the tiles of a square product that reach its lower triangle (a tile
+// is twice as high as wide: row of tiles ti has 2 ti + 2 of them).
+__device__ __forceinline__ void ot_lower_tile(int t, int& ti, int& tj) {
+    ti = (int)((sqrtf(4.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while ((ti + 1) * (ti + 2) <= t) ++ti;
+    while (ti * (ti + 1) > t) --ti;
+    tj = t - ti * (ti + 1);
+}
+
 template <bool GROUPED>
 __device__ __forceinline__ void ot_tile_coords(int t, int ntj, int nti, int64_t& i0, int64_t& j0) {
+    if (!GROUPED && ntj == 0) {
+        int ti, tj;
+        ot_lower_tile(t, ti, tj);
+        i0 = (int64_t)ti * OT_BM;
+        j0 = (int64_t)tj * OT_BN;
+        return;
+    }
     if (!GROUPED) {
         i0 = (int64_t)(t / ntj) * OT_BM;
         j0 = (int64_t)(t % ntj) * OT_BN;
@@ -462,7 +479,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
         auto slab_tile = [&](int g, int64_t& i0, int64_t& j0, int& kx) {
             const int tl = (int)blockIdx.x + (g / nslab) * (int)gridDim.x;
             kx = (int)(tl / zt * kc) + g % nslab * OT_BK;  // zt: tiles of a chunk
-            ot_tile_coords<XD == 3>(tl % zt, ntj, zt / ntj, i0, j0);
+            ot_tile_coords<XD == 3>(tl % zt, ntj, ntj ? zt / ntj : 0, i0, j0);
         };
         auto load_y = [&](int g) -> bool {
             int64_t i0, j0;
@@ -643,7 +660,7 @@ __global__ void __launch_bounds__(OT_THREADS, 1)
         for (int i = 0; i < ntl; ++i) {
             const int tile = (int)blockIdx.x + i * (int)gridDim.x;
             int64_t i0, j0;
-            ot_tile_coords<XD == 3>(tile % zt, ntj, zt / ntj, i0, j0);
+            ot_tile_coords<XD == 3>(tile % zt, ntj, ntj ? zt / ntj : 0, i0, j0);
             const int64_t row = i0 + quad * 32 + lane;
             const bool narrow = N - j0 <= 32;
             const int64_t c0 = j0 + cq * (narrow ? 8 : 16);
@@ -731,6 +748,13 @@ __host__ __device__ constexpr int o2_stages(int XD, int p) { return 2 * p + 1 < 
 template <bool GROUPED>
 __device__ __forceinline__ void o2_tile_coords(int t, int ntj, int nti, int64_t& i0, int64_t& j0) {
     constexpr int GM = OT_GM * OT_BM / O2_BM;
+    if (!GROUPED && ntj == 0) {
+        int ti, tj;
+        ot_lower_tile(t, ti, tj);
+        i0 = (int64_t)ti * O2_BM;
+        j0 = (int64_t)tj * O2_BN;
+        return;
+    }
     if (!GROUPED) {
         i0 = (int64_t)(t / ntj) * O2_BM;
         j0 = (int64_t)(t % ntj) * O2_BN;
@@ -766,7 +790,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(O2_THREADS, 1)
     const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
     const int nslab = (int)((K + OT_BK - 1) / OT_BK);
     const int ntl = ntiles > pair ? (ntiles - pair + npairs - 1) / npairs : 0;
-    const int nti = ntiles / ntj;
+    const int nti = ntj ? ntiles / ntj : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < O2_ST; ++s) {
@@ -1181,10 +1205,11 @@ static bool o2_faster(int ntiles, int ntiles2, int64_t K, int sms) {
 // at Y[k sk + j sj]) with FP64 accuracy on the tensor cores; K <= 512.
 // C_in may equal C_out (same ld).  xmode: 0 slice X here; 1 slice X with the
 // row exponents from the per-block exponents Eblk (blocks b0 .. b0+nbk-1).
+// lower (M = N): only the tiles that reach the lower triangle.
 lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t sk, int64_t sj, const double* Cin,
                           int64_t ldi, double* Cout, int64_t ldo, int64_t M, int64_t N, int64_t K, void* ws,
                           size_t ws_bytes, int32_t* err, cudaStream_t st, int xmode, const int32_t* Eblk, int64_t b0,
-                          int nbk, int x_digits) {
+                          int nbk, int x_digits, bool lower) {
     if (M <= 0 || N <= 0 || K <= 0) return LSQ_OK;
     // exact group sums: at most 8 pairs of digits (|d_t d_u| <= 2^12) per
     // group over K <= 512, or 3 pairs over K <= OT_KMAX3 with three X digits
@@ -1238,8 +1263,14 @@ lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t
     if (!ot_map(&tx, U.Zx, U.Kp, U.mp, OT_BM) || !ot_map(&ty, U.Zy, U.Kp, U.Np, OT_BN)) return LSQ_ERR_CUDA;
     const int stage = x_digits == 3 ? ST_K_UPDATE3 : ST_K_UPDATE;
     const int sms = device_sm_count();
-    const int ntj = (int)(U.Np / OT_BN), ntiles = (int)(ntj * (U.mp / OT_BM));
-    const int ntj2 = (int)ceil_div(U.Np, O2_BN), ntiles2 = (int)(ntj2 * ceil_div(U.mp, O2_BM));
+    int ntj = (int)(U.Np / OT_BN), ntiles = (int)(ntj * (U.mp / OT_BM));
+    int ntj2 = (int)ceil_div(U.Np, O2_BN), ntiles2 = (int)(ntj2 * ceil_div(U.mp, O2_BM));
+    if (lower) {
+        const int r1 = (int)(U.mp / OT_BM), r2 = (int)ceil_div(U.mp, O2_BM);
+        ntj = ntj2 = 0;
+        ntiles = r1 * (r1 + 1);
+        ntiles2 = r2 * (r2 + 1);
+    }
     if (o2_faster(ntiles, ntiles2, K, sms)) {
         const size_t smem = 1024 + (size_t)O2_ST * O2_STAGE + 512;
         auto kern = x_digits == 3 ? k_ot_update2<3> : k_ot_update2<OT_DIG>;
@@ -1339,6 +1370,13 @@ lsq_status ot_gemm_long(const double* X, int64_t ldx, const double* Y0, int64_t 
         LSQ_LAUNCH_CHECK();
     }
     return LSQ_OK;
+}
+
+// C -= X X^T (C: M x M, X: M x K, both ld), the tiles that reach the lower triangle.
+lsq_status ot_gemm_update_lower(const double* X, int64_t ld, double* C, int64_t ldc, int64_t M, int64_t K, void* ws,
+                                size_t ws_bytes, int32_t* err, cudaStream_t st) {
+    return ot_gemm_update(X, ld, X, ld, 1, C, ldc, C, ldc, M, M, K, ws, ws_bytes, err, st, 0, nullptr, 0, 0, OT_DIG,
+                          true);
 }
 
 static void ot_max_update(int64_t m, int64_t c0, int64_t c1, size_t& need) {

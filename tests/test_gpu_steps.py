@@ -237,6 +237,28 @@ def test_cholesky_solve(n):
     assert np.linalg.norm(to_np(x) - y_o) / np.linalg.norm(y_o) <= 8 * n * U64 * kG * O.kappa(R)
 
 
+@pytest.mark.parametrize("n", [255, 256, 257, 320, 321, 577, 2100])
+def test_cholesky_blocks(n):
+    """Sizes around the 256-column blocks (inner updates of up to 192 columns,
+    one product for the rest), against the oracle within the bound of
+    test_cholesky_solve; the upper triangle is cleared, and a matrix that is
+    not positive definite reports the pivot at which the oracle stops."""
+    rng = np.random.default_rng(40 + n)
+    X = rng.standard_normal((2 * n + 5, n))
+    G = X.T @ X
+    c = rng.standard_normal(n)
+    L_o, info_o = O.cholesky(G)
+    x, F, _, info = lsq.factor_solve(dev_colmajor(G), torch.from_numpy(c).cuda())
+    F = to_np(F)
+    assert int(to_np(info)[0]) == 0 == info_o and np.all(np.triu(F, 1) == 0)
+    assert np.linalg.norm(F - L_o) / np.linalg.norm(L_o) <= 8 * n * U64 * O.kappa(G)
+    k = n - 3
+    G[k, k] = -1.0
+    _, info_o = O.cholesky(G)
+    _, _, _, info = lsq.factor_solve(dev_colmajor(G), torch.from_numpy(c).cuda())
+    assert int(to_np(info)[0]) == info_o == k + 1
+
+
 @pytest.mark.parametrize("n", [1, 5, 33, 64, 200, 1024])
 def test_lu_solve(n):
     rng = np.random.default_rng(100 + n)
