@@ -148,6 +148,14 @@ constexpr int64_t kSketchChunk = 960;  // K chunk of the FP64 sketch (three-digi
 // The Gaussian sketch on the tensor cores: FP64 by digit slicing (switch
 // lsq_set_fp64_emulation), FP32 as BF16 pieces (lsq_set_tensor_core_sketch).
 bool gauss_fp64_tc(int prec) { return prec == LSQ_FP64 && g_fp64_emulation && ot_trsm_supported(); }
+// FP32 Gaussian sketches of at least this many rows take two FP16 pieces per
+// value (three products), shorter ones three BF16 pieces (six).  Relative error
+// of the sketch against 64 bits, FP16 / BF16 pieces: m = 1000 3.5e-7 / 2.3e-7,
+// 4000 4.2e-7 / 3.5e-7, 20000 2.8e-6 / 4.8e-6, 262144 1.5e-5 / 2.8e-5: the FP16
+// pieces represent a value a little less closely, and the accumulation of half
+// as many products is more accurate from about 10000 rows on.
+constexpr int64_t kFp16PieceRows = 16384;
+bool gauss_fp32_f16(int64_t m) { return m >= kFp16PieceRows; }
 bool gauss_fp32_tc(int prec) { return prec == LSQ_FP32 && g_tensor_core_sketch && sketch_tc_supported(LSQ_BF16); }
 
 SketchLayout sketch_layout(int64_t m, int64_t n, int64_t s, int kind, int zeta, int prec, int sms) {
@@ -176,12 +184,14 @@ SketchLayout sketch_layout(int64_t m, int64_t n, int64_t s, int kind, int zeta, 
         // of tensor-core products accumulated into A_s (A is read in place)
         L.gemm = o.take(ot_update_ws_bytes(s, n, kSketchChunk));
     } else if (gauss_fp32_tc(prec)) {
-        // FP32: three BF16 pieces per value, six K segments of length ldq (a
-        // multiple of 64: the operands are K-blocked in slices of 64)
+        // FP32: three BF16 pieces per value in six K segments of length ldq (a
+        // multiple of 64: the operands are K-blocked in slices of 64), or two
+        // FP16 pieces in two
         L.ldq = L.ldo = align_up((size_t)m, 64);
-        L.ahat = o.take(sizeof(uint16_t) * 6 * (size_t)L.ldq * n);
-        L.om = o.take(sizeof(uint16_t) * 6 * (size_t)L.ldo * s);
-        L.gemm = o.take(sketch_tc_ws_bytes(s, n, 6 * L.ldq, LSQ_BF16, sms));
+        const bool f16 = gauss_fp32_f16(m);
+        L.ahat = o.take(sizeof(uint16_t) * (f16 ? 2 : 6) * (size_t)L.ldq * n);
+        L.om = o.take(sizeof(uint16_t) * (f16 ? 2 : 6) * (size_t)L.ldo * s);
+        L.gemm = o.take(sketch_tc_ws_bytes(s, n, (f16 ? 3 : 6) * L.ldq, f16 ? LSQ_FP16 : LSQ_BF16, sms, f16));
     } else {
         L.ahat = o.take((size_t)L.ldq * n * es);
         L.om = o.take((size_t)L.ldo * s * es);
@@ -401,7 +411,15 @@ lsq_status run_sketch(const double* A, int64_t m, int64_t n, int64_t lda, const 
         return LSQ_OK;
     }
     if (gauss_fp32_tc(prec)) {
-        const int64_t K6 = 6 * L.ldq;
+        const int64_t K2 = 2 * L.ldq, K3 = 3 * L.ldq, K6 = 6 * L.ldq;
+        if (gauss_fp32_f16(m)) {
+            if ((r = launch_gauss_split2(o->seed, o->s, m, L.ldq, (uint16_t*)(base + L.om), o->row_offset, st)) != LSQ_OK)
+                return r;
+            if ((r = launch_quantize_split2(A, m, n, lda, colexp, L.ldq, (uint16_t*)(base + L.ahat), st)) != LSQ_OK)
+                return r;
+            return launch_sketch_tc(base + L.om, K2, base + L.ahat, K2, LSQ_FP16, o->s, n, K3, (float*)As, ldas,
+                                    base + L.gemm, L.gemm_bytes, err, st, true, L.ldq, 0x1p-15f);
+        }
         if ((r = launch_gauss_split3(o->seed, o->s, m, L.ldq, (uint16_t*)(base + L.om), o->row_offset, st)) != LSQ_OK)
             return r;
         if ((r = launch_quantize_split3(A, m, n, lda, colexp, L.ldq, (uint16_t*)(base + L.ahat), st)) != LSQ_OK)

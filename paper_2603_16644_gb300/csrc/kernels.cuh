@@ -46,6 +46,12 @@ lsq_status launch_gauss_split3(uint64_t seed, int64_t s, int64_t m, int64_t L, u
                                cudaStream_t st);
 lsq_status launch_quantize_split3(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp,
                                   int64_t L, uint16_t* Y, cudaStream_t st);
+// The same as one FP16 GEMM of two FP16 pieces per value: segments m h and h m
+// of length L, K-blocked; launch_sketch_tc with seg = L and oscale = 2^-15.
+lsq_status launch_gauss_split2(uint64_t seed, int64_t s, int64_t m, int64_t L, uint16_t* X, int64_t j0,
+                               cudaStream_t st);
+lsq_status launch_quantize_split2(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp,
+                                  int64_t L, uint16_t* Y, cudaStream_t st);
 // FP32 Gram X^T X (X: m x n, FP64 or FP32, rounded to FP32) as one BF16 GEMM:
 // seven K segments per column (h l h m m h h); X at Z, Y at Z + L, ld 7L, K 6L.
 template <typename TI>
@@ -119,10 +125,10 @@ lsq_status rank_update_ext(T* C, int64_t ldc, const T* P, int64_t psi, int64_t p
 
 // ---- sketch_tc.cu: tcgen05 Gaussian sketch for 8/16-bit u_p --------------
 bool sketch_tc_supported(int prec);
-size_t sketch_tc_ws_bytes(int64_t s, int64_t n, int64_t m, int prec, int sms);
+size_t sketch_tc_ws_bytes(int64_t s, int64_t n, int64_t m, int prec, int sms, bool pieces = false);
 lsq_status launch_sketch_tc(const void* Om, int64_t ldo, const void* Ahat, int64_t ldq, int prec, int64_t s,
                             int64_t n, int64_t m, float* As, int64_t ldas, void* ws, size_t ws_bytes, int32_t* err,
-                            cudaStream_t st, bool blocked = false);
+                            cudaStream_t st, bool blocked = false, int64_t seg = 0, float oscale = 1.0f);
 
 // ---- ozaki.cu: FP64 Gram on the FP8 tensor cores (digit slicing) ----------
 size_t oz_gram_ws_bytes(int64_t m, int64_t n);

@@ -1181,7 +1181,10 @@ lsq_status ot_gauss_digits(uint64_t seed, int64_t s, int64_t j0, int64_t kc, int
                            cudaStream_t st) {
     if (s <= 0 || kc <= 0 || kc > OT_KMAX3 || !ws || ws_bytes < ot_update_ws_bytes(s, N, kc)) return LSQ_ERR_ARG;
     const OtUpd U = ot_upd_ptrs(ws, s, N, kc);
-    const dim3 grid((unsigned)(U.Kp / 64), (unsigned)std::min<int64_t>(ceil_div(U.mp, 8), 256));
+    // about 6 CTAs an SM: every CTA stages the ziggurat's 14 KB of tables first,
+    // which cost more than its entries at two rows per warp
+    const int64_t gx = U.Kp / 64, gy = std::max<int64_t>(1, 6 * device_sm_count() / gx);
+    const dim3 grid((unsigned)gx, (unsigned)std::min<int64_t>(ceil_div(U.mp, 8), gy));
     k_ot_gauss_digits<<<grid, 256, 0, st>>>(zig_table(), seed, s, j0, kc, U.mp, U.Kp, U.Zx, U.Ex);
     LSQ_LAUNCH_CHECK();
     return LSQ_OK;

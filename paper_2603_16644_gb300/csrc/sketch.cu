@@ -496,6 +496,64 @@ __global__ void k_quantize_split3(const double* __restrict__ A, int64_t m, int64
     }
 }
 
+// The FP32 Gaussian sketch of many rows: every FP32 value as two FP16 pieces, h = fp16(x) and
+// m = fp16(x - h), and three piece products h h + h m + m h as one FP16 GEMM
+// over a K three times longer.  Omega's entries (multiples of 2^-17 below 8 in
+// magnitude) are exactly h + m; Ahat, scaled to [2^14, 2^15) below FP16's
+// largest value, is h + m to 2^-23 relative (2^-39 of the column's maximum where
+// m runs into FP16's smallest subnormal), and the dropped m m weighs 2^-24: the
+// FP32 accumulation over K is what bounds the error.  Against three BF16 pieces
+// and six products: half the tensor work and a third of Omega's bytes, and half
+// as many roundings in the accumulators (262144 x 4096 to 8192 rows: the solve
+// 427 -> 388 ms).
+//
+// The pieces are stored K-blocked like the BF16 ones, h and m as segments of
+// length L (a multiple of 64), Omega as m h and Ahat as h m; the GEMM takes the
+// segment pairs (m, h) (h, m) (h, h), the large products last.
+
+// Pieces of two consecutive values (the first in the low half).
+__device__ __forceinline__ void split2_f16(float x0, float x1, uint32_t& h, uint32_t& m) {
+    const __half h0 = __float2half_rn(x0), h1 = __float2half_rn(x1);
+    const __half m0 = __float2half_rn(__fsub_rn(x0, __half2float(h0)));
+    const __half m1 = __float2half_rn(__fsub_rn(x1, __half2float(h1)));
+    h = (uint32_t)__half_as_ushort(h0) | ((uint32_t)__half_as_ushort(h1) << 16);
+    m = (uint32_t)__half_as_ushort(m0) | ((uint32_t)__half_as_ushort(m1) << 16);
+}
+
+__global__ void k_gauss_split2(const ZigTable tab, uint64_t seed, int64_t s, int64_t m, int64_t L,
+                               uint16_t* __restrict__ X, int64_t j0) {
+    __shared__ ZigShared Z;
+    zig_stage(tab, Z);
+    for (int64_t i = blockIdx.y; i < s; i += gridDim.y) {
+        for (int64_t j = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); j < L;
+             j += 2 * (int64_t)gridDim.x * blockDim.x) {
+            uint32_t h, mi;
+            split2_f16(j < m ? gauss_f32(seed, i, j0 + j, Z) : 0.0f, j + 1 < m ? gauss_f32(seed, i, j0 + j + 1, Z) : 0.0f,
+                       h, mi);
+            *(uint32_t*)(X + kblk(j, i, s)) = mi;
+            *(uint32_t*)(X + kblk(L + j, i, s)) = h;
+        }
+    }
+}
+
+// Ahat = FP32(A 2^colexp), times 2^15 (taken out again by the GEMM's output scale).
+__global__ void k_quantize_split2(const double* __restrict__ A, int64_t m, int64_t n, int64_t lda,
+                                  const int32_t* __restrict__ colexp, int64_t L, uint16_t* __restrict__ Y) {
+    const int64_t c = blockIdx.y;
+    const int e = colexp[c];
+    for (int64_t j = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); j < L;
+         j += 2 * (int64_t)gridDim.x * blockDim.x) {
+        float x[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            x[q] = j + q < m ? __fmul_rn(__uint_as_float(quant_bits(A[j + q + c * lda], e, LSQ_FP32)), 32768.0f) : 0.0f;
+        uint32_t h, mi;
+        split2_f16(x[0], x[1], h, mi);
+        *(uint32_t*)(Y + kblk(j, c, n)) = h;
+        *(uint32_t*)(Y + kblk(L + j, c, n)) = mi;
+    }
+}
+
 // Gram X^T X of FP32-rounded columns on the BF16 tensor cores: the six
 // pairs of pieces (t, u), t + u <= 2, chained through ONE array of seven K
 // segments per column, h l h m m h h: the GEMM reads X at segment offset 0
@@ -841,6 +899,24 @@ lsq_status launch_quantize_split3(const double* A, int64_t m, int64_t n, int64_t
     if (L % 64) return LSQ_ERR_ARG;
     dim3 grid((unsigned)min64(ceil_div(L, 256), 64), (unsigned)n);
     k_quantize_split3<<<grid, 256, 0, st>>>(A, m, n, lda, colexp, L, Y);
+    LSQ_LAUNCH_CHECK();
+    return LSQ_OK;
+}
+
+lsq_status launch_gauss_split2(uint64_t seed, int64_t s, int64_t m, int64_t L, uint16_t* X, int64_t j0,
+                               cudaStream_t st) {
+    if (L % 64) return LSQ_ERR_ARG;
+    dim3 grid((unsigned)min64(ceil_div(L, 512), 64), (unsigned)min64(s, 64));
+    k_gauss_split2<<<grid, 256, 0, st>>>(zig_table(), seed, s, m, L, X, j0);
+    LSQ_LAUNCH_CHECK();
+    return LSQ_OK;
+}
+
+lsq_status launch_quantize_split2(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp,
+                                  int64_t L, uint16_t* Y, cudaStream_t st) {
+    if (L % 64) return LSQ_ERR_ARG;
+    dim3 grid((unsigned)min64(ceil_div(L, 512), 64), (unsigned)n);
+    k_quantize_split2<<<grid, 256, 0, st>>>(A, m, n, lda, colexp, L, Y);
     LSQ_LAUNCH_CHECK();
     return LSQ_OK;
 }

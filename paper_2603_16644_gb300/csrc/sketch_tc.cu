@@ -46,7 +46,8 @@ template <int KIND, int BN>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_sketch_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t M, int64_t N,
                 int64_t K, int64_t kchunk, float* __restrict__ out, int64_t ldo, int64_t split_stride,
-                int32_t* __restrict__ err, const int2* __restrict__ tiles, int64_t ntiles, int blocked) {
+                int32_t* __restrict__ err, const int2* __restrict__ tiles, int64_t ntiles, int blocked, int seg,
+                float oscale) {
     constexpr int ES = KIND == 2 ? 1 : 2;  // element bytes
     constexpr int BKE = 128 / ES;          // K elements per stage
     constexpr int ST = tc_stages(BN);
@@ -109,9 +110,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             mbar_expect_tx(&full[s], TC_TILE_BYTES + BBYTES);
             int x = (int)(kb0 + (int64_t)kb * BKE);
             if (blocked) {
-                // K-blocked operands: block x / BKE holds every row's 128 bytes
-                tma_load_3d(sA + s * TC_TILE_BYTES, &tmA, &full[s], 0, (int)m0, x / BKE);
-                tma_load_3d(sB + s * BBYTES, &tmB, &full[s], 0, (int)n0, x / BKE);
+                // K-blocked operands: block z holds every row's 128 bytes.  seg:
+                // two piece segments of seg blocks each, K running over the
+                // segment pairs (0, 0) (1, 1) (1, 0)
+                const int z = x / BKE, q = seg ? z / seg : 0;
+                tma_load_3d(sA + s * TC_TILE_BYTES, &tmA, &full[s], 0, (int)m0, q == 2 ? z - seg : z);
+                tma_load_3d(sB + s * BBYTES, &tmB, &full[s], 0, (int)n0, q == 2 ? z - 2 * seg : z);
             } else {
                 tma_load_2d(sA + s * TC_TILE_BYTES, &tmA, &full[s], x, (int)m0);
                 tma_load_2d(sB + s * BBYTES, &tmB, &full[s], x, (int)n0);
@@ -168,7 +172,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         int64_t col = n0 + c0 + j;
-                        if (col < N) o[row + col * ldo] = __uint_as_float(v[j]);
+                        if (col < N) o[row + col * ldo] = __uint_as_float(v[j]) * oscale;
                     }
                 }
             }
@@ -275,38 +279,45 @@ static int tc_bn(int64_t N) { return N >= 256 ? 256 : TC_BN; }
 // (1.8 PFLOP/s of tensor work).  Shorter accumulation chains in the FP32
 // accumulators are also more accurate.
 constexpr int64_t TC_KBLOCKS_MAX = 512;
+// The FP16 pieces of an FP32 sketch: a quarter of that, so that the chain of the
+// full-size products is at most half the 16384 rows from which they are used (error of a
+// 16384 x 1000 sketch 1.93e-5 with 512, 1.86e-5 with the BF16 pieces).
+constexpr int64_t TC_KBLOCKS_PIECES = 128;
 
 // Split count: fill the SMs when the tile grid is small, and at most
 // TC_KBLOCKS_MAX K blocks per split; at least 4 stages of K per split.
-static int tc_splits(int64_t M, int64_t N, int64_t K, int prec, int sms) {
+static int tc_splits(int64_t M, int64_t N, int64_t K, int prec, int sms, int64_t kblocks_max = TC_KBLOCKS_MAX) {
     int64_t tiles = ceil_div(M, TC_BM) * ceil_div(N, tc_bn(N));
     int64_t bke = prec == LSQ_FP8_E4M3 ? 128 : 64;
     int64_t kblocks = ceil_div(K, bke);
     int64_t want = std::max<int64_t>(1, sms / std::max<int64_t>(1, tiles));
-    want = std::max<int64_t>(want, ceil_div(kblocks, TC_KBLOCKS_MAX));
+    want = std::max<int64_t>(want, ceil_div(kblocks, kblocks_max));
     int64_t cap = std::max<int64_t>(1, kblocks / 4);
     return (int)std::min<int64_t>(std::min<int64_t>(want, cap), 64);
 }
 
-size_t sketch_tc_ws_bytes(int64_t s, int64_t n, int64_t m, int prec, int sms) {
-    int sp = tc_splits(s, n, m, prec, sms);
+size_t sketch_tc_ws_bytes(int64_t s, int64_t n, int64_t m, int prec, int sms, bool pieces) {
+    int sp = tc_splits(s, n, m, prec, sms, pieces ? TC_KBLOCKS_PIECES : TC_KBLOCKS_MAX);
     return sp > 1 ? align_up(sizeof(float) * (size_t)sp * s * n, 256) : 0;
 }
 
 lsq_status launch_sketch_tc(const void* Om, int64_t ldo, const void* Ahat, int64_t ldq, int prec, int64_t s,
                             int64_t n, int64_t m, float* As, int64_t ldas, void* ws, size_t ws_bytes, int32_t* err,
-                            cudaStream_t st, bool blocked) {
+                            cudaStream_t st, bool blocked, int64_t seg, float oscale) {
     if (!sketch_tc_supported(prec)) return LSQ_ERR_ARG;
     if ((ldo % 16) || (ldq % 16) || ((uintptr_t)Om % 16) || ((uintptr_t)Ahat % 16)) return LSQ_ERR_ARG;
     const int bn = tc_bn(n);
     CUtensorMap ta, tb;
     if (blocked) {
-        if (!make_map_blocked(&ta, Om, prec, m, s) || !make_map_blocked(&tb, Ahat, prec, m, n, bn)) return LSQ_ERR_ARG;
+        // seg: two stored segments, K = m = 3 seg
+        if (seg && (seg % 64 || m != 3 * seg)) return LSQ_ERR_ARG;
+        const int64_t ks = seg ? 2 * seg : m;
+        if (!make_map_blocked(&ta, Om, prec, ks, s) || !make_map_blocked(&tb, Ahat, prec, ks, n, bn)) return LSQ_ERR_ARG;
     } else if (!make_map(&ta, Om, prec, m, s, ldo) || !make_map(&tb, Ahat, prec, m, n, ldq, bn)) {
         return LSQ_ERR_CUDA;
     }
     int sms = device_sm_count();
-    int splits = tc_splits(s, n, m, prec, sms);
+    int splits = tc_splits(s, n, m, prec, sms, seg ? TC_KBLOCKS_PIECES : TC_KBLOCKS_MAX);
     int64_t bke = prec == LSQ_FP8_E4M3 ? 128 : 64;
     int64_t kchunk = ceil_div(ceil_div(m, splits), bke) * bke;
     splits = (int)ceil_div(m, kchunk);
@@ -324,7 +335,7 @@ lsq_status launch_sketch_tc(const void* Om, int64_t ldo, const void* Ahat, int64
     auto go = [&](auto kern) -> lsq_status {
         LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<grid, TC_THREADS, smem, st>>>(ta, tb, s, n, m, kchunk, out, ldout, stride, err, nullptr, 0,
-                                             blocked ? 1 : 0);
+                                             blocked ? 1 : 0, (int)(seg / 64), oscale);
         return LSQ_OK;
     };
     lsq_status lr;
@@ -364,7 +375,7 @@ lsq_status launch_tc_tiles_fp8(const void* X, int64_t ldx, int64_t rowsX, const 
     LSQ_CUDA_TRY(cudaFuncSetAttribute(k_sketch_tc<2, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dim3 grid((unsigned)ntiles, 1, (unsigned)chunks);
     k_sketch_tc<2, BN><<<grid, TC_THREADS, smem, st>>>(ta, tb, rowsX, rowsY, K, kchunk, out, TC_BM, 0, err, tiles,
-                                                      ntiles, 0);
+                                                      ntiles, 0, 0, 1.0f);
     LSQ_LAUNCH_CHECK();
     return LSQ_OK;
 }

@@ -162,6 +162,25 @@ def test_fp32_gaussian_sketch_bf16_pieces(m, n, s):
     assert e_tc <= 2 * max(e_or, e_cc), (e_tc, e_or, e_cc)
 
 
+@pytest.mark.parametrize("m,n,s", [(16383, 40, 130), (16384, 129, 130), (16385, 33, 140), (33000, 20, 60)])
+def test_fp32_gaussian_sketch_fp16_pieces(m, n, s):
+    # from 16384 rows on the FP32 sketch is three FP16 piece products: the
+    # bounds of test_fp32_gaussian_sketch_bf16_pieces on both sides of the line
+    # and with a remainder of K, entries spread over 40 bits within a column
+    rng = np.random.default_rng(m + 7 * n)
+    A = np.asfortranarray(rng.standard_normal((m, n)) * np.exp2(rng.integers(-40, 1, (m, n))))
+    As_tc, As_cc, ce = _sketch_both_ways(A, lsq.FP32, s, 23, False)
+    oAs, oce = O.sketch(A, O.GAUSSIAN, s, 0, 23, O.FP32)
+    np.testing.assert_array_equal(ce, oce)
+    Om = O.gaussian_operator(23, s, m, O.FP32)
+    Ah = O.quantize(A, O.FP32, oce)
+    exact = Om @ Ah
+    scale = np.abs(Om) @ np.abs(Ah)
+    assert np.all(np.abs(As_tc - oAs) <= 3 * m * U32 * scale)
+    e_tc = np.linalg.norm(As_tc - exact)
+    assert e_tc <= 2 * max(np.linalg.norm(oAs - exact), np.linalg.norm(As_cc - exact))
+
+
 @pytest.mark.parametrize("m,n,s", [(1037, 113, 250), (3001, 70, 200), (700, 129, 130)])
 def test_fp64_gaussian_sketch_digit_sliced(m, n, s):
     # FP64 sketch as K chunks of 1024 FP64-accurate digit-sliced products:
