@@ -592,82 +592,132 @@ __device__ __forceinline__ uint32_t u4_word(const U4& w, int k) {
     return k == 0 ? w.x : k == 1 ? w.y : k == 2 ? w.z : w.w;
 }
 
-template <typename T>
-__global__ void k_srft_load(const double* __restrict__ A, int64_t m, int64_t n, int64_t lda,
-                            const int32_t* __restrict__ colexp, int prec, uint64_t seed, int64_t mp, int64_t cpb,
-                            T* __restrict__ W) {
-    const int64_t c0 = (int64_t)blockIdx.y * cpb, c1 = min64(n, c0 + cpb);
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < mp; j += (int64_t)gridDim.x * blockDim.x) {
-        bool neg = false;
-        if (j < m) {
-            const U4 w = philox(U4{(uint32_t)((uint64_t)j >> 7), 0u, 0u, 3u}, (uint32_t)seed, (uint32_t)(seed >> 32));
-            neg = (u4_word(w, (int)((j >> 5) & 3)) >> (j & 31)) & 1u;
+// Order of a block of the first kernel, rows of one column held in one CTA.
+constexpr int FW_B = 4096;
+
+// A[j, c] rounded to the sketch precision (with the column scaling), exact in FP32
+template <int PREC>
+__device__ __forceinline__ float quant_f32(double a, int e) {
+    const uint32_t q = quant_bits(a, e, PREC);
+    if constexpr (PREC == LSQ_FP8_E4M3) return __half2float(__half(__nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)q, __NV_E4M3)));
+    else if constexpr (PREC == LSQ_FP16) return __half2float(__ushort_as_half((unsigned short)q));
+    else if constexpr (PREC == LSQ_BF16) return __uint_as_float(q << 16);
+    else return __uint_as_float(q);
+}
+
+// Rounding, signs, padding and the levels h = 1 .. B/2 for B = min(m', 4096)
+// consecutive rows of a column: one read of A and one write of W.  HBM bound
+// (8 bytes read and 4 written per element).  A thread holds 16 entries, all 16
+// loads in flight; index bits 0-4 are the lane (levels by shuffles), 5-8 the
+// register, 9-11 the warp (levels in registers after one exchange through
+// shared memory).  A separate load that rounded one entry at a time with a
+// run-time precision, and a transform with a pass over shared memory and two
+// barriers per level, took 525 + 377 us for 100000 x 400 to FP32; this 120 us.
+template <typename T, int PREC>
+__global__ void __launch_bounds__(256) k_srft_block(const double* __restrict__ A, int64_t m, int64_t lda,
+                                                    const int32_t* __restrict__ colexp, uint64_t seed, int64_t mp,
+                                                    T* __restrict__ W) {
+    __shared__ T x[FW_B];
+    const int B = (int)min64(mp, FW_B);
+    const int64_t c = blockIdx.y, b0 = (int64_t)blockIdx.x * B;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int i0 = 512 * warp + lane;  // entry of register k: i0 + 32 k
+    const double* col = A + c * lda;
+    double a[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const int i = i0 + 32 * k;
+        a[k] = i < B && b0 + i < m ? col[b0 + i] : 0.0;
+    }
+    // the sign words of the warp's 512 rows: four Philox counters, word k is
+    // component k & 3 of counter k >> 2, held by lane k >> 2
+    const U4 pw = philox(U4{(uint32_t)((uint64_t)(b0 + 512 * warp) >> 7) + (lane & 3), 0u, 0u, 3u}, (uint32_t)seed,
+                         (uint32_t)(seed >> 32));
+    const int e = PREC == LSQ_FP64 ? 0 : colexp[c];
+    T v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const uint32_t w = __shfl_sync(0xffffffffu, u4_word(pw, k & 3), k >> 2);
+        if constexpr (PREC == LSQ_FP64) v[k] = a[k];
+        else v[k] = quant_f32<PREC>(a[k], e);
+        // the padding stays +0
+        if (((w >> lane) & 1u) && b0 + i0 + 32 * k < m) v[k] = -v[k];
+    }
+#pragma unroll
+    for (int h = 1; h < 32; h <<= 1) {
+        if (h >= B) break;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const T o = __shfl_xor_sync(0xffffffffu, v[k], h);
+            v[k] = (lane & h) ? o - v[k] : v[k] + o;
         }
-        for (int64_t c = c0; c < c1; ++c) {
-            T v = (T)0;
-            if (j < m) {
-                if (prec == LSQ_FP64) {
-                    v = (T)A[j + c * lda];
-                } else {
-                    // the value rounded to u_p (with the column scaling) is exact in FP32
-                    double q = round_to_prec(ldexp(A[j + c * lda], colexp[c]), prec);
-                    v = (T)q;
-                }
-                if (neg) v = -v;
+    }
+#pragma unroll
+    for (int h = 1; h < 16; h <<= 1) {
+        if (32 * h >= B) break;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (!(k & h)) {
+                const T p = v[k], q = v[k + h];
+                v[k] = p + q;
+                v[k + h] = p - q;
             }
-            W[(size_t)c * mp + j] = v;
+    }
+    T* out = W + (size_t)c * mp + b0;
+    if (B <= 512) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (i0 + 32 * k < B) out[i0 + 32 * k] = v[k];
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[i0 + 32 * k] = v[k];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int l = t + 256 * r;
+        T u[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) u[k] = x[l + 512 * k];
+#pragma unroll
+        for (int h = 1; h < 8; h <<= 1) {
+            if (512 * h >= B) break;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (!(k & h)) {
+                    const T p = u[k], q = u[k + h];
+                    u[k] = p + q;
+                    u[k + h] = p - q;
+                }
         }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (l + 512 * k < B) out[l + 512 * k] = u[k];
     }
 }
 
-// levels h = 1 .. B/2 inside blocks of B consecutive entries of a column
-template <typename T>
-__global__ void __launch_bounds__(512) k_fwht_block(T* __restrict__ W, int64_t mp, int B) {
-    extern __shared__ __align__(16) unsigned char fw_raw[];
-    T* x = reinterpret_cast<T*>(fw_raw);
-    T* base = W + (size_t)blockIdx.y * mp + (size_t)blockIdx.x * B;
-    for (int i = threadIdx.x; i < B; i += blockDim.x) x[i] = base[i];
-    __syncthreads();
-    for (int h = 1; h < B; h <<= 1) {
-        for (int p = threadIdx.x; p < B / 2; p += blockDim.x) {
-            const int i = (p / h) * 2 * h + (p % h);
-            const T a = x[i], b = x[i + h];
-            x[i] = a + b;
-            x[i + h] = a - b;
-        }
-        __syncthreads();
-    }
-    for (int i = threadIdx.x; i < B; i += blockDim.x) base[i] = x[i];
-}
-
-// levels h = B .. mp/2: for 32 consecutive offsets o of a column, the
-// K = mp / B entries o + k B held in shared memory, levels k-wise
-template <typename T>
-__global__ void __launch_bounds__(256) k_fwht_stride(T* __restrict__ W, int64_t mp, int B) {
-    extern __shared__ __align__(16) unsigned char fs_raw[];
-    T* x = reinterpret_cast<T*>(fs_raw);  // [K][32]
-    const int K = (int)(mp / B);
-    const int o0 = blockIdx.x * 32;
-    T* col = W + (size_t)blockIdx.y * mp;
-    for (int q = threadIdx.x; q < K * 32; q += blockDim.x) {
-        const int k = q >> 5, o = q & 31;
-        x[q] = col[(size_t)k * B + o0 + o];
-    }
-    __syncthreads();
-    for (int h = 1; h < K; h <<= 1) {
-        for (int q = threadIdx.x; q < (K / 2) * 32; q += blockDim.x) {
-            const int p = q >> 5, o = q & 31;
-            const int i = (p / h) * 2 * h + (p % h);
-            const T a = x[i * 32 + o], b = x[(i + h) * 32 + o];
-            x[i * 32 + o] = a + b;
-            x[(i + h) * 32 + o] = a - b;
-        }
-        __syncthreads();
-    }
-    for (int q = threadIdx.x; q < K * 32; q += blockDim.x) {
-        const int k = q >> 5, o = q & 31;
-        col[(size_t)k * B + o0 + o] = x[q];
-    }
+// L further levels h0, 2 h0, ..., 2^(L-1) h0: a thread holds the 2^L entries of
+// a column that they join, in registers.  HBM bound (a read and a write of W):
+// with the entries in shared memory and two barriers per level 261 us for five
+// levels of 131072 x 400, 58 us so.
+template <typename T, int L>
+__global__ void __launch_bounds__(256) k_fwht_levels(T* __restrict__ W, int64_t mp, int64_t h0) {
+    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;  // < mp / 2^L
+    T* base = W + (size_t)blockIdx.y * mp + (p / h0) * (h0 << L) + p % h0;
+    T v[1 << L];
+#pragma unroll
+    for (int k = 0; k < (1 << L); ++k) v[k] = base[k * h0];
+#pragma unroll
+    for (int h = 1; h < (1 << L); h <<= 1)
+#pragma unroll
+        for (int k = 0; k < (1 << L); ++k)
+            if (!(k & h)) {
+                const T a = v[k], b = v[k + h];
+                v[k] = a + b;
+                v[k + h] = a - b;
+            }
+#pragma unroll
+    for (int k = 0; k < (1 << L); ++k) base[k * h0] = v[k];
 }
 
 template <typename T, typename TO>
@@ -691,40 +741,44 @@ size_t srft_ws_bytes(int64_t m, int64_t n, int prec) {
     return (prec == LSQ_FP64 ? 8 : 4) * (size_t)srft_order(m) * (size_t)n;
 }
 
-template <typename T>
-static lsq_status srft_run(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp, int prec,
-                           uint64_t seed, int64_t s, T* W, void* As, int64_t ldas, cudaStream_t st) {
+template <typename T, int PREC>
+static lsq_status srft_run(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp, uint64_t seed,
+                           int64_t s, T* W, void* As, int64_t ldas, cudaStream_t st) {
     const int64_t mp = srft_order(m);
-    if (mp > ((int64_t)1 << 30)) return LSQ_ERR_ARG;
-    const int64_t cpb = 8;  // columns per block of the load
-    dim3 gl((unsigned)min64(ceil_div(mp, 256), 4096), (unsigned)ceil_div(n, cpb));
-    k_srft_load<T><<<gl, 256, 0, st>>>(A, m, n, lda, colexp, prec, seed, mp, cpb, W);
+    // largest order: 2^10 blocks in FP32, 2^9 in FP64
+    if (mp > ((int64_t)FW_B << (sizeof(T) == 8 ? 9 : 10))) return LSQ_ERR_ARG;
+    k_srft_block<T, PREC><<<dim3((unsigned)ceil_div(mp, FW_B), (unsigned)n), 256, 0, st>>>(A, m, lda, colexp, seed, mp, W);
     LSQ_LAUNCH_CHECK();
-    const int B = (int)std::min<int64_t>(mp, 4096);
-    k_fwht_block<T><<<dim3((unsigned)(mp / B), (unsigned)n), 512, sizeof(T) * B, st>>>(W, mp, B);
-    LSQ_LAUNCH_CHECK();
-    if (mp > B) {
-        const int K = (int)(mp / B);
-        const size_t smem = sizeof(T) * (size_t)K * 32;
-        if (smem > 200 * 1024) return LSQ_ERR_ARG;
-        if (smem > 48 * 1024)
-            LSQ_CUDA_TRY(cudaFuncSetAttribute(k_fwht_stride<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_fwht_stride<T><<<dim3((unsigned)(B / 32), (unsigned)n), 256, smem, st>>>(W, mp, B);
+    // the levels above: at most five at a time
+    for (int64_t h = FW_B; h < mp;) {
+        int L = 0;
+        while (L < 5 && (h << L) < mp) ++L;
+        const dim3 g((unsigned)((mp >> L) / 256), (unsigned)n);
+        switch (L) {
+        case 1: k_fwht_levels<T, 1><<<g, 256, 0, st>>>(W, mp, h); break;
+        case 2: k_fwht_levels<T, 2><<<g, 256, 0, st>>>(W, mp, h); break;
+        case 3: k_fwht_levels<T, 3><<<g, 256, 0, st>>>(W, mp, h); break;
+        case 4: k_fwht_levels<T, 4><<<g, 256, 0, st>>>(W, mp, h); break;
+        default: k_fwht_levels<T, 5><<<g, 256, 0, st>>>(W, mp, h); break;
+        }
         LSQ_LAUNCH_CHECK();
+        h <<= L;
     }
     dim3 gg((unsigned)min64(ceil_div(s, 256), 1024), (unsigned)n);
-    if (prec == LSQ_FP64)
-        k_srft_gather<T, double><<<gg, 256, 0, st>>>(W, mp, n, seed, s, (double*)As, ldas);
-    else
-        k_srft_gather<T, float><<<gg, 256, 0, st>>>(W, mp, n, seed, s, (float*)As, ldas);
+    k_srft_gather<T, T><<<gg, 256, 0, st>>>(W, mp, n, seed, s, (T*)As, ldas);
     LSQ_LAUNCH_CHECK();
     return LSQ_OK;
 }
 
 lsq_status launch_srft(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp, int prec,
                        uint64_t seed, int64_t s, void* W, void* As, int64_t ldas, cudaStream_t st) {
-    if (prec == LSQ_FP64) return srft_run<double>(A, m, n, lda, colexp, prec, seed, s, (double*)W, As, ldas, st);
-    return srft_run<float>(A, m, n, lda, colexp, prec, seed, s, (float*)W, As, ldas, st);
+    switch (prec) {
+    case LSQ_FP64: return srft_run<double, LSQ_FP64>(A, m, n, lda, colexp, seed, s, (double*)W, As, ldas, st);
+    case LSQ_FP8_E4M3: return srft_run<float, LSQ_FP8_E4M3>(A, m, n, lda, colexp, seed, s, (float*)W, As, ldas, st);
+    case LSQ_BF16: return srft_run<float, LSQ_BF16>(A, m, n, lda, colexp, seed, s, (float*)W, As, ldas, st);
+    case LSQ_FP16: return srft_run<float, LSQ_FP16>(A, m, n, lda, colexp, seed, s, (float*)W, As, ldas, st);
+    default: return srft_run<float, LSQ_FP32>(A, m, n, lda, colexp, seed, s, (float*)W, As, ldas, st);
+    }
 }
 
 __global__ void k_gauss_inspect(const ZigTable tab, uint64_t seed, int64_t s, int64_t m, int prec,

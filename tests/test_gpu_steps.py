@@ -96,6 +96,26 @@ def test_srft_sketch_bit_exact(prec, m, n, s):
     np.testing.assert_array_equal(to_np(As).astype(np.float64), oAs)
 
 
+@pytest.mark.parametrize("prec", [O.FP8_E4M3, O.FP32, O.FP64])
+@pytest.mark.parametrize("m", [4, 17, 32, 33, 512, 513, 4095, 4097, 16384, 65537, 140000, 300000])
+def test_srft_block_orders(prec, m):
+    # orders below, at and above the 512 and 4096 entries that a warp and a CTA
+    # hold, one to five and seven levels above: bit for bit, with entries that
+    # round to subnormals and to zero, and a leading dimension above m
+    n, s = 3, min(m, 70)
+    rng = np.random.default_rng(m)
+    A = np.asfortranarray(rng.standard_normal((m, n)) * np.exp2(rng.integers(-40, 1, (m, n))))
+    A[rng.integers(0, m, 1 + m // 9), :] = 0.0
+    A[m // 2, :] = [1.0, -3.0, 2.0**-30]
+    opts = lsq.make_opts(kind=lsq.SRFT, s=s, zeta=0, seed=5, sketch_prec=prec)
+    big = dev_colmajor(np.asfortranarray(np.vstack([A, np.full((3, n), np.nan)])))
+    As, ce, info = lsq.sketch(big[:m], opts)
+    oAs, oce = O.sketch(A, O.SRFT, s, 0, 5, prec)
+    assert int(to_np(info)[0]) == 0
+    np.testing.assert_array_equal(to_np(ce), oce)
+    np.testing.assert_array_equal(to_np(As).astype(np.float64), oAs)
+
+
 @pytest.mark.parametrize("prec", [O.FP8_E4M3, O.BF16, O.FP16, O.FP32, O.FP64])
 def test_gaussian_sketch_within_rounding(prec):
     m, n, s = 1037, 113, 250
