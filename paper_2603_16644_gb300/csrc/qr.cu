@@ -179,7 +179,8 @@ __global__ void __launch_bounds__(QPT) k_qr_panel(T* __restrict__ W, int64_t ld,
 constexpr int QCT = 256;
 constexpr int QKG = QCT / 64;  // row groups of the previous-panel product (64 threads each)
 
-constexpr int QRC = 32;  // panel rows per warp kept in registers
+constexpr int QRC = 32;   // panel rows per warp kept in registers, FP64
+constexpr int QRC32 = 64;  // FP32
 
 // 4 consecutive values from 16-byte aligned shared memory
 __device__ __forceinline__ void load4(const float* p, float (&o)[4]) {
@@ -273,8 +274,8 @@ __global__ void __launch_bounds__(QCT)
     __shared__ T bsh[QNB];
     __shared__ T Wr[QNB][QNB + 1];  // this CTA's partial V_p^T C (read by the whole cluster)
     __shared__ T Ysm[QNB][QNB + 1];  // rank 0: Y = V^T V (strictly upper part), built column by column
-    __shared__ __align__(16) T bcv[QCT / 32][QRC];  // per warp: v_jj on its rows
-    __shared__ __align__(16) T bcx[QCT / 32][QRC];  // per warp: x_{jj+1} below its diagonal
+    // FP32, per warp: u_jj and the next column on its rows (by the column's parity)
+    __shared__ __align__(16) T bcx[2][QCT / 32][std::is_same<T, float>::value ? QRC32 : 4];
     __shared__ T rowbuf[QNB];                      // row jj of the panel (owning CTA)
     __shared__ T scal_sh[4];                       // FP64: mu, b, v1, 1 / v1 of the column (warp 0)
     __shared__ T wc_sh[QNB], f_sh[QNB];            // FP64: w_c and w_c / v1 of the column (warp 0)
@@ -342,6 +343,7 @@ __global__ void __launch_bounds__(QCT)
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int b = 0; b < 4; ++b) acc[a][b] = (T)0;
+#pragma unroll 4
             for (int i = i0; i < i1; ++i) {
                 T v[4], c[4];
 #pragma unroll
@@ -353,8 +355,9 @@ __global__ void __launch_bounds__(QCT)
 #pragma unroll
                     for (int b = 0; b < 4; ++b) acc[a][b] = fma(v[a], c[b], acc[a][b]);
             }
-            if (rank == 0 && kg == 0)
-                for (int i = 0; i < QNB; ++i) {
+            if (rank == 0)
+#pragma unroll 4
+                for (int i = kg * (QNB / QKG); i < (kg + 1) * (QNB / QKG); ++i) {
                     T v[4], c[4];
 #pragma unroll
                     for (int a = 0; a < 4; ++a) v[a] = Vt[i * (QNB + 1) + 4 * tp + a];
@@ -393,39 +396,50 @@ __global__ void __launch_bounds__(QCT)
         }
         for (int q = tid; q < QNB * QNB; q += QCT) Ts[q & 31][q >> 5] = Tp[q];  // Ts[k][p] = T_p[k, p]
         __syncthreads();
-        for (int q = tid; q < QNB * QNB; q += QCT) {
-            const int p = q >> 5, c = q & 31;
-            T w = (T)0;
-            for (int kk = 0; kk <= p; ++kk) w = fma(Ts[kk][p], Wf[kk * (QNB + 1) + c], w);
-            W2[p * QNB + c] = w;  // (T_p^T W)[p, c]
+        {
+            // T_p^T W: rows warp, warp + 8, ... (T_p is zero below its diagonal)
+            T w[QNB * 32 / QCT];
+#pragma unroll
+            for (int e = 0; e < QNB * 32 / QCT; ++e) w[e] = (T)0;
+#pragma unroll 8
+            for (int kk = 0; kk < QNB; ++kk) {
+                const T f = Wf[kk * (QNB + 1) + lane];
+#pragma unroll
+                for (int e = 0; e < QNB * 32 / QCT; ++e) w[e] = fma(Ts[kk][warp + e * (QCT / 32)], f, w[e]);
+            }
+#pragma unroll
+            for (int e = 0; e < QNB * 32 / QCT; ++e) W2[(warp + e * (QCT / 32)) * QNB + lane] = w[e];
         }
         __syncthreads();
-        // C -= V_p W2, one row per thread
-        for (int i = tid; i < nloc; i += QCT) {
+        // C -= V_p W2, one row per thread; rank 0's rows above the panel follow its own
+        const int nrow = nloc + (rank == 0 ? QNB : 0);
+        for (int i = tid; i < nrow; i += QCT) {
+            const bool own = i < nloc;
+            T* cp = own ? P + i : Ct + (i - nloc) * (QNB + 1);
+            const T* vp = own ? Vl + i : Vt + (i - nloc) * (QNB + 1);
+            const int st = own ? Rp : 1;
             T a[QNB];
 #pragma unroll
-            for (int c = 0; c < QNB; ++c) a[c] = P[c * Rp + i];
+            for (int c = 0; c < QNB; ++c) a[c] = cp[c * st];
+#pragma unroll 2
             for (int p = 0; p < QNB; ++p) {
-                const T v = Vl[p * Rp + i];
+                const T v = vp[p * st];
 #pragma unroll
-                for (int c = 0; c < QNB; ++c) a[c] = fma(-v, W2[p * QNB + c], a[c]);
+                for (int c = 0; c < QNB; c += 4) {
+                    T w[4];
+                    load4(W2 + p * QNB + c, w);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) a[c + e] = fma(-v, w[e], a[c + e]);
+                }
             }
+            if (own) {
 #pragma unroll
-            for (int c = 0; c < QNB; ++c) P[c * Rp + i] = a[c];
-        }
-        if (rank == 0 && tid < QNB) {
-            const int64_t gi = k0 - QNB + tid;
-            T a[QNB];
+                for (int c = 0; c < QNB; ++c) P[c * Rp + i] = a[c];
+            } else {
 #pragma unroll
-            for (int c = 0; c < QNB; ++c) a[c] = Ct[tid * (QNB + 1) + c];
-            for (int p = 0; p < QNB; ++p) {
-                const T v = Vt[tid * (QNB + 1) + p];
-#pragma unroll
-                for (int c = 0; c < QNB; ++c) a[c] = fma(-v, W2[p * QNB + c], a[c]);
+                for (int c = 0; c < QNB; ++c)
+                    if (c < nb) W[(k0 - QNB + i - nloc) + (k0 + c) * ld] = a[c];
             }
-#pragma unroll
-            for (int c = 0; c < QNB; ++c)
-                if (c < nb) W[gi + (k0 + c) * ld] = a[c];
         }
         __syncthreads();
     }
@@ -483,7 +497,8 @@ __global__ void __launch_bounds__(QCT)
     // scalars, w_c for each column and (rank 0) column jj - 1 of Y.
     struct Scal {
         T mu, b, v1, rv1, wc;  // R's diagonal entry, beta, v's leading entry before scaling, its reciprocal, w_c
-        T f;                   // FP64: w_c / v1
+        T f;                   // w_c / v1 (register forms)
+        T rc;                  // FP32 register form: R[jj][c]
         bool scale;
     };
     // FP64: the sign of v1 is that of x1 (no cancellation, no case distinction;
@@ -532,6 +547,38 @@ __global__ void __launch_bounds__(QCT)
         if (rank == owner && tid == 0) beta_out[k0 + jj] = sc.b;
         return sc;
     };
+    // The same in FP32, by IEEE operations: two divisions after the root, and
+    // w_c and w_c / v1 need none.
+    auto scalars32 = [&](int jj, int buf, int owner) -> Scal {
+        Scal sc;
+        const T dsum = tree_sum<T, QCL>(&all_part[buf][0][lane], QNB);
+        const T sigma = __shfl_sync(0xffffffffu, dsum, jj);
+        const T x1 = all_row[buf][jj], ac = all_row[buf][lane];
+        sc.scale = sigma != (T)0;
+        sc.mu = x1;
+        sc.b = (T)0;
+        sc.v1 = (T)1;
+        sc.rv1 = (T)1;
+        sc.wc = sc.f = (T)0;
+        if (sc.scale) {
+            // beta = 2 / v^T v from 1 / v1 as it is used: its error is common to
+            // all rows and would show in R
+            const T mu = sqrt(fma(x1, x1, sigma)), av = fabs(x1) + mu, rv = (T)1 / av;
+            sc.b = (T)2 / fma(sigma * rv, rv, (T)1);
+            sc.v1 = x1 < (T)0 ? -av : av;
+            sc.rv1 = x1 < (T)0 ? -rv : rv;
+            sc.mu = x1 < (T)0 ? mu : -mu;
+            if (lane > jj && lane < nb) {
+                sc.wc = sc.b * fma(dsum, sc.rv1, ac);
+                sc.f = sc.wc * sc.rv1;
+                sc.rc = ac - sc.wc;
+            }
+        }
+        if (rank == 0 && warp == 0 && lane + 1 < jj) Ysm[lane][jj - 1] = dsum;
+        if (tid == 0) bsh[jj] = sc.b;
+        if (rank == owner && tid == 0) beta_out[k0 + jj] = sc.b;
+        return sc;
+    };
     // The Householder scalars of column jj from the exchanged partials (the
     // same in every CTA) and, per lane c > jj, w_c.
     auto scalars = [&](int jj, int buf, int owner) -> Scal {
@@ -562,7 +609,7 @@ __global__ void __launch_bounds__(QCT)
         if (rank == owner && tid == 0) beta_out[k0 + jj] = sc.b;
         return sc;
     };
-    auto exchange = [&](int jj, T acc, const T* rowsrc, int rowstride) -> Scal {
+    auto exchange = [&](int jj, T acc, const T* rowsrc, int rowstride, bool unscaled = false) -> Scal {
         const int buf = jj & 1;
         const int owner = (int)(jj / R);
         part[warp][lane] = acc;
@@ -604,11 +651,13 @@ __global__ void __launch_bounds__(QCT)
             sc.f = f_sh[lane];
             return sc;
         }
-        return scalars(jj, buf, owner);
+        return unscaled ? scalars32(jj, buf, owner) : scalars(jj, buf, owner);
     };
     T acc;
-    T yscale = (T)1;  // scale of lane i's entry of Y's last column
-    if (std::is_same<T, double>::value && chunk <= QRC) {
+    T ysc0 = (T)1, ysc1 = (T)1;  // scales of lane i's entry of Y's last column
+    bool done = false;  // columns kept in registers
+    if constexpr (std::is_same<T, double>::value) {
+      if (chunk <= QRC) {
         // FP64: each thread keeps its column's QRC rows of this warp in
         // registers; per column every lane of a warp takes the raw column jj
         // from lane jj and, after the update, column jj + 1 from lane jj + 1 by
@@ -697,7 +746,7 @@ __global__ void __launch_bounds__(QCT)
                 for (int q = 0; q < QR; ++q) s4[q & 3] = fma(ylane ? u[q] : xn[q], a[q], s4[q & 3]);
                 acc = (ylane || dlane) ? (s4[0] + s4[1]) + (s4[2] + s4[3]) : (T)0;
             }
-            yscale = myscale * rprev;  // of Y's last column, formed below
+            ysc0 = myscale * rprev;  // of Y's last column, formed below
             // R on and above the diagonal, v below it
             if (lane < nb) {
 #pragma unroll
@@ -718,121 +767,130 @@ __global__ void __launch_bounds__(QCT)
         else if (chunk <= 24) f64_cols(std::integral_constant<int, 24>{});
         else if (chunk <= 28) f64_cols(std::integral_constant<int, 28>{});
         else f64_cols(std::integral_constant<int, QRC>{});
-    } else if (chunk <= QRC) {
-        // Each thread keeps its column's QRC rows of this warp in registers
-        // (rows g0 + q); per column a warp broadcasts v_jj and x_{jj+1} through
-        // its own QRC-entry shared buffers, read 4 rows per load.
-        T a[QRC];
-#pragma unroll
-        for (int q = 0; q < QRC; ++q) a[q] = g0 + q < g1 ? P[lane * Rp + g0 + q] : (T)0;
-        T* bv = &bcv[warp][0];
-        T* bx = &bcx[warp][0];
-        const int gr0 = r0 + g0;  // global row (from k0) of a[0]
-        const int nv = g1 - g0;   // valid rows of this warp (<= 0: none)
-        // the diagonal row value a_lane[row] of this warp (0 when not here)
-        auto row_of = [&](int row) -> T {
-            T v = (T)0;
-#pragma unroll
-            for (int q = 0; q < QRC; ++q)
-                if (gr0 + q == row && q < nv) v = a[q];
-            return v;
-        };
-        // x_0 below row 0, then the dots of column 0
-        if (lane == 0) {
-#pragma unroll
-            for (int q = 0; q < QRC; q += 4) {
-                T o[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) o[e] = (q + e < nv && gr0 + q + e > 0) ? a[q + e] : (T)0;
-                store4(bx + q, o[0], o[1], o[2], o[3]);
-            }
-        }
-        if (0 >= gr0 && 0 < gr0 + nv) rowbuf[lane] = row_of(0);
-        __syncwarp();
-        acc = (T)0;
-        if (lane < nb) {
-            T s4[4] = {(T)0, (T)0, (T)0, (T)0};  // 4 chains of 8 FMAs
-#pragma unroll
-            for (int q = 0; q < QRC; q += 4) {
-                T xv[4];
-                load4(bx + q, xv);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) s4[e] = fma(xv[e], a[q + e], s4[e]);
-            }
-            acc = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-        }
-        for (int jj = 0; jj < nb; ++jj) {
-            // rowbuf (row jj, written by the warp that owns it) is read after
-            // the CTA barrier inside the exchange
-            const Scal sc = exchange(jj, acc, rowbuf, 1);
-            // v_jj of this warp's rows: raw column from lane jj, scaled by all lanes
-            if (lane == jj) {
-#pragma unroll
-                for (int q = 0; q < QRC; q += 4) store4(bv + q, a[q], a[q + 1], a[q + 2], a[q + 3]);
-            }
-            __syncwarp();
-            if (lane < QRC) {  // lane = row of this warp here
-                const int gr = gr0 + lane;
-                const T x = bv[lane];
-                bv[lane] = (gr < jj || lane >= nv) ? (T)0 : (gr == jj ? (T)1 : (sc.scale ? x * sc.rv1 : x));
-            }
-            __syncwarp();
-            if (lane == jj) {
-#pragma unroll
-                for (int q = 0; q < QRC; q += 4) {
-                    T vv[4];
-                    load4(bv + q, vv);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        if (q + e < nv && gr0 + q + e > jj) a[q + e] = vv[e];
-                        if (q + e < nv && gr0 + q + e == jj) a[q + e] = sc.mu;  // R diagonal (v there is 1)
-                    }
-                }
-            }
-            if (lane > jj && lane < nb && sc.b != (T)0) {
-#pragma unroll
-                for (int q = 0; q < QRC; q += 4) {
-                    T vv[4];
-                    load4(bv + q, vv);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) a[q + e] = fma(-sc.wc, vv[e], a[q + e]);
-                }
-            }
-            // x_{jj+1} below its diagonal and row jj + 1 for the next exchange
-            const int jn = jj + 1;
-            if (jn < nb) {
-                if (lane == jn) {
-#pragma unroll
-                    for (int q = 0; q < QRC; q += 4) {
-                        T o[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) o[e] = (q + e < nv && gr0 + q + e > jn) ? a[q + e] : (T)0;
-                        store4(bx + q, o[0], o[1], o[2], o[3]);
-                    }
-                }
-                if (jn >= gr0 && jn < gr0 + nv) rowbuf[lane] = row_of(jn);
-            }
-            __syncwarp();
-            // lanes c > jj: dots of column jj + 1; lanes i < jj: Y[i][jj]
-            const bool ylane = lane < jj, dlane = lane >= jn && lane < nb && jn < nb;
-            acc = (T)0;
-            if (ylane || dlane) {
-                const T* src = ylane ? bv : bx;
-                T s4[4] = {(T)0, (T)0, (T)0, (T)0};  // 4 chains of 8 FMAs
-#pragma unroll
-                for (int q = 0; q < QRC; q += 4) {
-                    T xv[4];
-                    load4(src + q, xv);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) s4[e] = fma(xv[e], a[q + e], s4[e]);
-                }
-                acc = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < QRC; ++q)
-            if (q < nv) P[lane * Rp + g0 + q] = a[q];
+        done = true;
+      }
     } else {
+        // Each thread keeps its column's QR rows of this warp in registers; per
+        // column the warp broadcasts u_jj and x_{jj+1} through its own buffers,
+        // read 4 rows per load.  The columns stay unscaled as in the FP64 form:
+        // with v formed and stored back, a row's place compared at each of five
+        // passes over 32 rows and three dependent divisions, a column cost 3000
+        // cycles beside its exchange whatever the rows of the warp: the panels of a
+        // 1200 x 400 sketch 105 us each, 68 us so (with the previous panel's product
+        // above spread over the CTA).  QR = 8 ... 64 is the fewest that hold the rows.
+        auto f32_cols = [&](auto qr_tag) {
+            constexpr int QR = decltype(qr_tag)::value;
+            T a[QR];
+#pragma unroll
+            for (int q = 0; q < QR; ++q) a[q] = g0 + q < g1 ? P[lane * Rp + g0 + q] : (T)0;
+            const int gr0 = r0 + g0;  // global row (from k0) of a[0]
+            const int nv = g1 - g0;   // valid rows of this warp (<= 0: none); a is zero beyond
+            auto row_of = [&](int row) -> T {
+                T v = (T)0;
+#pragma unroll
+                for (int q = 0; q < QR; ++q)
+                    if (gr0 + q == row) v = a[q];
+                return v;
+            };
+            // lane c: its column below row `row`
+            auto put_below = [&](T* x, int row) {
+                if (gr0 > row) {
+#pragma unroll
+                    for (int q = 0; q < QR; q += 4) store4(x + q, a[q], a[q + 1], a[q + 2], a[q + 3]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < QR; ++q) x[q] = gr0 + q > row ? a[q] : (T)0;
+                }
+            };
+            auto dot = [&](const T* x) -> T {
+                constexpr int CH = QR > 32 ? 8 : 4;  // chains
+                T s4[CH];
+#pragma unroll
+                for (int e = 0; e < CH; ++e) s4[e] = (T)0;
+#pragma unroll
+                for (int q = 0; q < QR; q += 4) {
+                    T xv[4];
+                    load4(x + q, xv);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) s4[(q + e) % CH] = fma(xv[e], a[q + e], s4[(q + e) % CH]);
+                }
+                T r = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+                if constexpr (CH == 8) r += (s4[4] + s4[5]) + (s4[6] + s4[7]);
+                return r;
+            };
+            T myscale = (T)1, myR = (T)0, rprev = (T)1;
+            if (lane == 0) put_below(&bcx[0][warp][0], 0);
+            if (0 >= gr0 && 0 < gr0 + nv) rowbuf[lane] = row_of(0);
+            __syncwarp();
+            acc = dot(&bcx[0][warp][0]);
+            if (lane >= nb) acc = (T)0;
+            for (int jj = 0; jj < nb; ++jj) {
+                const Scal sc = exchange(jj, acc, rowbuf, 1, true);
+                // Y[i][j] = v_i^T v_j from u_i^T u_j (lane i; rank 0, warp 0)
+                if (rank == 0 && warp == 0 && lane < jj - 1) Ysm[lane][jj - 1] = Ysm[lane][jj - 1] * myscale * rprev;
+                T* u = &bcx[jj & 1][warp][0];
+                T* xn = &bcx[(jj + 1) & 1][warp][0];
+                if (jj >= gr0 && jj < gr0 + nv) {  // the leading entry of u_jj
+                    if (lane == 0) u[jj - gr0] = sc.v1;
+                    __syncwarp();
+                }
+                if (lane == jj) {
+                    myscale = sc.rv1;
+                    myR = sc.mu;
+                }
+                rprev = sc.rv1;
+                if (lane > jj && lane < nb && sc.b != (T)0) {
+                    const T f = sc.f;
+#pragma unroll
+                    for (int q = 0; q < QR; q += 4) {
+                        T uv[4];
+                        load4(u + q, uv);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) a[q + e] = fma(-f, uv[e], a[q + e]);
+                    }
+                    // R's row without the roundings of f and v1
+                    if (jj >= gr0 && jj < gr0 + nv) {
+#pragma unroll
+                        for (int q = 0; q < QR; ++q) a[q] = gr0 + q == jj ? sc.rc : a[q];
+                    }
+                }
+                const int jn = jj + 1;
+                if (jn < nb) {
+                    if (lane == jn) put_below(xn, jn);
+                    if (jn >= gr0 && jn < gr0 + nv) rowbuf[lane] = row_of(jn);
+                }
+                __syncwarp();
+                // lanes c > jj: dots of column jj + 1; lanes i < jj: u_i^T u_jj
+                const bool ylane = lane < jj, dlane = lane >= jn && lane < nb && jn < nb;
+                acc = dot(ylane ? u : xn);
+                if (!(ylane || dlane)) acc = (T)0;
+            }
+            // lane < nb - 1: the scales of Y's last column, formed below
+            if (rank == 0 && warp == 0) {
+                ysc0 = myscale;
+                ysc1 = rprev;
+            }
+            // R on and above the diagonal, v below it
+            if (lane < nb) {
+#pragma unroll
+                for (int q = 0; q < QR; ++q) {
+                    const int gr = gr0 + q;
+                    a[q] = gr > lane ? a[q] * myscale : (gr == lane ? myR : a[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < QR; ++q)
+                if (q < nv) P[lane * Rp + g0 + q] = a[q];
+        };
+        done = true;
+        if (chunk <= 8) f32_cols(std::integral_constant<int, 8>{});
+        else if (chunk <= 16) f32_cols(std::integral_constant<int, 16>{});
+        else if (chunk <= 24) f32_cols(std::integral_constant<int, 24>{});
+        else if (chunk <= 32) f32_cols(std::integral_constant<int, 32>{});
+        else if (chunk <= QRC32) f32_cols(std::integral_constant<int, QRC32>{});
+        else done = false;
+    }
+    if (!done) {
         acc = dots(0);
         for (int jj = 0; jj < nb; ++jj) {
             T* xj = P + jj * Rp;
@@ -880,11 +938,12 @@ __global__ void __launch_bounds__(QCT)
     }
     cluster.sync();
     if (rank == 0 && warp == 0 && lane + 1 < nb)
-        Ysm[lane][nb - 1] = tree_sum<T, QCL>(&all_part[nb & 1][0][lane], QNB) * yscale;
+        Ysm[lane][nb - 1] = tree_sum<T, QCL>(&all_part[nb & 1][0][lane], QNB) * ysc0 * ysc1;
     // write R / v back to W and the explicit V (0 above, 1 on the diagonal)
-    for (int c = 0; c < QNB; ++c)
-        for (int i = tid; i < nloc; i += QCT) {
-            const int64_t gi = r0 + i;
+    for (int i = tid; i < nloc; i += QCT) {
+        const int64_t gi = r0 + i;
+#pragma unroll 8
+        for (int c = 0; c < QNB; ++c) {
             if (c < nb) {
                 const T pv = P[c * Rp + i];
                 W[(k0 + gi) + (k0 + c) * ld] = pv;
@@ -893,6 +952,7 @@ __global__ void __launch_bounds__(QCT)
                 V[gi + c * ldv] = (T)0;
             }
         }
+    }
     __syncthreads();
     if (rank == 0) {
         __syncthreads();
