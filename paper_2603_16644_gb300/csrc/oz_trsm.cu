@@ -169,7 +169,7 @@ __global__ void k_ot_rowexp(const unsigned long long* __restrict__ Mx, int64_t m
 }
 
 // The same, with the digit planes written as whole 128-byte lines: a CTA
-// converts a 64-row x 64-column block of X (two threads per row, 32 columns
+// converts a 64-row x 64-column block of X (four threads per row, 16 columns
 // each, reading X a column at a time, coalesced over rows), stages the 8 BF16
 // digit tiles in shared memory in the 128-byte-swizzled layout of the TMA
 // (16-byte chunk j of row r at chunk j ^ (r mod 8): conflict-free for one
@@ -177,7 +177,12 @@ __global__ void k_ot_rowexp(const unsigned long long* __restrict__ Mx, int64_t m
 // of 16 bytes to 32 different rows per warp instruction reach ~1 TB/s; whole
 // lines reach ~6 TB/s.)  tmZ: the X digit planes, boxes of 64 columns x 64
 // rows x 1 plane.
+// Bytes (8 read and 16 written an element) and the conversion's latency bound
+// it: with two threads per row and X's block beside the tiles, two CTAs of 4
+// warps fitted an SM and 65536 x 64 took 27 us, 65536 x 512 175 us; three CTAs of
+// 8 warps, the block's space reused for the tiles, take 20.6 and 135 us.
 constexpr int OT_RS_ROWS = 64;
+constexpr int OT_RS_THREADS = 256;  // 4 per row, 16 columns each
 // tma_x: X's block comes in by one TMA load (tmX: FP64, boxes of 64 rows x 64
 // columns, zero outside) into shared memory [64 columns][64 rows]; otherwise
 // every thread loads its values (coalesced over rows, a column at a time).
@@ -185,7 +190,7 @@ constexpr int OT_RS_ROWS = 64;
 // largest values, formed here (the two threads of a row combine their maxima)
 // instead of from the diagonal kernel's per-block exponents.
 template <bool tma_x, bool own_exp>
-__global__ void __launch_bounds__(128) k_ot_rowslice_s(const __grid_constant__ CUtensorMap tmZ,
+__global__ void __launch_bounds__(OT_RS_THREADS, 3) k_ot_rowslice_s(const __grid_constant__ CUtensorMap tmZ,
                                                        const __grid_constant__ CUtensorMap tmX,
                                                        const double* __restrict__ X, int64_t m, int64_t mp, int64_t K,
                                                        int64_t ld, int32_t* __restrict__ Ex,
@@ -193,9 +198,10 @@ __global__ void __launch_bounds__(128) k_ot_rowslice_s(const __grid_constant__ C
                                                        int32_t* __restrict__ err) {
     extern __shared__ unsigned char rs_raw[];
     uint8_t* stage = (uint8_t*)(((uintptr_t)rs_raw + 1023) & ~(uintptr_t)1023);  // [8][64 rows][128 B]
-    const double* xt = (const double*)(stage + OT_DIG * OT_RS_ROWS * 128);      // [64 columns][64 rows]
+    // X's block [64 columns][64 rows], read into registers before the tiles are written
+    const double* xt = (const double*)stage;
     __shared__ uint64_t xfull;
-    __shared__ unsigned long long rmax[2][OT_RS_ROWS];
+    __shared__ unsigned long long rmax[4][OT_RS_ROWS];
     __shared__ int rs_bad;
     const int r = threadIdx.x & (OT_RS_ROWS - 1), h = threadIdx.x >> 6;
     const int64_t i0 = (int64_t)blockIdx.x * OT_RS_ROWS, kb = (int64_t)blockIdx.y * 64;
@@ -218,8 +224,6 @@ __global__ void __launch_bounds__(128) k_ot_rowslice_s(const __grid_constant__ C
             for (int b = 0; b < nbk; ++b) eb = max(eb, Eblk[(b0 + b) * m + i]);
         E = eb == INT32_MIN ? 0 : eb;
     }
-    const double* row = X + i;
-    const int64_t Kr = i < m ? K : 0;
     if constexpr (tma_x) {
         if (!mbar_wait(&xfull, 0)) rs_bad = 1;
         __syncthreads();
@@ -231,45 +235,49 @@ __global__ void __launch_bounds__(128) k_ot_rowslice_s(const __grid_constant__ C
             return;
         }
     }
+    // this thread's 16 columns of row i
+    const int kl = 16 * h;
+    double xv[16];
+    if constexpr (tma_x) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) xv[q] = xt[(kl + q) * OT_RS_ROWS + r];  // zero outside X (TMA fill)
+    } else {
+        const double* row = X + i;
+        const int64_t k0 = kb + kl, Kr = i < m ? K : 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) xv[q] = k0 + q < Kr ? row[(k0 + q) * ld] : 0.0;
+    }
     if constexpr (own_exp) {
         unsigned long long mx = 0;
-        for (int q = 0; q < 32; ++q) {
-            const unsigned long long v =
-                (unsigned long long)__double_as_longlong(xt[(32 * h + q) * OT_RS_ROWS + r]) & 0x7fffffffffffffffull;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const unsigned long long v = (unsigned long long)__double_as_longlong(xv[q]) & 0x7fffffffffffffffull;
             mx = v > mx ? v : mx;
         }
         rmax[h][r] = mx;
-        __syncthreads();
-        mx = rmax[0][r] > rmax[1][r] ? rmax[0][r] : rmax[1][r];
+    }
+    if constexpr (tma_x) __syncthreads();  // every value read: the tiles may be written
+    if constexpr (own_exp) {
+        unsigned long long mx = 0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) mx = rmax[g][r] > mx ? rmax[g][r] : mx;
         E = ot_exp_of_max(mx);
     }
     if (blockIdx.y == 0 && h == 0) Ex[i] = E;
-#pragma unroll 1
-    for (int bb = 0; bb < 2; ++bb) {
-        const int kl = 32 * h + 16 * bb;  // first of 16 columns within the block
-        const int64_t k0 = kb + kl;
-        double xv[16];
-        if constexpr (tma_x) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) xv[q] = xt[(kl + q) * OT_RS_ROWS + r];  // zero outside X (TMA fill)
-        } else {
+    for (int g = 0; g < 2; ++g) {  // 8 columns: one 16-byte chunk of each digit tile
+        uint32_t pk[OT_DIG][4];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) xv[q] = k0 + q < Kr ? row[(k0 + q) * ld] : 0.0;
-        }
-        uint32_t pk[OT_DIG][8];
-#pragma unroll
-        for (int q2 = 0; q2 < 8; ++q2) {
-            const unsigned long long W0 = ot_fields(xv[2 * q2], E), W1 = ot_fields(xv[2 * q2 + 1], E);
+        for (int q2 = 0; q2 < 4; ++q2) {
+            const unsigned long long W0 = ot_fields(xv[8 * g + 2 * q2], E), W1 = ot_fields(xv[8 * g + 2 * q2 + 1], E);
 #pragma unroll
             for (int t = 0; t < OT_DIG; ++t) pk[t][q2] = ot_digit_pair(W0, W1, t);
         }
-        const int j = kl / 8;  // first 16-byte chunk of the 32 bytes of these columns
+        const int j = kl / 8 + g;
 #pragma unroll
-        for (int t = 0; t < OT_DIG; ++t) {
-            uint8_t* rowp = stage + ((size_t)t * OT_RS_ROWS + r) * 128;
-            *(uint4*)(rowp + ((j ^ (r & 7)) << 4)) = make_uint4(pk[t][0], pk[t][1], pk[t][2], pk[t][3]);
-            *(uint4*)(rowp + (((j + 1) ^ (r & 7)) << 4)) = make_uint4(pk[t][4], pk[t][5], pk[t][6], pk[t][7]);
-        }
+        for (int t = 0; t < OT_DIG; ++t)
+            *(uint4*)(stage + ((size_t)t * OT_RS_ROWS + r) * 128 + ((j ^ (r & 7)) << 4)) =
+                make_uint4(pk[t][0], pk[t][1], pk[t][2], pk[t][3]);
     }
     // the tiles are written through the generic proxy and read by the TMA
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1228,22 +1236,22 @@ lsq_status ot_gemm_update(const double* X, int64_t ldx, const double* Y, int64_t
     } else if (xmode == 1 && ot_map(&tzs, U.Zx, U.Kp, U.mp, OT_RS_ROWS)) {
         const dim3 rg((unsigned)(U.mp / OT_RS_ROWS), (unsigned)(U.Kp / 64));
         if (ldx % 2 == 0 && ((uintptr_t)X % 16) == 0 && ot_map_f64(&txs, X, M, K, ldx)) {
-            const size_t rsm = 1024 + (size_t)OT_DIG * OT_RS_ROWS * 128 + (size_t)OT_RS_ROWS * 64 * 8;
+            const size_t rsm = 1024 + (size_t)OT_DIG * OT_RS_ROWS * 128;
             LSQ_CUDA_TRY(
                 cudaFuncSetAttribute(k_ot_rowslice_s<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
-            k_ot_rowslice_s<true, false><<<rg, 128, rsm, st>>>(tzs, txs, X, M, U.mp, K, ldx, U.Ex, Eblk, b0, nbk, err);
+            k_ot_rowslice_s<true, false><<<rg, OT_RS_THREADS, rsm, st>>>(tzs, txs, X, M, U.mp, K, ldx, U.Ex, Eblk, b0, nbk, err);
         } else {
             const size_t rsm = 1024 + (size_t)OT_DIG * OT_RS_ROWS * 128;
             LSQ_CUDA_TRY(
                 cudaFuncSetAttribute(k_ot_rowslice_s<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
-            k_ot_rowslice_s<false, false><<<rg, 128, rsm, st>>>(tzs, tzs, X, M, U.mp, K, ldx, U.Ex, Eblk, b0, nbk, err);
+            k_ot_rowslice_s<false, false><<<rg, OT_RS_THREADS, rsm, st>>>(tzs, tzs, X, M, U.mp, K, ldx, U.Ex, Eblk, b0, nbk, err);
         }
     } else if (xmode == 0 && K <= 64 && ldx % 2 == 0 && ((uintptr_t)X % 16) == 0 &&
                ot_map(&tzs, U.Zx, U.Kp, U.mp, OT_RS_ROWS) && ot_map_f64(&txs, X, M, K, ldx)) {
-        const size_t rsm = 1024 + (size_t)OT_DIG * OT_RS_ROWS * 128 + (size_t)OT_RS_ROWS * 64 * 8;
+        const size_t rsm = 1024 + (size_t)OT_DIG * OT_RS_ROWS * 128;
         LSQ_CUDA_TRY(cudaFuncSetAttribute(k_ot_rowslice_s<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)rsm));
-        k_ot_rowslice_s<true, true><<<dim3((unsigned)(U.mp / OT_RS_ROWS), 1u), 128, rsm, st>>>(
+        k_ot_rowslice_s<true, true><<<dim3((unsigned)(U.mp / OT_RS_ROWS), 1u), OT_RS_THREADS, rsm, st>>>(
             tzs, txs, X, M, U.mp, K, ldx, U.Ex, nullptr, 0, 0, err);
     } else if (xmode == 1) {
         k_ot_rowslice_e<<<dim3((unsigned)(U.mp / 128), (unsigned)(U.Kp / 64)), 128, 0, st>>>(
