@@ -109,120 +109,100 @@ template lsq_status rank_update_ext<float>(float*, int64_t, const float*, int64_
 // ---------------------------------------------------------------------------
 // Cholesky
 // ---------------------------------------------------------------------------
-// 1 / sqrt(d) for d > 0.  FP64: an FP32 estimate (the operand and the
-// estimate moved between FP64 and FP32 with integer operations on the bit
-// patterns, no conversion instruction) refined by one third-order step
-//   e = 1 - d y^2,  y <- y + y e (1/2 + 3/8 e)
-// (from ~23 correct bits to beyond FP64 precision): four dependent FP64
-// operations, since each costs about a hundred cycles of latency on this part
-// and the pivots form the factorization's critical path.  Relative error a
-// few units in the last place.
+// 1 / sqrt(d) for a positive finite d.  FP64: an FP32 estimate y of the
+// significand's root refined by one third-order step
+//   e = 1 - m y^2,  y <- y + y (e / 2 + 3/8 e^2),  d = m 4^k, m in [1, 4)
+// in 64-bit integers (e to 2^-61): a warp issues one FP64 instruction in 64
+// cycles on this part, dependent or not, and the pivots form the
+// factorization's critical path; the integer chain takes about as long as two
+// of them.  Relative error below one unit in the last place.
 template <typename T>
 __device__ __forceinline__ T rsqrt_pivot(T d) {
     if constexpr (sizeof(T) == 4) {
         return (T)1 / sqrtf(d);
     } else {
-        if (!(d > 1e-30 && d < 1e30)) return 1.0 / sqrt(d);
         const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-        // d in the FP32 normal range: rebias the exponent, keep 23 bits of the significand
-        const uint32_t fb = (uint32_t)((((b >> 52) & 0x7ff) - 1023 + 127) << 23) | (uint32_t)((b >> 29) & 0x7fffff);
-        const uint32_t yb = __float_as_uint(rsqrtf(__uint_as_float(fb)));
-        double y = __longlong_as_double((long long)(((unsigned long long)(((yb >> 23) & 0xff) - 127 + 1023) << 52) |
-                                                    ((unsigned long long)(yb & 0x7fffff) << 29)));
-        const double t = d * y;
-        const double e = fma(-t, y, 1.0);
-        const double c = fma(0.375, e, 0.5);
-        const double ye = y * e;
-        y = fma(ye, c, y);
-        return y;
+        if ((b >> 52) == 0) return 1.0 / sqrt(d);  // subnormal
+        const int e2 = ((int)(b >> 52) - 1023) & ~1;  // 2 k
+        const unsigned long long mb = b - ((unsigned long long)(long long)e2 << 52);  // bits of m
+        const int sh = (int)(mb >> 52) - 1023;                                       // 0 or 1
+        const unsigned long long M = ((mb & 0x000fffffffffffffull) | 0x0010000000000000ull) << (10 + sh);  // m 2^62
+        const float y0 = rsqrtf(__uint_as_float((uint32_t)((mb >> 52) - 1023 + 127) << 23 | (uint32_t)((mb >> 29) & 0x7fffff)));
+        const uint32_t Y0 = (uint32_t)(y0 * 16777216.0f);  // the estimate, 2^-24 units, about (1/2, 1]
+        const unsigned long long Q = ((unsigned long long)Y0 * Y0) << 15;  // y0^2 2^63
+        const long long e = (long long)((1ull << 61) - __umul64hi(M, Q));  // 2^-61 units, below 2^41
+        const int eh = (int)(e >> 12);                                    // 2^-49 units
+        const long long ee = ((long long)eh * eh) >> 37;                  // e^2, 2^-61 units
+        const long long c = ((e >> 1) + ((3 * ee) >> 3)) >> 4;            // 2^-57 units, below 2^37
+        const unsigned long long Y = ((unsigned long long)Y0 << 36) + (unsigned long long)(((long long)Y0 * c) >> 21);  // y 2^60
+        const unsigned long long yb = ((Y + 64) >> 7) + (1021ull << 52);  // a carry to 1.0 moves into the exponent
+        return __longlong_as_double((long long)(yb - ((unsigned long long)(long long)(e2 / 2) << 52)));
     }
 }
 
-// Diagonal block (CNB x CNB) in one CTA, right-looking.  Per column j the
-// column is scaled by r_j = 1/sqrt(d_j) into a separate buffer; then thread 0
-// applies column j's update to the next diagonal entry and forms the next
-// pivot (L_jj = d r, r = 1/sqrt(d)) while the six warps of the other three
-// schedulers (warps 1-3, 5-7) update the rest of the active triangle
-// j < c <= r (row-major enumeration from a table, so that every warp issues
-// full-width FP64 instructions): the pivot's dependent FP64 chain runs on a
-// scheduler whose FP64 pipe the update leaves idle, overlapping the update.
+// d > 0 and finite, without FP64 instructions
+template <typename T>
+__device__ __forceinline__ bool pivot_ok(T d) {
+    if constexpr (sizeof(T) == 4) return d > (T)0 && isfinite(d);
+    else return (unsigned long long)(__double_as_longlong(d) - 1) < 0x7fefffffffffffffull;
+}
+
+// Diagonal block (CNB x CNB) in one CTA, right-looking, the entries of columns
+// 1 .. 63 in registers (8 a thread).  They are numbered by columns from the last
+// to the second, so that the active ones, c > j, are a prefix: thread t holds
+// entries t, t + 256, ..., and a column takes as many rounds as the prefix has.
+// Per column j: the raw column (published by its holders) times 1/sqrt(d_j),
+// then the update of the active entries.  Bound by the chain of a column (the
+// root, two FP64 operations, two barriers) and, for the first third, by the FP64
+// pipe (one warp instruction in 16 cycles per SM).  With the block in shared
+// memory, a table look-up, three loads and a store an entry, and the root in
+// FP64, a block took 49 us (87 thousand cycles, 67 of them in the update); 43 us so.
 template <typename T>
 __global__ void __launch_bounds__(256) k_potrf_diag(T* __restrict__ G, int64_t ld, int64_t n, int64_t k0,
                                                     int32_t* __restrict__ info) {
     if (*info != 0) return;
-    __shared__ T D[CNB][CNB + 1];
-    __shared__ T colj[CNB];
-    __shared__ uint16_t tri[CNB * (CNB - 1) / 2];  // e -> (rr << 8) | cc, lower triangle by rows
-    __shared__ T rj;
+    constexpr int NE = CNB * (CNB - 1) / 2, NR = (NE + 255) / 256;  // entries of columns 1 .., rounds
+    __shared__ T Ls[CNB][CNB + 1];
+    __shared__ T raw[CNB], colj[CNB];  // column j before and after the scaling
     __shared__ int bad;
     const int nb = (int)min64(CNB, n - k0);
     const int tid = threadIdx.x;
-    {
-        // all loads of the block in flight before the stores
-        T x[CNB * CNB / 256];
+    int rr[NR], cc[NR];
+    T a[NR];
 #pragma unroll
-        for (int u = 0; u < CNB * CNB / 256; ++u) {
-            const int q = tid + 256 * u, r = q & 63, c = q >> 6;
-            x[u] = (r < nb && c < nb) ? G[(k0 + r) + (k0 + c) * ld] : (T)0;
-        }
-#pragma unroll
-        for (int u = 0; u < CNB * CNB / 256; ++u) {
-            const int q = tid + 256 * u;
-            D[q & 63][q >> 6] = x[u];
-        }
+    for (int u = 0; u < NR; ++u) {
+        const int e = tid + 256 * u;
+        // column 63 - w, w (w + 1) / 2 <= e: the root is exact to a unit
+        int w = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+        if ((w + 1) * (w + 2) / 2 <= e) ++w;
+        if (w * (w + 1) / 2 > e) --w;
+        cc[u] = e < NE ? CNB - 1 - w : CNB - 1;
+        rr[u] = e < NE ? cc[u] + e - w * (w + 1) / 2 : CNB - 1;
+        a[u] = (e < NE && rr[u] < nb) ? G[(k0 + rr[u]) + (k0 + cc[u]) * ld] : (T)0;
     }
-    for (int e = tid; e < CNB * (CNB - 1) / 2; e += 256) {
-        int rr = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-        while ((rr + 1) * (rr + 2) / 2 <= e) ++rr;
-        while (rr * (rr + 1) / 2 > e) --rr;
-        tri[e] = (uint16_t)((rr << 8) | (e - rr * (rr + 1) / 2));
-    }
-    __syncthreads();
-    if (tid == 0) {
-        bad = 0;
-        const T d = D[0][0];
-        if (!(d > (T)0) || !isfinite(d)) {
-            bad = 1;
-        } else {
-            const T r = rsqrt_pivot<T>(d);
-            rj = r;
-            D[0][0] = d * r;
-        }
-    }
+    if (tid < CNB) raw[tid] = tid < nb ? G[(k0 + tid) + k0 * ld] : (T)0;
+    if (tid == 0) bad = 0;
     __syncthreads();
     for (int j = 0; j < nb; ++j) {
-        if (bad) break;
-        const T r = rj;
-        if (tid > j && tid < nb) {
-            const T l = D[tid][j] * r;
-            D[tid][j] = l;
-            colj[tid] = l;
-        }
-        __syncthreads();
-        if (j + 1 < nb) {
-            if (tid == 0) {
-                const T d = fma(-colj[j + 1], colj[j + 1], D[j + 1][j + 1]);
-                if (!(d > (T)0) || !isfinite(d)) {
-                    bad = j + 2;
-                } else {
-                    const T rn = rsqrt_pivot<T>(d);
-                    rj = rn;
-                    D[j + 1][j + 1] = d * rn;
-                }
-            } else if ((tid >> 5) & 3) {
-                // entries 1 .. E-1 of the active triangle (entry 0 is the next
-                // pivot), over warps 1-3 and 5-7
-                const int w = tid >> 5;
-                const int widx = (w - 1 - (w > 4 ? 1 : 0)) * 32 + (tid & 31);  // 0 .. 191
-                const int a = nb - 1 - j;
-                const int E = a * (a + 1) / 2;
-                for (int e = widx + 1; e < E; e += 192) {
-                    const int rc = tri[e];
-                    const int rr = j + 1 + (rc >> 8), cc = j + 1 + (rc & 255);
-                    D[rr][cc] = fma(-colj[rr], colj[cc], D[rr][cc]);
-                }
+        if (tid < CNB) {
+            const T d = raw[j];
+            if (pivot_ok<T>(d)) {
+                const T l = raw[tid] * rsqrt_pivot<T>(d);
+                colj[tid] = l;
+                Ls[tid][j] = l;  // row j: d / sqrt(d)
+            } else if (tid == 0) {
+                bad = j + 1;
             }
         }
+        __syncthreads();
+        if (bad) break;
+        const int E = (CNB - 1 - j) * (CNB - j) / 2;
+#pragma unroll
+        for (int u = NR - 1; u >= 0; --u)
+            if (256 * u < E) {
+                a[u] = fma(-colj[rr[u]], colj[cc[u]], a[u]);
+                if (cc[u] == j + 1) raw[rr[u]] = a[u];
+            }
         __syncthreads();
     }
     if (bad) {
@@ -231,7 +211,7 @@ __global__ void __launch_bounds__(256) k_potrf_diag(T* __restrict__ G, int64_t l
     }
     for (int q = tid; q < CNB * CNB; q += 256) {
         const int r = q & 63, c = q >> 6;
-        if (r < nb && c < nb) G[(k0 + r) + (k0 + c) * ld] = r >= c ? D[r][c] : (T)0;
+        if (r < nb && c < nb) G[(k0 + r) + (k0 + c) * ld] = r >= c ? Ls[r][c] : (T)0;
     }
 }
 

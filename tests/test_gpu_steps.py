@@ -257,6 +257,28 @@ def test_cholesky_solve(n):
     assert np.linalg.norm(to_np(x) - y_o) / np.linalg.norm(y_o) <= 8 * n * U64 * kG * O.kappa(R)
 
 
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 63, 64, 65, 127])
+def test_cholesky_diagonal_block(n):
+    """Orders around the 64-column block: against the oracle within the bound of
+    test_cholesky_solve; a power of 4 in the matrix is the power of 2 in the
+    factor, exactly, over the exponent range; every failing pivot is reported."""
+    rng = np.random.default_rng(90 + n)
+    X = rng.standard_normal((2 * n + 5, n))
+    G = X.T @ X
+    c = torch.zeros(n, dtype=torch.float64, device="cuda")
+    L_o, _ = O.cholesky(G)
+    F = to_np(lsq.factor_solve(dev_colmajor(G), c)[1])
+    assert np.linalg.norm(F - L_o) / np.linalg.norm(L_o) <= 8 * n * U64 * O.kappa(G)
+    for k in (-240, -17, 3, 250):
+        Fk = to_np(lsq.factor_solve(dev_colmajor(G * 4.0**k), c)[1])
+        np.testing.assert_array_equal(Fk, F * 2.0**k)
+    for p in sorted({0, n // 3, n // 2, n - 1}):
+        for v in (-1.0, np.inf):
+            B = G.copy()
+            B[p, p] = v
+            assert int(to_np(lsq.factor_solve(dev_colmajor(B), c)[3])[0]) == O.cholesky(B)[1] == p + 1
+
+
 @pytest.mark.parametrize("n", [255, 256, 257, 320, 321, 577, 2100])
 def test_cholesky_blocks(n):
     """Sizes around the 256-column blocks (inner updates of up to 192 columns,
