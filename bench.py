@@ -400,7 +400,8 @@ def roofline(stages, recs, per_solve_stage_ms, step_mix):
         emul, bound, unit_peak = work / (w36 / 36.0 + w21 / 21.0), "tensor", peak
         kname = "k_ot_update (FP64 products by BF16 digit slicing: TRSM updates, Cholesky updates, FP64 sketch)"
     elif top == "k_sketch_tc":
-        # FP32 sketches: six BF16 piece products per FP32 product
+        # FP32 sketches: three FP16 piece products per FP32 product (six of BF16
+        # pieces below 16384 rows)
         emul, bound, unit_peak = step_mix.get("sketch_emulation", 1.0), "tensor", peak
         kname = "k_sketch_tc (Gaussian sketch GEMM on tcgen05)"
     else:
@@ -762,7 +763,7 @@ def main():
         per_kernel = {k: {"ms_per_solve": round(v[0] / args.steps, 3), "launches_per_solve": v[1] / args.steps}
                       for k, v in stages.items() if v[1] and k.startswith("k_")}
         n32 = sum(1 for v in chosen.values() if v["prec"] == lsq.FP32)
-        mix = {"sketch_emulation": 6.0 if n32 == len(chosen) else 1.0}
+        mix = {"sketch_emulation": (3.0 if M >= 16384 else 6.0) if n32 == len(chosen) else 1.0}
         roof = roofline(stages, None, per_stage, mix)
         if roof is not None:
             roof["share_of_timed_region"] = stages[next(k for k in ("k_ot_update", "k_qr_panel", "k_sketch_tc")
