@@ -255,8 +255,7 @@ __device__ __forceinline__ double qr_rcp(double d) {
     return ed < 1021 ? __longlong_as_double(__double_as_longlong(y) - ((long long)ed << 52)) : 1.0 / d;
 }
 
-// QCL: CTAs per cluster (16, non-portable, where the device allows it; else
-// 8).  Dynamic shared memory: the local panel (Rp x QNB) and, in the fused
+// QCL: CTAs per cluster (1 to 16; 16 is non-portable, else 8).  Dynamic shared memory: the local panel (Rp x QNB) and, in the fused
 // form, the previous panel's reflector rows and the partial products behind it.
 template <typename T, int QCL>
 __global__ void __launch_bounds__(QCT)
@@ -1206,19 +1205,42 @@ struct QrCluster {
     bool fused = false;  // each panel applies the previous panel's update to its own columns
 };
 
-// 16 CTAs per cluster where the device can schedule that with the panel's
-// shared memory (non-portable size), else 8; 0 if neither fits (the
-// single-CTA panel kernel then runs).  The fused form (each panel applies the
-// previous panel's update to its own columns) is preferred where its shared
-// memory fits.  Decided once per precision and size.
+// The panel kernel of a cluster size.
+template <typename T>
+static auto qr_panel_kernel(int qcl) {
+    if constexpr (std::is_same<T, float>::value) {
+        switch (qcl) {
+        case 1: return k_qr_panel_cl<T, 1>;
+        case 2: return k_qr_panel_cl<T, 2>;
+        case 4: return k_qr_panel_cl<T, 4>;
+        default: break;
+        }
+    }
+    return qcl == 16 ? k_qr_panel_cl<T, 16> : k_qr_panel_cl<T, 8>;
+}
+
+// CTAs per cluster.  FP32: the fewest that leave a CTA at most 64 rows (8 a
+// warp), and 16 beyond 512.  A column costs an exchange whose price grows with
+// the cluster while the rows of a small sketch are little work: with 16 CTAs
+// whatever the size a 1000 x 100 solve took 685 us, 660 with at most 128 rows a
+// CTA and 654 with 64.  FP64, whose pipe bounds a CTA: 16.  16 CTAs where the
+// device can schedule that with the panel's shared memory (non-portable size),
+// else 8; 0 if neither fits (the single-CTA panel kernel then runs).  The fused
+// form (each panel applies the previous panel's update to its own columns) is
+// preferred where its shared memory fits.  Decided once per precision and size.
 template <typename T>
 static QrCluster qr_cluster_query(int64_t s) {
     const size_t lim = 200 * 1024;
-    for (bool fused : {true, false})
-        for (int qcl : {16, 8}) {
+    const int64_t rows_per_cta = 64;
+    for (bool fused : {true, false}) {
+        bool tried16 = false;
+        for (int qcl : {1, 2, 4, 8, 16, 8}) {
+            // ascending while too many rows per CTA; the last 8 is the fallback for 16
+            if (qcl < 16 && !tried16 && (sizeof(T) == 8 || ceil_div(s, qcl) > rows_per_cta)) continue;
+            tried16 = tried16 || qcl == 16;
             const size_t sm = qr_cluster_smem<T>(s, qcl, fused);
             if (sm > lim) continue;
-            auto kern = qcl == 16 ? k_qr_panel_cl<T, 16> : k_qr_panel_cl<T, 8>;
+            auto kern = qr_panel_kernel<T>(qcl);
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
                 (qcl > 8 &&
                  cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
@@ -1245,6 +1267,7 @@ static QrCluster qr_cluster_query(int64_t s) {
             }
             cudaGetLastError();
         }
+    }
     return QrCluster();
 }
 
@@ -1268,7 +1291,7 @@ static QrCluster qr_cluster_size(int64_t s) {
 template <typename T>
 static cudaError_t qr_launch_cluster(int qcl, size_t smem, cudaStream_t st, T* W, int64_t s, int64_t k0, int nb,
                                      T* beta, T* Tm, T* V, int64_t rows, const T* Vp, int64_t ldvp, const T* Tp) {
-    auto kern = qcl == 16 ? k_qr_panel_cl<T, 16> : k_qr_panel_cl<T, 8>;
+    auto kern = qr_panel_kernel<T>(qcl);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

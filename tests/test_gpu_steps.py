@@ -191,6 +191,34 @@ def test_precond_qr_fp64_rows_per_lane(s, n):
     assert err.max() <= 20 * n * U64 * O.kappa(B), err.max()
 
 
+@pytest.mark.parametrize("s,n", [(64, 40), (65, 33), (128, 64), (129, 40), (257, 70), (513, 40), (1030, 33), (2500, 40),
+                                 (4200, 40), (8192, 33), (8300, 40)])
+def test_precond_qr_fp32_rows_and_clusters(s, n):
+    """FP32 panels over every cluster size and row count per warp (and more rows
+    than the registers hold): the bound of test_precond_qr_fp64_rows_per_lane
+    with FP32's unit, columns graded over 2^+-30; and an upper triangular input
+    comes back with its rows' signs made positive, exactly."""
+    rng = np.random.default_rng(5 * s + n)
+    B = rng.standard_normal((s, n))
+    B[0] += 3.0 * np.where(np.arange(n) % 2, 1.0, -1.0)
+    As = O.round_to(np.asfortranarray(B * np.exp2(rng.integers(-30, 31, n))[None, :]), O.FP32).reshape((s, n), order="F")
+
+    def qr(M):
+        R, info = lsq.precond_qr(torch.from_numpy(np.ascontiguousarray(M.T)).cuda().float().t(), None, O.FP32)
+        assert int(to_np(info)[0]) == 0
+        return to_np(R)
+
+    R = qr(As)
+    assert np.all(np.diag(R) > 0)
+    Ro = np.linalg.qr(As, mode="r")
+    Ro *= np.sign(np.diag(Ro))[:, None]
+    err = np.linalg.norm(R - Ro, axis=0) / np.linalg.norm(Ro, axis=0)
+    assert err.max() <= 20 * n * U32 * O.kappa(B), err.max()
+    T = np.zeros((s, n))
+    T[:n] = np.triu(As[:n])
+    np.testing.assert_array_equal(qr(T), T[:n] * np.sign(np.diag(T))[:, None])
+
+
 def test_precond_qr_fp64_triangular_input():
     """Columns that are zero below the diagonal already (sigma = 0) with
     diagonal entries of either sign: R is the input with its rows' signs
