@@ -182,6 +182,18 @@ constexpr int QKG = QCT / 64;  // row groups of the previous-panel product (64 t
 constexpr int QRC = 32;   // panel rows per warp kept in registers, FP64
 constexpr int QRC32 = 64;  // FP32
 
+// The register forms keep u = [v1; x] unscaled: w_c / v1 and the products
+// u_i^T u_j stay in range while |v1| lies within 2^+-400, FP32 2^+-45 (columns
+// whose squares are in range have norms between about 2^-538 and 2^512, FP32
+// 2^-74 and 2^64).  Outside, a column's u is scaled by 1 / v1 before it is used.
+// On the exponent field: an FP64 comparison costs a warp 64 cycles.
+__device__ __forceinline__ bool qr_far(double av) {
+    return (unsigned)(((int)(__double_as_longlong(av) >> 52) & 0x7ff) - (1023 - 400)) > 800u;
+}
+__device__ __forceinline__ bool qr_far(float av) {
+    return (unsigned)((int)(__float_as_uint(av) >> 23 & 0xff) - (127 - 45)) > 90u;
+}
+
 // 4 consecutive values from 16-byte aligned shared memory
 __device__ __forceinline__ void load4(const float* p, float (&o)[4]) {
     const float4 v = *(const float4*)p;
@@ -496,9 +508,10 @@ __global__ void __launch_bounds__(QCT)
     // scalars, w_c for each column and (rank 0) column jj - 1 of Y.
     struct Scal {
         T mu, b, v1, rv1, wc;  // R's diagonal entry, beta, v's leading entry before scaling, its reciprocal, w_c
-        T f;                   // w_c / v1 (register forms)
+        T f;                   // w_c / v1 (register forms), w_c when far
         T rc;                  // FP32 register form: R[jj][c]
         bool scale;
+        bool far;              // register forms: u is scaled by 1 / v1 (qr_far)
     };
     // FP64: the sign of v1 is that of x1 (no cancellation, no case distinction;
     // R's diagonal entry is then -sign(x1) mu, and k_qr_extract makes the
@@ -518,6 +531,7 @@ __global__ void __launch_bounds__(QCT)
         sc.v1 = (T)1;
         sc.rv1 = (T)1;
         sc.wc = sc.f = (T)0;
+        sc.far = false;
         if (sc.scale) {
             const T y = (T)qr_rsqrt((double)s2);
             T mu = s2 * y;
@@ -527,6 +541,7 @@ __global__ void __launch_bounds__(QCT)
             sc.v1 = x1 < (T)0 ? -av : av;
             sc.rv1 = x1 < (T)0 ? -r : r;
             sc.mu = x1 < (T)0 ? mu : -mu;
+            sc.far = qr_far(av);
             // tau = 2 / u^T u = 1 / (mu |v1|) and beta = |v1| / mu, each corrected
             // once: their errors are common to all rows, so that they would
             // show in R's where those of single entries average out
@@ -537,8 +552,8 @@ __global__ void __launch_bounds__(QCT)
             sc.b = bt;
             if (lane > jj && lane < nb) {
                 const T ac = all_row[buf][lane];
-                sc.f = tau * fma(sc.v1, ac, dsum);
                 sc.wc = bt * fma(dsum, sc.rv1, ac);
+                sc.f = sc.far ? sc.wc : tau * fma(sc.v1, ac, dsum);
             }
         }
         if (rank == 0 && warp == 0 && lane + 1 < jj) Ysm[lane][jj - 1] = dsum;
@@ -559,6 +574,7 @@ __global__ void __launch_bounds__(QCT)
         sc.v1 = (T)1;
         sc.rv1 = (T)1;
         sc.wc = sc.f = (T)0;
+        sc.far = false;
         if (sc.scale) {
             // beta = 2 / v^T v from 1 / v1 as it is used: its error is common to
             // all rows and would show in R
@@ -567,9 +583,10 @@ __global__ void __launch_bounds__(QCT)
             sc.v1 = x1 < (T)0 ? -av : av;
             sc.rv1 = x1 < (T)0 ? -rv : rv;
             sc.mu = x1 < (T)0 ? mu : -mu;
+            sc.far = qr_far(av);
             if (lane > jj && lane < nb) {
                 sc.wc = sc.b * fma(dsum, sc.rv1, ac);
-                sc.f = sc.wc * sc.rv1;
+                sc.f = sc.far ? sc.wc : sc.wc * sc.rv1;
                 sc.rc = ac - sc.wc;
             }
         }
@@ -586,7 +603,7 @@ __global__ void __launch_bounds__(QCT)
         const T x1 = all_row[buf][jj];
         sc.v1 = (T)1;
         sc.rv1 = (T)1;
-        sc.scale = false;
+        sc.scale = sc.far = false;
         if (sigma == (T)0) {
             sc.mu = fabs(x1);
             sc.b = x1 >= (T)0 ? (T)0 : (T)2;
@@ -635,7 +652,7 @@ __global__ void __launch_bounds__(QCT)
                     scal_sh[1] = sc.b;
                     scal_sh[2] = sc.v1;
                     scal_sh[3] = sc.rv1;
-                    scale_sh = sc.scale ? 1 : 0;
+                    scale_sh = (sc.scale ? 1 : 0) | (sc.far ? 2 : 0);
                 }
                 wc_sh[lane] = sc.wc;
                 f_sh[lane] = sc.f;
@@ -645,7 +662,8 @@ __global__ void __launch_bounds__(QCT)
             sc.b = scal_sh[1];
             sc.v1 = scal_sh[2];
             sc.rv1 = scal_sh[3];
-            sc.scale = scale_sh != 0;
+            sc.scale = (scale_sh & 1) != 0;
+            sc.far = (scale_sh & 2) != 0;
             sc.wc = wc_sh[lane];
             sc.f = f_sh[lane];
             return sc;
@@ -721,11 +739,15 @@ __global__ void __launch_bounds__(QCT)
                     const int gr = gr0 + q;
                     u[q] = (gr < jj || q >= nv) ? (T)0 : (gr == jj ? sc.v1 : x);
                 }
+                if (sc.far) {
+#pragma unroll
+                    for (int q = 0; q < QR; ++q) u[q] *= sc.rv1;
+                }
                 if (lane == jj) {
                     myscale = sc.rv1;
                     myR = sc.mu;
                 }
-                rprev = sc.rv1;
+                rprev = sc.far ? (T)1 : sc.rv1;
                 // later columns: a_c -= w_c v = (w_c / v1) u
                 const bool upd = lane > jj && lane < nb && sc.b != (T)0;
                 const T f = sc.f;
@@ -833,11 +855,15 @@ __global__ void __launch_bounds__(QCT)
                     if (lane == 0) u[jj - gr0] = sc.v1;
                     __syncwarp();
                 }
+                if (sc.far) {
+                    for (int q = lane; q < QR; q += 32) u[q] *= sc.rv1;
+                    __syncwarp();
+                }
                 if (lane == jj) {
                     myscale = sc.rv1;
                     myR = sc.mu;
                 }
-                rprev = sc.rv1;
+                rprev = sc.far ? (T)1 : sc.rv1;
                 if (lane > jj && lane < nb && sc.b != (T)0) {
                     const T f = sc.f;
 #pragma unroll

@@ -219,6 +219,35 @@ def test_precond_qr_fp32_rows_and_clusters(s, n):
     np.testing.assert_array_equal(qr(T), T[:n] * np.sign(np.diag(T))[:, None])
 
 
+@pytest.mark.parametrize("s,n", [(200, 40), (1300, 70), (3000, 300)])
+@pytest.mark.parametrize("prec,lo,hi", [(O.FP64, -516, -516), (O.FP64, -516, 0), (O.FP64, -500, 500), (O.FP64, 480, 480),
+                                        (O.FP32, -64, -64), (O.FP32, -66, 63), (O.FP32, 60, 60)])
+def test_precond_qr_extreme_column_norms(prec, lo, hi, s, n):
+    """Columns with norms of 2^lo and 2^hi in turn, up to where their squares
+    leave the normal range: finite, and columnwise within the bound of
+    test_precond_qr_fp64_rows_per_lane, the unit enlarged by the rounding of a
+    squared norm of s terms on the subnormal grid (2^-1074, FP32 2^-149)."""
+    rng = np.random.default_rng(11 * s + n)
+    B = rng.standard_normal((s, n))
+    B[0] += 3.0 * np.sqrt(s) * np.where(np.arange(n) % 2, 1.0, -1.0)
+    B /= np.linalg.norm(B, axis=0)
+    e = np.where(np.arange(n) % 2, hi, lo).astype(float)
+    As = B * np.exp2(e)
+    u, grid = (U64, -1074) if prec == O.FP64 else (U32, -149)
+    if prec == O.FP32:
+        As = As.astype(np.float32).astype(np.float64)
+    t = torch.from_numpy(np.ascontiguousarray(As.T)).cuda()
+    R, info = lsq.precond_qr((t if prec == O.FP64 else t.float()).t(), None, prec)
+    R = to_np(R)
+    assert int(to_np(info)[0]) == 0 and np.isfinite(R).all() and np.all(np.diag(R) > 0)
+    Bs = As * np.exp2(-e)
+    Ro = np.linalg.qr(Bs, mode="r")
+    Ro *= np.sign(np.diag(Ro))[:, None]
+    err = np.linalg.norm(R * np.exp2(-e) - Ro, axis=0) / np.linalg.norm(Ro, axis=0)
+    unit = u + s * 2.0 ** (grid - 2 * min(lo, hi))
+    assert err.max() <= 20 * n * unit * O.kappa(Bs), err.max()
+
+
 def test_precond_qr_fp64_triangular_input():
     """Columns that are zero below the diagonal already (sigma = 0) with
     diagonal entries of either sign: R is the input with its rows' signs
