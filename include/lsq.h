@@ -360,15 +360,14 @@ lsq_status lsq_tc_gemm(int32_t prec, const void* X, int64_t ldx, const void* Y, 
                        int64_t K, float* C, int64_t ldc, int32_t* info, void* ws, size_t ws_bytes, void* stream);
 
 /* FP64 Gram G = X^T X (the left-hand side of Eq. e_pne with X = A_p) on the
- * FP8 tensor cores: every column p of X (m x n, ld) is written as 11
+ * FP8 tensor cores: every column p of X (m x n, ld) is written as 12
  * balanced base-32 digits in [-16, 16] relative to 2^(e_p) > max_i |x_ip|
- * (rounded to 2^(e_p - 54), with integer operations); the digit-pair products
- * t + u <= 10
- * are exact integer sums in the FP32 accumulators (K chunks of 65536 rows)
- * and are combined in FP64 smallest weight first, then scaled by
- * 2^(e_p + e_q).  Per entry the error is below ~2^-55 m max|x_p| max|x_q|,
- * the order of FP64 rounding.  G: n x n FP64, full symmetric, ld ldg.
- * Workspace lsq_gram_tc_workspace_size(m, n) (about 11 m n bytes of digits
+ * (rounded to 2^(e_p - 59), with integer operations); the digit-pair products
+ * t + u <= 11 are exact integer sums in the FP32 accumulators (K chunks of
+ * 65536 rows), combined exactly in integers, scaled by 2^(e_p + e_q) and rounded
+ * once.  Beside that rounding the error of an entry is below 2^-54 m max|x_p|
+ * max|x_q|, whatever the values.  G: n x n FP64, full symmetric, ld ldg.
+ * Workspace lsq_gram_tc_workspace_size(m, n) (about 12 m n bytes of digits
  * plus 64 KiB per digit tile).  info (device, may be NULL): -2 on a pipeline
  * timeout. */
 size_t lsq_gram_tc_workspace_size(int64_t m, int64_t n);
@@ -377,10 +376,10 @@ lsq_status lsq_gram_tc(const double* X, int64_t m, int64_t n, int64_t ld, double
 
 /* G = X^T Y (n x n, FP64 accuracy) for two m x n column-major FP64 matrices,
  * by the same FP8 digit slicing as lsq_gram_tc with one exponent per column
- * of X and of Y; the HPNE matrix A_p^T A (Eq. e_hpne).  All 66 digit-pair
- * blocks are formed (no symmetry).  Per entry the error is below ~2^-55 m
- * max|x_p| max|y_q|.  Workspace lsq_gemm_tn_tc_workspace_size(m, n) (about
- * 22 m n bytes of digits plus 64 KiB per digit tile).  info (device, may be
+ * of X and of Y; the HPNE matrix A_p^T A (Eq. e_hpne).  All 78 digit-pair
+ * blocks are formed (no symmetry).  Beside its rounding the error of an entry
+ * is below 2^-54 m max|x_p| max|y_q|.  Workspace lsq_gemm_tn_tc_workspace_size(m, n) (about
+ * 24 m n bytes of digits plus 64 KiB per digit tile).  info (device, may be
  * NULL): -2 on a pipeline timeout. */
 size_t lsq_gemm_tn_tc_workspace_size(int64_t m, int64_t n);
 lsq_status lsq_gemm_tn_tc(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t n,

@@ -1,29 +1,32 @@
 // FP64 Gram matrix G = X^T X (and the product X^T Y of two m x n matrices)
-// on the FP8 tensor cores, exact to a 54-bit plus sign
+// on the FP8 tensor cores, exact to a 59-bit plus sign
 // fixed-point representation of every column (digit slicing in the manner
 // of Ozaki, Ogita & Oishi's error-free matrix multiplication):
 //
 //   x_ip = 2^(e_p - 4) * sum_{t=0}^{S-1} d_t(i,p) 32^-t + r_ip,
-//          d_t in [-16, 16], |r_ip| <= 2^(e_p - 55)   (S = 11 digits),
+//          d_t in [-16, 16], |r_ip| <= 2^(e_p - 60)   (S = 12 digits),
 //
 // where 2^(e_p) bounds column p.  Digit products are integers up to 2^8, so
 // a K-chunk of up to 65536 rows sums exactly in the FP32 accumulators of
 // tcgen05.mma (kind::f8f6f4, E4M3 operands).  Every digit-pair block (t, u)
 // with t + u <= S - 1 is one tensor-core contraction over the rows; the
 // blocks are combined exactly in integers, scaled by 2^(e_p + e_q) and
-// rounded once.  Dropped pairs and the residuals r contribute about 2^-55 of
-// 2^(e_p + e_q) per row, with signs that vary from row to row, the same order
-// as FP64 rounding.
+// rounded once.  The dropped pairs weigh at most 2^-60 of 2^(e_p + e_q) each (11
+// with t + u = 12, 10 more at 2^-65, ...) and the residuals 2^-60 each: below
+// 2^-56.2 of 2^(e_p + e_q) a row, whatever the values.
 //
-// Why balanced digits: E4M3 holds every integer up to 16, so a signed digit
-// carries 5 bits, against 4 for a sign and a nibble, and 66 digit pairs take
-// the place of the 105 of 14 sign-and-magnitude digits (the tensor work is
-// what bounds the Gram).  The error is no larger: against
-// quadruple precision, relative to |x_p| |x_q|, 60000 normal rows: rms 2^-57.2
-// off the diagonal and 2^-53.5 on it, against 2^-56.4 and 2^-48.5 with the
-// 14 digits (whose dropped pairs all have the sign of x_ip x_iq).  Measured: A_p and Gram of a
-// 131072 x 2000 problem 58.3 -> 51.7 ms (digit products 16.7 -> 10.5 ms), a
-// 262144 x 4096 solve 556 -> 501 ms.
+// Why balanced digits, and 12: E4M3 holds every integer up to 16, so a signed
+// digit carries 5 bits, against 4 for a sign and a nibble, and 78 digit pairs
+// take the place of the 105 of 14 sign-and-magnitude digits (the tensor work is
+// what bounds the Gram).  11 digits and 66 pairs would be as accurate on random
+// data, but drop up to 2^-51.6 a row, and in columns of equal entries every row
+// drops the same: 2^-53.0 a row for columns of 0.7, where 14 digits lose 2^-57.4
+// and 12 2^-57.4 (the entry's own rounding).  Error against quadruple precision
+// relative to |x_p| |x_q|, 60000 normal rows, off the diagonal / on it: 2^-61.1 /
+// 2^-54.2, 14 digits 2^-56.3 / 2^-48.4.  Measured: A_p and Gram of a
+// 131072 x 2000 problem 58.3 -> 51.7 ms and a 262144 x 4096 solve 556 -> 501 ms from
+// 14 to 11 digits, 42.1 -> 44.2 and 377 -> 395 ms (other kernels faster by then) from
+// 11 to 12.
 //
 // Digits are extracted with integer operations on the FP64 bit pattern (no
 // FP64 instruction in the slicing pass).
@@ -34,7 +37,7 @@
 
 namespace lsq {
 
-constexpr int OZ_S = 11;        // digits per value
+constexpr int OZ_S = 12;        // digits per value
 constexpr int OZ_B = 5;         // bits per digit: balanced base-32 digits in [-16, 16]
 constexpr int OZ_F = OZ_B * (OZ_S - 1) + 4;  // fraction bits of a value relative to 2^(e_p)
 constexpr int64_t OZ_KCHUNK = 65536;  // rows summed exactly per FP32 accumulator
@@ -89,7 +92,7 @@ constexpr unsigned long long oz_bias() {
 // columns i >= m (padding) are zero.  4 consecutive rows per thread: a warp
 // reads 1 KB of a column and writes 128 contiguous bytes of every digit
 // plane.  V = |x| 2^(F - e_p) rounded to the nearest integer (V <= 2^F); field
-// t of W = V + bias is the digit of |x| plus 16 (the top field, W >> 50, is
+// t of W = V + bias is the digit of |x| plus 16 (the top field, W >> 55, is
 // the digit itself), and the signed digit is s (2^23 1.5 + field) -
 // s (2^23 1.5 + 16) with s = +-1 (exact in FP32, +0 for a zero digit), converted
 // in pairs by the hardware.  The digits are those of |x| times the sign, not
@@ -116,7 +119,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double* __restrict__ X, 
             if (Eb != 0 && Eb != 0x7ff && ep != OZ_NONFINITE) {
                 const unsigned long long sig = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
                 const int sh = (Eb - 1023) - ep + (OZ_F - 52);  // x 2^(F - e_p) = sig 2^(E_a - 52 + F - e_p)
-                if (sh >= 0) V = sig << sh;                     // sh <= 1: V < 2^F
+                if (sh >= 0) V = sig << sh;                     // sh <= 6: V < 2^F
                 else if (sh > -64) V = (sig + (1ull << (-sh - 1))) >> (-sh);
             }
             W[q] = V + BIAS;

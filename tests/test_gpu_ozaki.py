@@ -109,6 +109,30 @@ def test_within_fp64_error_order(m, n, spread):
     np.testing.assert_array_equal(G, G.T)
 
 
+@pytest.mark.parametrize("m", [1000, 100001])
+def test_equal_entries_stay_within_the_bound(m):
+    """Columns of equal entries (or of two values in turn): every row drops the
+    same digit pairs, so nothing averages out.  The bound of the scheme holds
+    for any values: 2^-54 m max|x_p| max|x_q| (twelve digits, pairs t + u > 11
+    dropped: below 13.4 2^-60 2^(e_p + e_q) a row) and the rounding of the entry."""
+    low = float(sum(Fraction(d, 16 * 32 ** t) for t, d in enumerate([9] + [-16] * 10)))  # 0.53, all digits large
+    vals = [low, 0.7, 1 / 3, 0.1, np.pi / 4, 1 - 2.0 ** -53, 1.0]
+    X = np.empty((m, len(vals) + 1))
+    X[:, :-1] = vals
+    X[:, -1] = np.where(np.arange(m) % 2, 0.9, -0.3)
+    Y = X[:, ::-1].copy()
+    G = gram_tc(X)
+    Gxy, info = lsq.gemm_tn_tc(dev_colmajor(X), dev_colmajor(Y))
+    assert int(to_np(info)[0]) == 0
+    for got, Z in ((G, X), (to_np(Gxy), Y)):
+        for p in range(X.shape[1]):
+            for q in range(X.shape[1]):
+                a, b = Fraction(X[0, p]) * Fraction(Z[0, q]), Fraction(X[1, p]) * Fraction(Z[1, q])
+                ex = a * ((m + 1) // 2) + b * (m // 2)
+                tol = Fraction(m * np.abs(X[:2, p]).max() * np.abs(Z[:2, q]).max()) / 2 ** 54 + abs(ex) / 2 ** 53
+                assert abs(Fraction(float(got[p, q])) - ex) <= tol, (p, q, float(abs(Fraction(float(got[p, q])) - ex) / tol))
+
+
 @pytest.mark.parametrize("m,n", [(3000, 200), (70000, 130), (1000, 1)])
 def test_gemm_tn_exact_on_integer_data(m, n):
     rng = np.random.default_rng(m + 3 * n)
