@@ -283,7 +283,7 @@ lsq_status lsq_trsm_gram_noalloc(const double* A, int64_t m, int64_t n, int64_t 
  * synchronised through flags in the workspace; the Cholesky trailing
  * updates are FP64-accurate tensor-core products (as in lsq_trsm_tc) with
  * their digits in the workspace too.  Workspace:
- * lsq_workspace_size(LSQ_OP_FACTOR_SOLVE, m, n, NULL), about 2 n 256 x 16
+ * lsq_workspace_size(LSQ_OP_FACTOR_SOLVE, m, n, NULL), about 2 n 64 x 16
  * bytes (LSQ_ERR_NOMEM when smaller).  A wait that runs out (2 s) sets
  * info = -2. */
 lsq_status lsq_factor_solve(int32_t hpne, double* G, int64_t n, int64_t ldg, const double* c,

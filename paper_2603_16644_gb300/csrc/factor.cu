@@ -22,7 +22,6 @@
 namespace lsq {
 
 constexpr int CNB = 64;   // Cholesky block
-constexpr int CBB = 256;  // Cholesky blocks whose trailing update is one product
 constexpr int LNB = 32;   // LU panel width
 
 // ---------------------------------------------------------------------------
@@ -264,60 +263,39 @@ __global__ void k_zero_upper(T* __restrict__ G, int64_t n, int64_t ld, const int
     }
 }
 
-// Scratch of the digit-sliced products: an inner update (n - 64 rows, up to 192
-// columns, K = 64) and a trailing one (K = 256).
-size_t cholesky_ws_bytes(int64_t n) {
-    if (n <= CNB) return 256;
-    size_t b = ot_update_ws_bytes(n - CNB, std::min<int64_t>(n, CBB) - CNB, CNB);
-    if (n > CBB) b = std::max(b, ot_update_ws_bytes(n - CBB, n - CBB, CBB));
-    return b;
-}
+size_t cholesky_ws_bytes(int64_t n) { return n > CNB ? ot_update_ws_bytes(n - CNB, n - CNB, CNB) : 256; }
 
-// FP64 with scratch: 64-column steps inside blocks of 256, the later columns of
-// the block updated after each step and everything right of the block once, with
-// K = 256 and only the tiles that reach the lower triangle (the rest of the
-// upper triangle keeps its old values until it is cleared).  One K = 64 update
-// of the whole trailing matrix per step was bound by its epilogue (8 bytes
-// converted, read and written per output for 64 products): 6.3 of the 12.4 ms
-// of a factorization and solve of order 4096; 8.9 ms in this form.
+// Right-looking in steps of 64 columns.  FP64 with scratch: each step's product is
+// digit-sliced, over the tiles that reach the lower triangle (the rest of the
+// upper triangle keeps its old values until it is cleared); its epilogue bounds
+// it (8 bytes converted, read and written per output for 64 products).  One
+// product with K = 256 per four steps takes 0.7 ms off the 9.3 ms of a
+// factorization and solve of order 4096, but its one exponent per row covers 256
+// columns of L: with L's 64-column pieces graded by 2^20 the residual of G - L L^T
+// relative to |L| |L|^T grew from 1.2e-15 to 1.4e-11.
 template <typename T>
 lsq_status launch_cholesky(T* G, int64_t n, int64_t ld, int32_t* info, cudaStream_t st, void* ws, size_t ws_bytes) {
     const bool tc = std::is_same<T, double>::value && ws && ws_bytes >= cholesky_ws_bytes(n) && ot_trsm_supported();
-    const int64_t bb = tc ? CBB : CNB;
-    for (int64_t j0 = 0; j0 < n; j0 += bb) {
-        const int64_t j1 = std::min<int64_t>(n, j0 + bb);
-        for (int64_t k0 = j0; k0 < j1; k0 += CNB) {
-            const int nb = (int)std::min<int64_t>(CNB, n - k0);
-            k_potrf_diag<T><<<1, 256, 0, st>>>(G, ld, n, k0, info);
-            LSQ_LAUNCH_CHECK();
-            const int64_t rest = n - k0 - nb;
-            if (rest <= 0) break;
-            k_potrf_panel<T><<<(unsigned)ceil_div(rest, 8), 128, 0, st>>>(G, ld, n, k0, info);
-            LSQ_LAUNCH_CHECK();
-            T* L21 = G + (k0 + nb) + k0 * ld;
-            T* A22 = G + (k0 + nb) + (k0 + nb) * ld;
-            lsq_status s = LSQ_OK;
-            if constexpr (std::is_same<T, double>::value) {
-                if (tc) {
-                    // the block's later columns, FP64 accuracy on the tensor cores
-                    const int64_t cols = j1 - k0 - nb;
-                    if (cols > 0) s = ot_gemm_update(L21, ld, L21, ld, 1, A22, ld, A22, ld, rest, cols, nb, ws, ws_bytes, nullptr, st);
-                    if (s != LSQ_OK) return s;
-                    continue;
-                }
-            }
-            s = rank_update_ext<T>(A22, ld, L21, 1, ld, L21, 1, ld, rest, rest, nb, true, info, st);
-            if (s != LSQ_OK) return s;
-        }
+    for (int64_t k0 = 0; k0 < n; k0 += CNB) {
+        const int nb = (int)std::min<int64_t>(CNB, n - k0);
+        k_potrf_diag<T><<<1, 256, 0, st>>>(G, ld, n, k0, info);
+        LSQ_LAUNCH_CHECK();
+        const int64_t rest = n - k0 - nb;
+        if (rest <= 0) break;
+        k_potrf_panel<T><<<(unsigned)ceil_div(rest, 8), 128, 0, st>>>(G, ld, n, k0, info);
+        LSQ_LAUNCH_CHECK();
+        T* L21 = G + (k0 + nb) + k0 * ld;
+        T* A22 = G + (k0 + nb) + (k0 + nb) * ld;
+        lsq_status s;
         if constexpr (std::is_same<T, double>::value) {
-            const int64_t rest = n - j1;
-            if (tc && rest > 0) {
-                double* L21 = G + j1 + j0 * ld;
-                double* A22 = G + j1 + j1 * ld;
-                lsq_status s = ot_gemm_update_lower(L21, ld, A22, ld, rest, j1 - j0, ws, ws_bytes, nullptr, st);
+            if (tc) {
+                s = ot_gemm_update_lower(L21, ld, A22, ld, rest, nb, ws, ws_bytes, nullptr, st);
                 if (s != LSQ_OK) return s;
+                continue;
             }
         }
+        s = rank_update_ext<T>(A22, ld, L21, 1, ld, L21, 1, ld, rest, rest, nb, true, info, st);
+        if (s != LSQ_OK) return s;
     }
     k_zero_upper<T><<<(unsigned)std::min<int64_t>(ceil_div(n * n, 256), 4096), 256, 0, st>>>(G, n, ld, info);
     LSQ_LAUNCH_CHECK();

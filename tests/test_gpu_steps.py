@@ -336,6 +336,30 @@ def test_cholesky_diagonal_block(n):
             assert int(to_np(lsq.factor_solve(dev_colmajor(B), c)[3])[0]) == O.cholesky(B)[1] == p + 1
 
 
+@pytest.mark.parametrize("n", [130, 330, 449])
+def test_cholesky_graded_pieces_componentwise(n):
+    """Rows whose 64-column pieces of L are graded over 2^30 independently: the
+    residual of every entry within (n + 1) u |L| |L|^T (the bound of Cholesky in
+    FP64, for the FP64 operations) plus the digit products' 64 2^-50.6 times the
+    two rows' largest entries, piece by piece, and a rounding of the entry."""
+    rng = np.random.default_rng(60 + n)
+    L0 = np.tril(rng.standard_normal((n, n)))
+    L0 *= np.repeat(np.exp2(-rng.uniform(0, 30, (n, (n + 63) // 64))), 64, axis=1)[:, :n]
+    L0[np.arange(n), np.arange(n)] = 2.0 * np.linalg.norm(np.tril(L0, -1), axis=1) + 2.0**-30
+    G = L0 @ L0.T
+    G = np.tril(G) + np.tril(G, -1).T
+    x, F, _, info = lsq.factor_solve(dev_colmajor(G), torch.ones(n, dtype=torch.float64, device="cuda"))
+    assert int(to_np(info)[0]) == 0
+    F = np.tril(to_np(F))
+    Fl = F.astype(np.longdouble)
+    res = np.abs(Fl @ Fl.T - G).astype(np.float64)
+    tol = (n + 1) * U64 * (np.abs(F) @ np.abs(F).T) + U64 * np.abs(G)
+    for k in range(0, n, 64):
+        mx = np.abs(F[:, k:k + 64]).max(axis=1)
+        tol += 64 * 2.0**-50.6 * np.outer(mx, mx)
+    assert np.all(res <= tol), (res / tol).max()
+
+
 @pytest.mark.parametrize("n", [255, 256, 257, 320, 321, 577, 2100])
 def test_cholesky_blocks(n):
     """Sizes around the 256-column blocks (inner updates of up to 192 columns,
