@@ -421,6 +421,12 @@ int32_t lsq_set_fp64_emulation(int32_t enable);
  * ns <= 0. */
 int64_t lsq_test_set_solve_wait_ns(int64_t ns);
 
+/* Test-only query (host arithmetic): how many products one FP32 accumulator of
+ * an m-row FP32 Gaussian sketch (s x n) sums before its partial sketch is
+ * written, on a device of `sms` SMs; 0 below the row count from which it is
+ * formed from FP16 pieces (three products a row). */
+int64_t lsq_test_sketch_chain(int64_t s, int64_t n, int64_t m, int32_t sms);
+
 /* ---- Batched solves (many independent problems of uneven shape) --------- */
 
 /* One problem of a batch: device pointers A (m x n, ld lda), b (m), x (n),

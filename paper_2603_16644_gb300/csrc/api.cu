@@ -151,9 +151,13 @@ bool gauss_fp64_tc(int prec) { return prec == LSQ_FP64 && g_fp64_emulation && ot
 // FP32 Gaussian sketches of at least this many rows take two FP16 pieces per
 // value (three products), shorter ones three BF16 pieces (six).  Relative error
 // of the sketch against 64 bits, FP16 / BF16 pieces: m = 1000 3.5e-7 / 2.3e-7,
-// 4000 4.2e-7 / 3.5e-7, 20000 2.8e-6 / 4.8e-6, 262144 1.5e-5 / 2.8e-5: the FP16
-// pieces represent a value a little less closely, and the accumulation of half
-// as many products is more accurate from about 10000 rows on.
+// 4000 4.2e-7 / 3.5e-7, 16384 (1000 columns) 6.8e-6 / 1.9e-5, 131072 7.3e-6 / 3.8e-5,
+// 262144 7.3e-6 / 3.8e-5: the FP16 pieces represent a value a little less closely
+// (to 2^-23 of it, or 2^-39 of its column's maximum), and the accumulation of
+// fewer products in shorter runs is what bounds the error from there on.  The
+// same with rows or entries spread over 2^30 and 2^40 and with a nonzero mean; in
+// a column that one row dominates, both are at 1e-7 to 3e-6 and within 25 % of each
+// other or better.
 constexpr int64_t kFp16PieceRows = 16384;
 bool gauss_fp32_f16(int64_t m) { return m >= kFp16PieceRows; }
 bool gauss_fp32_tc(int prec) { return prec == LSQ_FP32 && g_tensor_core_sketch && sketch_tc_supported(LSQ_BF16); }
@@ -773,6 +777,11 @@ int32_t lsq_set_tensor_core_sketch(int32_t enable) {
     int32_t prev = g_tensor_core_sketch ? 1 : 0;
     g_tensor_core_sketch = enable != 0;
     return prev;
+}
+
+int64_t lsq_test_sketch_chain(int64_t s, int64_t n, int64_t m, int32_t sms) {
+    if (s <= 0 || n <= 0 || m <= 0 || sms <= 0) return -1;
+    return gauss_fp32_f16(m) ? sketch_pieces_chain(s, n, m, sms) : 0;
 }
 
 int32_t lsq_profile(int32_t enable) {

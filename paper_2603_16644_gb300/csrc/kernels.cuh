@@ -126,6 +126,8 @@ lsq_status rank_update_ext(T* C, int64_t ldc, const T* P, int64_t psi, int64_t p
 // ---- sketch_tc.cu: tcgen05 Gaussian sketch for 8/16-bit u_p --------------
 bool sketch_tc_supported(int prec);
 size_t sketch_tc_ws_bytes(int64_t s, int64_t n, int64_t m, int prec, int sms, bool pieces = false);
+// Products summed by one FP32 accumulator of an FP32 sketch as FP16 pieces.
+int64_t sketch_pieces_chain(int64_t s, int64_t n, int64_t m, int sms);
 lsq_status launch_sketch_tc(const void* Om, int64_t ldo, const void* Ahat, int64_t ldq, int prec, int64_t s,
                             int64_t n, int64_t m, float* As, int64_t ldas, void* ws, size_t ws_bytes, int32_t* err,
                             cudaStream_t st, bool blocked = false, int64_t seg = 0, float oscale = 1.0f);

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     k_sketch_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t M, int64_t N,
                 int64_t K, int64_t kchunk, float* __restrict__ out, int64_t ldo, int64_t split_stride,
                 int32_t* __restrict__ err, const int2* __restrict__ tiles, int64_t ntiles, int blocked, int seg,
-                float oscale) {
+                float oscale, int64_t kfirst) {
     constexpr int ES = KIND == 2 ? 1 : 2;  // element bytes
     constexpr int BKE = 128 / ES;          // K elements per stage
     constexpr int ST = tc_stages(BN);
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int2 tl = tiles ? tiles[blockIdx.x] : make_int2(0, 0);
     const int64_t m0 = tiles ? (int64_t)tl.x : (int64_t)blockIdx.y * TC_BM;
     const int64_t n0 = tiles ? (int64_t)tl.y : (int64_t)blockIdx.x * BN;
-    const int64_t kb0 = (int64_t)blockIdx.z * kchunk;
+    const int64_t kb0 = kfirst + (int64_t)blockIdx.z * kchunk;
     const int64_t kb1 = min64(K, kb0 + kchunk);
     const int nk = (int)((kb1 - kb0 + BKE - 1) / BKE);
 
@@ -196,13 +196,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 }
 
+// The splits' sums added in order, onto C when `onto`.
 __global__ void k_reduce_f32(const float* __restrict__ part, int splits, int64_t M, int64_t N, float* __restrict__ C,
-                             int64_t ldc) {
+                             int64_t ldc, bool onto) {
     int64_t total = M * N;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
-        float s = 0.0f;
+        float* c = C + (q % M) + (q / M) * ldc;
+        float s = onto ? *c : 0.0f;
         for (int z = 0; z < splits; ++z) s += part[(int64_t)z * total + q];
-        C[(q % M) + (q / M) * ldc] = s;
+        *c = s;
     }
 }
 
@@ -279,25 +281,44 @@ static int tc_bn(int64_t N) { return N >= 256 ? 256 : TC_BN; }
 // (1.8 PFLOP/s of tensor work).  Shorter accumulation chains in the FP32
 // accumulators are also more accurate.
 constexpr int64_t TC_KBLOCKS_MAX = 512;
-// The FP16 pieces of an FP32 sketch: a quarter of that, so that the chain of the
-// full-size products is at most half the 16384 rows from which they are used (error of a
-// 16384 x 1000 sketch 1.93e-5 with 512, 1.86e-5 with the BF16 pieces).
-constexpr int64_t TC_KBLOCKS_PIECES = 128;
+// The FP16 pieces of an FP32 sketch: fewer, so that the chain of the full-size
+// products (6144 rows) is below half the 16384 rows from which they are used and
+// their sketch is the more accurate one also where a part of the rows carries all
+// the weight.  Error of a 16384 x 1000 sketch with 512 / 128 / 96 K blocks 1.93e-5 /
+// 9.7e-6 / 6.8e-6, six BF16 products 1.87e-5; with the second half of the rows
+// near zero 9.7e-6 (128) / 4.9e-6 (96), BF16 9.1e-6.  The limit holds at any number
+// of rows: splits beyond TC_SPLITS run in further launches, added onto the sketch
+// (262144 x 1024: 1.44e-5 in 64 splits, 7.3e-6 in two launches of 64; the
+// 262144 x 4096 solve takes the same time within its runs' spread).
+constexpr int64_t TC_KBLOCKS_PIECES = 96;
+constexpr int TC_SPLITS = 64;  // splits of a launch (partial sketches held) at most
 
 // Split count: fill the SMs when the tile grid is small, and at most
-// TC_KBLOCKS_MAX K blocks per split; at least 4 stages of K per split.
-static int tc_splits(int64_t M, int64_t N, int64_t K, int prec, int sms, int64_t kblocks_max = TC_KBLOCKS_MAX) {
+// TC_KBLOCKS_MAX K blocks per split; at least 4 stages of K per split; TC_SPLITS
+// at most.  pieces: TC_KBLOCKS_PIECES whatever the count.
+static int tc_splits(int64_t M, int64_t N, int64_t K, int prec, int sms, bool pieces) {
     int64_t tiles = ceil_div(M, TC_BM) * ceil_div(N, tc_bn(N));
     int64_t bke = prec == LSQ_FP8_E4M3 ? 128 : 64;
     int64_t kblocks = ceil_div(K, bke);
     int64_t want = std::max<int64_t>(1, sms / std::max<int64_t>(1, tiles));
-    want = std::max<int64_t>(want, ceil_div(kblocks, kblocks_max));
-    int64_t cap = std::max<int64_t>(1, kblocks / 4);
-    return (int)std::min<int64_t>(std::min<int64_t>(want, cap), 64);
+    want = std::max<int64_t>(want, ceil_div(kblocks, pieces ? TC_KBLOCKS_PIECES : TC_KBLOCKS_MAX));
+    want = std::min<int64_t>(want, std::max<int64_t>(1, kblocks / 4));
+    const int64_t limit = pieces ? std::max<int64_t>(TC_SPLITS, ceil_div(kblocks, TC_KBLOCKS_PIECES)) : TC_SPLITS;
+    return (int)std::min<int64_t>(want, limit);
+}
+
+// K per split.
+static int64_t tc_kchunk(int64_t M, int64_t N, int64_t K, int prec, int sms, bool pieces) {
+    const int64_t bke = prec == LSQ_FP8_E4M3 ? 128 : 64;
+    return ceil_div(ceil_div(K, tc_splits(M, N, K, prec, sms, pieces)), bke) * bke;
+}
+
+int64_t sketch_pieces_chain(int64_t s, int64_t n, int64_t m, int sms) {
+    return tc_kchunk(s, n, 3 * (int64_t)align_up((size_t)m, 64), LSQ_FP16, sms, true);
 }
 
 size_t sketch_tc_ws_bytes(int64_t s, int64_t n, int64_t m, int prec, int sms, bool pieces) {
-    int sp = tc_splits(s, n, m, prec, sms, pieces ? TC_KBLOCKS_PIECES : TC_KBLOCKS_MAX);
+    int sp = std::min(tc_splits(s, n, m, prec, sms, pieces), TC_SPLITS);
     return sp > 1 ? align_up(sizeof(float) * (size_t)sp * s * n, 256) : 0;
 }
 
@@ -316,39 +337,43 @@ lsq_status launch_sketch_tc(const void* Om, int64_t ldo, const void* Ahat, int64
     } else if (!make_map(&ta, Om, prec, m, s, ldo) || !make_map(&tb, Ahat, prec, m, n, ldq, bn)) {
         return LSQ_ERR_CUDA;
     }
-    int sms = device_sm_count();
-    int splits = tc_splits(s, n, m, prec, sms, seg ? TC_KBLOCKS_PIECES : TC_KBLOCKS_MAX);
-    int64_t bke = prec == LSQ_FP8_E4M3 ? 128 : 64;
-    int64_t kchunk = ceil_div(ceil_div(m, splits), bke) * bke;
-    splits = (int)ceil_div(m, kchunk);
+    const int64_t kchunk = tc_kchunk(s, n, m, prec, device_sm_count(), seg != 0);
+    const int splits = (int)ceil_div(m, kchunk);
+    // launches of about equal split counts, TC_SPLITS at most
+    const int launches = (int)ceil_div(splits, TC_SPLITS), per = (int)ceil_div(splits, launches);
     float* out = As;
     int64_t ldout = ldas, stride = 0;
     if (splits > 1) {
-        if (!ws || ws_bytes < sizeof(float) * (size_t)splits * s * n) return LSQ_ERR_NOMEM;
+        if (!ws || ws_bytes < sizeof(float) * (size_t)per * s * n) return LSQ_ERR_NOMEM;
         out = (float*)ws;
         ldout = s;
         stride = s * n;
     }
     size_t smem = 1024 + (size_t)tc_stages(bn) * (TC_TILE_BYTES + (size_t)bn * 128) + 256;
-    dim3 grid((unsigned)ceil_div(n, bn), (unsigned)ceil_div(s, TC_BM), (unsigned)splits);
-    stage_mark(ST_K_SKETCHTC, true, st);
-    auto go = [&](auto kern) -> lsq_status {
-        LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kern<<<grid, TC_THREADS, smem, st>>>(ta, tb, s, n, m, kchunk, out, ldout, stride, err, nullptr, 0,
-                                             blocked ? 1 : 0, (int)(seg / 64), oscale);
-        return LSQ_OK;
-    };
-    lsq_status lr;
-    if (prec == LSQ_BF16) lr = bn == 256 ? go(k_sketch_tc<0, 256>) : go(k_sketch_tc<0, TC_BN>);
-    else if (prec == LSQ_FP16) lr = bn == 256 ? go(k_sketch_tc<1, 256>) : go(k_sketch_tc<1, TC_BN>);
-    else lr = bn == 256 ? go(k_sketch_tc<2, 256>) : go(k_sketch_tc<2, TC_BN>);
-    if (lr != LSQ_OK) return lr;
-    LSQ_LAUNCH_CHECK();
-    stage_mark(ST_K_SKETCHTC, false, st, 2.0 * (double)s * (double)n * (double)m);
-    if (splits > 1) {
-        k_reduce_f32<<<(unsigned)std::min<int64_t>(ceil_div(s * n, 256), 8192), 256, 0, st>>>(out, splits, s, n, As,
-                                                                                            ldas);
+    for (int z0 = 0; z0 < splits; z0 += per) {
+        const int nz = std::min(per, splits - z0);
+        const int64_t kfirst = z0 * kchunk;
+        dim3 grid((unsigned)ceil_div(n, bn), (unsigned)ceil_div(s, TC_BM), (unsigned)nz);
+        stage_mark(ST_K_SKETCHTC, true, st);
+        auto go = [&](auto kern) -> lsq_status {
+            LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            kern<<<grid, TC_THREADS, smem, st>>>(ta, tb, s, n, m, kchunk, out, ldout, stride, err, nullptr, 0,
+                                                 blocked ? 1 : 0, (int)(seg / 64), oscale, kfirst);
+            return LSQ_OK;
+        };
+        lsq_status lr;
+        if (prec == LSQ_BF16) lr = bn == 256 ? go(k_sketch_tc<0, 256>) : go(k_sketch_tc<0, TC_BN>);
+        else if (prec == LSQ_FP16) lr = bn == 256 ? go(k_sketch_tc<1, 256>) : go(k_sketch_tc<1, TC_BN>);
+        else lr = bn == 256 ? go(k_sketch_tc<2, 256>) : go(k_sketch_tc<2, TC_BN>);
+        if (lr != LSQ_OK) return lr;
         LSQ_LAUNCH_CHECK();
+        const int64_t kz = std::min<int64_t>(m, kfirst + nz * kchunk) - kfirst;
+        stage_mark(ST_K_SKETCHTC, false, st, 2.0 * (double)s * (double)n * (double)kz);
+        if (splits > 1) {
+            k_reduce_f32<<<(unsigned)std::min<int64_t>(ceil_div(s * n, 256), 8192), 256, 0, st>>>(out, nz, s, n, As,
+                                                                                                ldas, z0 > 0);
+            LSQ_LAUNCH_CHECK();
+        }
     }
     return LSQ_OK;
 }
@@ -375,7 +400,7 @@ lsq_status launch_tc_tiles_fp8(const void* X, int64_t ldx, int64_t rowsX, const 
     LSQ_CUDA_TRY(cudaFuncSetAttribute(k_sketch_tc<2, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dim3 grid((unsigned)ntiles, 1, (unsigned)chunks);
     k_sketch_tc<2, BN><<<grid, TC_THREADS, smem, st>>>(ta, tb, rowsX, rowsY, K, kchunk, out, TC_BM, 0, err, tiles,
-                                                      ntiles, 0, 0, 1.0f);
+                                                      ntiles, 0, 0, 1.0f, 0);
     LSQ_LAUNCH_CHECK();
     return LSQ_OK;
 }

@@ -69,3 +69,15 @@ def test_calls_fail_loudly_without_cuda_tensors(liblsq):
     A = torch.zeros((10, 3), dtype=torch.float64)
     with pytest.raises(lsq.LsqError):
         lsq.pne(A, torch.zeros(10, dtype=torch.float64))
+
+
+@pytest.mark.parametrize("s,n", [(96, 48), (600, 300), (2000, 1000), (8192, 4096)])
+def test_sketch_accumulation_chain_is_bounded(liblsq, s, n):
+    """One accumulator of an FP32 Gaussian sketch sums at most 96 K blocks of
+    64 products, whatever the rows (64 splits reach that at 131072 rows)."""
+    f = liblsq.lsq_test_sketch_chain
+    f.restype = C.c_int64
+    f.argtypes = [C.c_int64, C.c_int64, C.c_int64, C.c_int32]
+    assert f(s, n, 16383, 152) == 0 and f(s, n, 0, 152) == -1
+    for m in [16384, 16385, 50001, 131072, 131073, 200000, 262144, 262145, 1000000, 3000017]:
+        assert 0 < f(s, n, m, 152) <= 96 * 64, m

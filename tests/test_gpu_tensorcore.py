@@ -181,6 +181,13 @@ def test_fp32_gaussian_sketch_fp16_pieces(m, n, s):
     assert e_tc <= 2 * max(np.linalg.norm(oAs - exact), np.linalg.norm(As_cc - exact))
 
 
+@pytest.mark.parametrize("m,n,s", [(262144, 20, 40), (600011, 5, 17)])
+def test_fp32_gaussian_sketch_in_several_launches(m, n, s):
+    # more splits than one launch holds: the bounds of
+    # test_fp32_gaussian_sketch_fp16_pieces
+    test_fp32_gaussian_sketch_fp16_pieces(m, n, s)
+
+
 @pytest.mark.parametrize("m,n,s", [(1037, 113, 250), (3001, 70, 200), (700, 129, 130)])
 def test_fp64_gaussian_sketch_digit_sliced(m, n, s):
     # FP64 sketch as K chunks of 1024 FP64-accurate digit-sliced products:
