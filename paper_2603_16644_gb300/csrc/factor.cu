@@ -325,7 +325,9 @@ template lsq_status launch_cholesky<float>(float*, int64_t, int64_t, int32_t*, c
 // a 2000 x 2000 matrix went from 35.5 to 13.8 ms, with the same bits.
 //
 // l = a / d is formed as q = a r, q + r (a - q d) with r = 1/d correctly
-// rounded: the correctly rounded quotient (Markstein) at 3 FP64 operations.
+// rounded: the correctly rounded quotient (Markstein) at 3 FP64 operations,
+// while a - q d and q are well inside the normal range; tiny and zero a and q take
+// the division (by their exponent fields, no FP64 compare).
 template <typename T>
 struct LuKey;
 template <>
@@ -339,6 +341,10 @@ struct LuKey<double> {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
         return b == 0 || b >= 0x7ff0000000000000ull;
     }
+    // |v| < 2^-895
+    static __device__ __forceinline__ bool tiny(double v) {
+        return ((unsigned)(__double_as_longlong(v) >> 32) & 0x7fffffffu) < (128u << 20);
+    }
 };
 template <>
 struct LuKey<float> {
@@ -350,6 +356,8 @@ struct LuKey<float> {
         const unsigned b = __float_as_uint(v) & 0x7fffffffu;
         return b == 0 || b >= 0x7f800000u;
     }
+    // |v| < 2^-67
+    static __device__ __forceinline__ bool tiny(float v) { return (__float_as_uint(v) & 0x7fffffffu) < (60u << 23); }
 };
 
 // Largest key of the warp, then the smallest position that has it (key 0: none).
@@ -432,7 +440,8 @@ __global__ void __launch_bounds__(NT) k_lu_panel_cl(T* __restrict__ H, int64_t l
             pos = pos == bp ? (unsigned)j : (pos == (unsigned)j ? bp : pos);
             if (!zero && live && pos > (unsigned)j) {
                 const T q = a[j] * rd;
-                const T l = isinf(rd) ? a[j] / d : fma(fma(-q, d, a[j]), rd, q);  // 1/d overflows for a subnormal d
+                // (a tiny d has only tiny a)
+                const T l = LuKey<T>::tiny(a[j]) || LuKey<T>::tiny(q) ? a[j] / d : fma(fma(-q, d, a[j]), rd, q);
                 a[j] = l;
 #pragma unroll
                 for (int c = j + 1; c < LNB; ++c) a[c] = fma(-l, u[c], a[c]);

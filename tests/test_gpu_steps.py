@@ -414,6 +414,31 @@ def test_lu_panel_rows_per_cluster(n):
     assert np.linalg.norm(to_np(F) - LU_o) / np.linalg.norm(LU_o) <= 8 * n * U64 * kH
 
 
+@pytest.mark.parametrize("n", [30, 300, 700])
+@pytest.mark.parametrize("d", [1.5, 3.0 * 2.0**1008, 1.3 * 2.0**-1000, 1.7 * 2.0**-1021, 5.0 * 2.0**-1074])
+def test_lu_multipliers_are_the_divisions(n, d):
+    """The first column's multipliers are entry / pivot as IEEE division gives
+    them, bit for bit (the sign of zeros too), for entries over the whole
+    exponent range below the pivot and for pivots down to subnormal ones."""
+    rng = np.random.default_rng(n + int(np.log2(d)) + 2000)
+    H = np.diag(np.full(n, 1.0)) + 0.01 * rng.standard_normal((n, n))
+    col = d * rng.uniform(-1, 1, n) * np.exp2(-rng.uniform(0, 60, n))
+    wide = rng.random(n) < 0.4
+    col[wide] = (rng.uniform(-1, 1, n) * np.exp2(-rng.uniform(0, 1074, n)))[wide] * min(d, 1.0)
+    col[rng.integers(0, n, 3)] = [0.0, -0.0, 2.0**-1074 if d > 2.0**-1070 else 0.0]
+    at = int(rng.integers(0, n))
+    col[at] = d
+    H[:, 0] = col
+    _, F, piv, _ = lsq.factor_solve(dev_colmajor(H), torch.ones(n, dtype=torch.float64, device="cuda"), hpne=True)
+    F, piv = to_np(F), to_np(piv)
+    assert piv[0] == at
+    want = col.copy()
+    for k in range(n):  # the row interchanges
+        want[[k, piv[k]]] = want[[piv[k], k]]
+    want[1:] = want[1:] / d
+    np.testing.assert_array_equal(F[:, 0].view(np.int64), want.view(np.int64))
+
+
 @pytest.mark.parametrize("n", [1, 40, 300])
 def test_lu_zero_pivot_reported(n):
     """A zero column breaks down at its own index on both sides."""
