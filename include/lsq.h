@@ -427,6 +427,11 @@ int64_t lsq_test_set_solve_wait_ns(int64_t ns);
  * formed from FP16 pieces (three products a row). */
 int64_t lsq_test_sketch_chain(int64_t s, int64_t n, int64_t m, int32_t sms);
 
+/* Test-only query (host arithmetic): CTAs of the cluster that factors an LU
+ * panel of `rows` rows on a device that schedules clusters of up to max_cluster
+ * CTAs (16, 8 or 0), 0 for the one-CTA kernel. */
+int32_t lsq_test_lu_cluster(int64_t rows, int32_t max_cluster);
+
 /* ---- Batched solves (many independent problems of uneven shape) --------- */
 
 /* One problem of a batch: device pointers A (m x n, ld lda), b (m), x (n),

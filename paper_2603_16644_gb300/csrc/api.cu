@@ -779,6 +779,8 @@ int32_t lsq_set_tensor_core_sketch(int32_t enable) {
     return prev;
 }
 
+int32_t lsq_test_lu_cluster(int64_t rows, int32_t max_cluster) { return rows > 0 ? lu_panel_cluster(rows, max_cluster) : -1; }
+
 int64_t lsq_test_sketch_chain(int64_t s, int64_t n, int64_t m, int32_t sms) {
     if (s <= 0 || n <= 0 || m <= 0 || sms <= 0) return -1;
     return gauss_fp32_f16(m) ? sketch_pieces_chain(s, n, m, sms) : 0;

@@ -17,6 +17,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 namespace lsq {
@@ -456,7 +457,7 @@ __global__ void __launch_bounds__(NT) k_lu_panel_cl(T* __restrict__ H, int64_t l
 }
 
 // The same panel by one block of 1024 threads in global memory: panels with
-// more rows than the cluster holds (16 x 512).
+// more rows than the cluster holds (512 a CTA).
 template <typename T>
 __global__ void __launch_bounds__(1024) k_lu_panel(T* __restrict__ H, int64_t ld, int64_t rows, int64_t k0, int nb,
                                                    int32_t* __restrict__ piv, int32_t* __restrict__ info) {
@@ -566,15 +567,21 @@ __global__ void __launch_bounds__(32) k_lu_u12(T* __restrict__ H, int64_t ld, in
         if (i < nb) H[(k0 + i) + c * ld] = u[i];
 }
 
-// Launch of one panel: a cluster with about 64 rows per CTA (at most 16
-// CTAs), fewer where the device cannot hold the larger one.
+// CTAs of the cluster for a panel of prow rows: about 64 rows each up to
+// max_cluster CTAs, at most 512 (a thread holds a row); 0: no cluster holds it.
+int lu_panel_cluster(int64_t prow, int max_cluster) {
+    int cl = 1;
+    while (cl < max_cluster && cl * 64 < prow) cl *= 2;
+    return max_cluster > 0 && ceil_div(prow, cl) <= 512 ? cl : 0;
+}
+
 template <typename T, int NT>
-static bool lu_panel_try(int cl, T* H, int64_t ld, int64_t rows, int64_t k0, int nb, int32_t* piv, int32_t* info,
-                         cudaStream_t st, cudaError_t& e) {
+static cudaError_t lu_panel_launch(int cl, bool query, int* fits, T* H, int64_t ld, int64_t rows, int64_t k0, int nb,
+                                   int32_t* piv, int32_t* info, cudaStream_t st) {
     auto kern = k_lu_panel_cl<T, NT>;
-    if (cl > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
+    if (cl > 8) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -587,25 +594,57 @@ static bool lu_panel_try(int cl, T* H, int64_t ld, int64_t rows, int64_t k0, int
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, H, ld, rows, k0, nb, piv, info);
-    return true;
+    if (query) return cudaOccupancyMaxActiveClusters(fits, kern, &cfg);
+    return cudaLaunchKernelEx(&cfg, kern, H, ld, rows, k0, nb, piv, info);
+}
+
+// The panel kernel of at least R threads, launched or (query) asked how many
+// clusters of cl CTAs the device holds.
+template <typename T>
+static cudaError_t lu_panel_do(int64_t R, int cl, bool query, int* fits, T* H, int64_t ld, int64_t rows, int64_t k0,
+                               int nb, int32_t* piv, int32_t* info, cudaStream_t st) {
+    if (R <= 64) return lu_panel_launch<T, 64>(cl, query, fits, H, ld, rows, k0, nb, piv, info, st);
+    if (R <= 128) return lu_panel_launch<T, 128>(cl, query, fits, H, ld, rows, k0, nb, piv, info, st);
+    if (R <= 256) return lu_panel_launch<T, 256>(cl, query, fits, H, ld, rows, k0, nb, piv, info, st);
+    return lu_panel_launch<T, 512>(cl, query, fits, H, ld, rows, k0, nb, piv, info, st);
+}
+
+// Largest cluster that the device schedules with every thread count: 16
+// (non-portable), else 8, else 0.  Asked once per device.
+template <typename T>
+static int lu_max_cluster() {
+    static std::mutex mu;
+    static int last_dev = -1, last = 0;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev == last_dev) return last;
+    last = 0;
+    for (int cl : {LUC, 8}) {
+        bool all = true;
+        for (int64_t R : {64, 128, 256, 512}) {
+            int fits = 0;
+            all = all && lu_panel_do<T>(R, cl, true, &fits, nullptr, 0, 0, 0, 0, nullptr, nullptr, nullptr) == cudaSuccess &&
+                  fits >= 1;
+        }
+        if (all) {
+            last = cl;
+            break;
+        }
+        cudaGetLastError();
+    }
+    last_dev = dev;
+    return last;
 }
 
 template <typename T>
 static lsq_status launch_lu_panel(T* H, int64_t ld, int64_t rows, int64_t k0, int nb, int32_t* piv, int32_t* info,
                                   cudaStream_t st) {
-    const int64_t prow = rows - k0;
-    int cl = 1;
-    while (cl < LUC && cl * 64 < prow) cl *= 2;
-    const int64_t R = ceil_div(prow, cl);
-    cudaError_t e = cudaSuccess;
-    bool done = false;
-    if (R <= 64) done = lu_panel_try<T, 64>(cl, H, ld, rows, k0, nb, piv, info, st, e);
-    else if (R <= 128) done = lu_panel_try<T, 128>(cl, H, ld, rows, k0, nb, piv, info, st, e);
-    else if (R <= 256) done = lu_panel_try<T, 256>(cl, H, ld, rows, k0, nb, piv, info, st, e);
-    else if (R <= 512) done = lu_panel_try<T, 512>(cl, H, ld, rows, k0, nb, piv, info, st, e);
-    if (!done) k_lu_panel<T><<<1, 1024, 0, st>>>(H, ld, rows, k0, nb, piv, info);
-    LSQ_CUDA_TRY(e);
+    const int cl = lu_panel_cluster(rows - k0, lu_max_cluster<T>());
+    if (cl > 0)
+        LSQ_CUDA_TRY(lu_panel_do<T>(ceil_div(rows - k0, cl), cl, false, nullptr, H, ld, rows, k0, nb, piv, info, st));
+    else
+        k_lu_panel<T><<<1, 1024, 0, st>>>(H, ld, rows, k0, nb, piv, info);
     LSQ_LAUNCH_CHECK();
     return LSQ_OK;
 }

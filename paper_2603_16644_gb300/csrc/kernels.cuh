@@ -107,6 +107,8 @@ template <typename T>
 lsq_status launch_cholesky(T* G, int64_t n, int64_t ld, int32_t* info, cudaStream_t st, void* ws = nullptr,
                            size_t ws_bytes = 0);
 size_t cholesky_ws_bytes(int64_t n);
+// CTAs of the LU panel's cluster (0: the one-CTA kernel) where clusters of up to max_cluster run.
+int lu_panel_cluster(int64_t prow, int max_cluster);
 lsq_status launch_lu(double* H, int64_t n, int64_t ld, int32_t* piv, int32_t* info, cudaStream_t st);
 enum TrsvKind { TRSV_LOWER = 0, TRSV_LOWER_T = 1, TRSV_UPPER = 2, TRSV_UNIT_LOWER = 3, TRSV_UPPER_T = 4 };
 // sync: trsv_sync_ints(n) int32 of scratch (cleared by the launch); err: the

@@ -81,3 +81,21 @@ def test_sketch_accumulation_chain_is_bounded(liblsq, s, n):
     assert f(s, n, 16383, 152) == 0 and f(s, n, 0, 152) == -1
     for m in [16384, 16385, 50001, 131072, 131073, 200000, 262144, 262145, 1000000, 3000017]:
         assert 0 < f(s, n, m, 152) <= 96 * 64, m
+
+
+def test_lu_panel_cluster_follows_the_device(liblsq):
+    """The LU panel's cluster never exceeds what the device schedules, leaves a
+    CTA at most 512 rows, and gives way to the one-CTA kernel beyond."""
+    f = liblsq.lsq_test_lu_cluster
+    f.restype = C.c_int32
+    f.argtypes = [C.c_int64, C.c_int32]
+    for cap in (16, 8, 0):
+        for rows in [1, 63, 64, 65, 128, 129, 512, 513, 1024, 1025, 4096, 4097, 8192, 8193, 100000]:
+            cl = f(rows, cap)
+            assert 0 <= cl <= cap
+            if cl:
+                assert cl * 512 >= rows and (cl == cap or cl * 64 >= rows)
+            else:
+                assert cap * 512 < rows
+    assert [f(r, 16) for r in (64, 65, 1024, 8192, 8193)] == [1, 2, 16, 16, 0]
+    assert [f(r, 8) for r in (512, 513, 4096, 4097)] == [8, 8, 8, 0]
