@@ -459,7 +459,8 @@ size_t lsq_batched_workspace_size(int32_t hpne, int32_t count, const lsq_batch_p
  * grows with it), heaviest first to the least-loaded stream, and the whole
  * fan-out is captured into one
  * CUDA graph; the executable graph is cached and replayed on `stream` while
- * the descriptors (pointers, shapes, options, workspace) stay the same.  A
+ * the descriptors (pointers, shapes, options, workspace), the process-wide
+ * switches and the reduction hook stay the same.  A
  * call with new descriptors enqueues the fan-out directly (forked from and
  * joined to `stream`) and captures the graph while the GPU works.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
  * batched condition-estimate pass (the same fan-out, in a cached graph of

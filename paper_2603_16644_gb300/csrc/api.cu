@@ -50,6 +50,10 @@ lsq_status reduce_partial(void* buf, int64_t count, int kind, cudaStream_t st) {
     return r == LSQ_OK ? LSQ_OK : LSQ_ERR_CUDA;
 }
 bool reduce_hook_set() { return g_reduce_fn != nullptr; }
+void reduce_hook(const void** fn, const void** user) {
+    *fn = (const void*)g_reduce_fn;
+    *user = g_reduce_fn ? g_reduce_user : nullptr;
+}
 bool profiling_on() {
     std::lock_guard<std::mutex> lk(g_prof.mu);
     return g_prof.on;

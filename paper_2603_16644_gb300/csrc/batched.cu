@@ -84,6 +84,23 @@ lsq_status ensure_streams() {
     return LSQ_OK;
 }
 
+// What the kernels of a fan-out depend on beside its descriptors, at the end of
+// its graph's key: the buffers, which call it is (tag) and the library's switches
+// and reduction hook (a captured hook is part of the graph).
+void key_tail(std::vector<unsigned char>& key, const void* ws, size_t ws_bytes, int tag) {
+    struct Tail {
+        const void* ws;
+        uint64_t ws_bytes;
+        int64_t tag, emulation, tc_sketch;
+        uint64_t wait_ns;
+        const void *hook, *hook_user;
+    } t{ws, ws_bytes, tag, fp64_emulation_enabled() ? 1 : 0, tensor_core_sketch_enabled() ? 1 : 0, trsv_wait_ns(), nullptr,
+        nullptr};
+    reduce_hook(&t.hook, &t.hook_user);
+    static_assert(sizeof(Tail) == 64, "no padding");
+    key.insert(key.end(), (const unsigned char*)&t, (const unsigned char*)&t + sizeof(t));
+}
+
 struct Plan {
     std::vector<int> stream_of;   // problem -> internal stream
     std::vector<int> order;       // launch order (heaviest first)
@@ -262,11 +279,9 @@ lsq_status batched(bool hpne, int32_t count, const lsq_batch_problem* probs, voi
         std::vector<int> est_order;
         for (int i : P.order)
             if (is_auto(q[i].opts.sketch_prec)) est_order.push_back(i);
-        std::vector<unsigned char> ekey(sizeof(lsq_batch_problem) * count + 64, 0);
+        std::vector<unsigned char> ekey(sizeof(lsq_batch_problem) * count);
         std::memcpy(ekey.data(), probs, sizeof(lsq_batch_problem) * count);
-        unsigned char* et = ekey.data() + sizeof(lsq_batch_problem) * count;
-        std::memcpy(et, &ws, sizeof(ws));
-        std::memcpy(et + 8, &ws_bytes, sizeof(ws_bytes));
+        key_tail(ekey, ws, ws_bytes, 0);
         r = capture_fanout(g_est, est_order, P.stream_of, slots, P.slot_bytes, ekey, st,
                            [&](int i, cudaStream_t sk, char* slot) {
                                if (q[i].opts.sketch_prec == LSQ_AUTO)
@@ -287,15 +302,10 @@ lsq_status batched(bool hpne, int32_t count, const lsq_batch_problem* probs, voi
             }
     }
 
-    // key of the captured graph: the resolved descriptors and the buffers
-    std::vector<unsigned char> key(sizeof(lsq_batch_problem) * count + 64);
+    // key of the captured graph: the resolved descriptors, the buffers and the settings
+    std::vector<unsigned char> key(sizeof(lsq_batch_problem) * count);
     std::memcpy(key.data(), q.data(), sizeof(lsq_batch_problem) * count);
-    unsigned char* tail = key.data() + sizeof(lsq_batch_problem) * count;
-    std::memset(tail, 0, 64);
-    std::memcpy(tail, &ws, sizeof(ws));
-    std::memcpy(tail + 8, &ws_bytes, sizeof(ws_bytes));
-    int32_t hp = hpne ? 1 : 0;
-    std::memcpy(tail + 16, &hp, sizeof(hp));
+    key_tail(key, ws, ws_bytes, hpne ? 1 : 0);
     return capture_fanout(g_main, P.order, P.stream_of, slots, P.slot_bytes, key, st,
                           [&](int i, cudaStream_t sk, char* slot) {
                               return solve_impl_ext(hpne, q[i].A, q[i].m, q[i].n, q[i].lda, q[i].b, &q[i].opts,
@@ -340,12 +350,9 @@ lsq_status batched_steps(int tag, int32_t count, const Prob* probs, void* ws, si
     if (r != LSQ_OK) return r;
     std::vector<int> order, stream_of;
     assign_streams(work, order, stream_of);
-    std::vector<unsigned char> key(sizeof(Prob) * count + 64, 0);
+    std::vector<unsigned char> key(sizeof(Prob) * count);
     std::memcpy(key.data(), probs, sizeof(Prob) * count);
-    unsigned char* tail = key.data() + sizeof(Prob) * count;
-    std::memcpy(tail, &ws, sizeof(ws));
-    std::memcpy(tail + 8, &ws_bytes, sizeof(ws_bytes));
-    std::memcpy(tail + 16, &tag, sizeof(tag));
+    key_tail(key, ws, ws_bytes, tag);
     return capture_fanout(g_main, order, stream_of, base, slot, key, st,
                           [&](int i, cudaStream_t sk, char* sl) { return run(probs[i], sl, slot, sk); });
 }

@@ -951,6 +951,8 @@ size_t trsv_sync_ints(int64_t n) { return 2 + 2 * (size_t)n; }
 // Bound of one wait for another block's solution (2 s; shorter only in tests).
 static uint64_t g_trsv_wait_ns = 2000000000ull;
 
+uint64_t trsv_wait_ns() { return g_trsv_wait_ns; }
+
 uint64_t set_trsv_wait_ns(uint64_t ns) {
     const uint64_t old = g_trsv_wait_ns;
     g_trsv_wait_ns = ns;

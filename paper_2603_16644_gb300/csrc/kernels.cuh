@@ -116,6 +116,7 @@ enum TrsvKind { TRSV_LOWER = 0, TRSV_LOWER_T = 1, TRSV_UPPER = 2, TRSV_UNIT_LOWE
 size_t trsv_sync_ints(int64_t n);
 // Bound of the wavefront solves' waits (process-wide; returns the previous one).
 uint64_t set_trsv_wait_ns(uint64_t ns);
+uint64_t trsv_wait_ns();
 template <typename T>
 lsq_status launch_trsv(int kind, const T* M, int64_t n, int64_t ld, T* y, const int32_t* info, int32_t* sync,
                        int32_t* err, cudaStream_t st);
@@ -194,6 +195,7 @@ lsq_status launch_colnorm1_max(const float* M, int64_t n, int64_t ld, bool upper
 
 // Whether a reduction hook is registered / the stage timing is on (api.cu).
 bool reduce_hook_set();
+void reduce_hook(const void** fn, const void** user);
 bool profiling_on();
 
 // While one lives, this thread's steps stay on the stream they are given (no

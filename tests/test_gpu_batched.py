@@ -3,6 +3,8 @@ every problem's result equals the single-problem call bit for bit (same
 kernels, same inputs), replays reuse the graph and see new data, AUTO
 precisions are resolved per problem, and the results meet the solution
 tolerance against the oracle."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -104,6 +106,70 @@ def test_batched_bad_input():
         lsq.batched_workspace(desc)
     with pytest.raises(lsq.LsqError):
         lsq.solve_batched(desc, torch.empty(1024, dtype=torch.uint8, device="cuda"))
+
+
+def batch_buffers(probs, opts):
+    As = [dev_colmajor(p.A) for p in probs]
+    bs = [torch.from_numpy(p.b).cuda() for p in probs]
+    xs = [torch.full((p.shape[1],), float("nan"), dtype=torch.float64, device="cuda") for p in probs]
+    infos = [torch.full((1,), -9, dtype=torch.int32, device="cuda") for _ in probs]
+    desc = lsq.batch_descriptors(As, bs, xs, infos, opts)
+    return As, bs, xs, infos, desc, lsq.batched_workspace(desc)
+
+
+def set_tc_sketch(on):
+    f = lsq.lib().lsq_set_tensor_core_sketch
+    f.restype = C.c_int32
+    f.argtypes = [C.c_int32]
+    return bool(f(int(on)))
+
+
+@pytest.mark.parametrize("auto", [False, True])
+@pytest.mark.parametrize("switch", [lsq.set_fp64_emulation, set_tc_sketch])
+def test_batched_follows_the_switches(switch, auto):
+    """The same descriptors after a switch was changed: the bits of single calls
+    under the new setting, and of the old one once it is back."""
+    probs, opts = make_batch(4, 21)
+    for o in opts:
+        o.kind, o.sketch_prec, o.qr_prec = lsq.GAUSSIAN, lsq.AUTO if auto else lsq.FP32, lsq.FP32
+    As, bs, xs, infos, desc, ws = batch_buffers(probs, opts)
+    lsq.solve_batched(desc, ws)
+    first = [to_np(x).copy() for x in xs]
+    prev = switch(False)
+    try:
+        lsq.solve_batched(desc, ws)
+        got = [to_np(x).copy() for x in xs]
+        want = [to_np(lsq.pne(A, b, opts=o)[0]) for A, b, o in zip(As, bs, opts)]
+    finally:
+        switch(prev)
+    for g, w in zip(got, want):
+        np.testing.assert_array_equal(g, w)
+    assert any(np.any(g != f) for g, f in zip(got, first))
+    lsq.solve_batched(desc, ws)
+    for x, f in zip(xs, first):
+        np.testing.assert_array_equal(to_np(x), f)
+
+
+def test_batched_follows_the_reduction_hook():
+    """A hook set after a batch ran is called by the same batch's next run, and
+    no more once it is removed."""
+    probs, opts = make_batch(3, 22)
+    As, bs, xs, infos, desc, ws = batch_buffers(probs, opts)
+    lsq.solve_batched(desc, ws)
+    first = [to_np(x).copy() for x in xs]
+    calls = []
+    lsq.set_reduce_hook(lambda buf, count, kind, stream: calls.append(count) or 0)
+    try:
+        lsq.solve_batched(desc, ws)
+        torch.cuda.synchronize()
+    finally:
+        lsq.set_reduce_hook(None)
+    assert len(calls) >= 3 * len(probs)  # the sketch, the Gram and the right-hand side of each
+    n = len(calls)
+    lsq.solve_batched(desc, ws)
+    assert len(calls) == n
+    for x, f in zip(xs, first):
+        np.testing.assert_array_equal(to_np(x), f)
 
 
 def test_autotuner_picks_a_candidate(tmp_path):
