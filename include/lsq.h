@@ -590,7 +590,8 @@ int32_t lsq_set_tensor_core_sketch(int32_t enable);
  * process ("no error" if none). */
 const char* lsq_last_cuda_error(void);
 
-/* Number of kernel launches this library has issued since it was loaded. */
+/* Number of kernel launches this library has issued since it was loaded, one by
+ * one (the kernels of a replayed batched graph are not counted again). */
 int64_t lsq_launch_count(void);
 
 /* Stage timing.  lsq_profile(1) clears the records and starts recording a

@@ -14,7 +14,9 @@ using namespace lsq;
 namespace lsq {
 
 static std::atomic<long long> g_launches{0};
-void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+void note_launch() {
+    if (!UncountedScope::active()) g_launches.fetch_add(1, std::memory_order_relaxed);
+}
 
 // Pool of event pairs, one pair per (solve, stage) while profiling is on.
 struct StageProf {

@@ -20,6 +20,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <optional>
 #include <vector>
 
 namespace lsq {
@@ -213,7 +214,10 @@ lsq_status capture_fanout(GraphCache& cache, const std::vector<int>& order, cons
     // stream, which cannot be captured); the graph is then launched on st.
     cudaStream_t cs = g_batch.cap;
     LSQ_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
+    std::optional<UncountedScope> uncounted;
+    if (direct) uncounted.emplace();
     const lsq_status cap = enqueue_fanout(cs, order, stream_of, slots, slot_bytes, run);
+    uncounted.reset();
     cudaError_t ec = cudaStreamEndCapture(cs, &graph);
     if (cap != LSQ_OK || ec != cudaSuccess || !graph) {
         if (graph) cudaGraphDestroy(graph);

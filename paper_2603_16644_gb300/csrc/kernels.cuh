@@ -198,12 +198,13 @@ bool reduce_hook_set();
 void reduce_hook(const void** fn, const void** user);
 bool profiling_on();
 
-// While one lives, this thread's steps stay on the stream they are given (no
-// look-ahead on the library's shared streams): the batched fan-out, whose
-// problems run side by side.
-struct FanoutScope {
-    FanoutScope() { ++depth(); }
-    ~FanoutScope() { --depth(); }
+// Per-thread state that holds while an object of it lives.
+template <typename Tag>
+struct ThreadScope {
+    ThreadScope() { ++depth(); }
+    ~ThreadScope() { --depth(); }
+    ThreadScope(const ThreadScope&) = delete;
+    ThreadScope& operator=(const ThreadScope&) = delete;
     static bool active() { return depth() > 0; }
 
 private:
@@ -212,6 +213,11 @@ private:
         return d;
     }
 };
+// This thread's steps stay on the stream they are given (no look-ahead on the
+// library's shared streams): the batched fan-out, whose problems run side by side.
+using FanoutScope = ThreadScope<struct FanoutTag>;
+// Launches are not counted: the capture of a fan-out that has been enqueued already.
+using UncountedScope = ThreadScope<struct UncountedTag>;
 
 // ---- qr.cu -------------------------------------------------------------------
 size_t qr_ws_bytes(int64_t s, int64_t n, int prec);

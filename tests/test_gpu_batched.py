@@ -172,6 +172,25 @@ def test_batched_follows_the_reduction_hook():
         np.testing.assert_array_equal(to_np(x), f)
 
 
+def test_batched_launches_are_counted_once():
+    """lsq_launch_count over a new batch is the sum over single calls (problems
+    of one QR panel, where both run the same kernels), and a replay adds none."""
+    probs, opts = [], []
+    for i in range(3):
+        probs.append(P.make_problem(900 + 100 * i, 30, 1e3, 1e-6, 77 + i))
+        opts.append(lsq.make_opts(kind=lsq.SPARSE_SIGN, s=120, zeta=8, seed=i, sketch_prec=lsq.FP32))
+    As, bs, xs, infos, desc, ws = batch_buffers(probs, opts)
+    n0 = lsq.launch_count()
+    for A, b, o in zip(As, bs, opts):
+        lsq.pne(A, b, opts=o)
+    n1 = lsq.launch_count()
+    lsq.solve_batched(desc, ws)
+    n2 = lsq.launch_count()
+    assert n2 - n1 == n1 - n0 > 0
+    lsq.solve_batched(desc, ws)
+    assert lsq.launch_count() == n2
+
+
 def test_autotuner_picks_a_candidate(tmp_path):
     from paper_2603_16644_gb300.autotune import CANDIDATES, Autotuner
 
