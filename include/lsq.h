@@ -462,7 +462,9 @@ size_t lsq_batched_workspace_size(int32_t hpne, int32_t count, const lsq_batch_p
  * the descriptors (pointers, shapes, options, workspace), the process-wide
  * switches and the reduction hook stay the same.  A
  * call with new descriptors enqueues the fan-out directly (forked from and
- * joined to `stream`) and captures the graph while the GPU works.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
+ * joined to `stream`) and captures the graph while the GPU works; a CUDA error
+ * while it enqueues leaves the outputs undefined, and what a single solve
+ * refuses is refused before any problem runs.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
  * batched condition-estimate pass (the same fan-out, in a cached graph of
  * its own) and one readback of the chosen precisions (a stream
  * synchronisation).  Each problem's status goes to its own info.

@@ -1056,6 +1056,12 @@ lsq_status solve_impl_ext(bool hpne, const double* A, int64_t m, int64_t n, int6
     return solve_impl(hpne, A, m, n, lda, b, o, x, Rs_out, info, ws, ws_bytes, st, Rs_in);
 }
 
+// What every solve and sketch refuses about its options, sketch_prec a precision or AUTO*.
+lsq_status check_opts_ext(const lsq_opts* o, int64_t m, int64_t n) {
+    lsq_status r = check_opts(o, m, n, true);
+    if (r != LSQ_OK) return r;
+    return o->kind == LSQ_SRFT && !is_auto(o->sketch_prec) && !srft_fits(m, o->sketch_prec) ? LSQ_ERR_ARG : LSQ_OK;
+}
 size_t solve_ws_bytes_ext(int64_t m, int64_t n, const lsq_opts* o, bool hpne) {
     return solve_layout(m, n, o, layout_prec(o->sketch_prec), hpne, device_sm_count()).total + 256;
 }

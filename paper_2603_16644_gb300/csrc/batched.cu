@@ -28,6 +28,7 @@ lsq_status solve_impl_ext(bool hpne, const double* A, int64_t m, int64_t n, int6
                           const lsq_opts* o, double* x, double* Rs_out, int32_t* info, void* ws, size_t ws_bytes,
                           cudaStream_t st, const double* Rs_in);
 size_t solve_ws_bytes_ext(int64_t m, int64_t n, const lsq_opts* o, bool hpne);
+lsq_status check_opts_ext(const lsq_opts* o, int64_t m, int64_t n);
 }  // namespace lsq
 
 namespace {
@@ -213,7 +214,12 @@ lsq_status capture_fanout(GraphCache& cache, const std::vector<int>& order, cons
     // Capture on an internal stream (the caller may use the legacy default
     // stream, which cannot be captured); the graph is then launched on st.
     cudaStream_t cs = g_batch.cap;
-    LSQ_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
+    const cudaError_t eb = cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed);
+    if (eb != cudaSuccess) {
+        cudaGetLastError();
+        note_cuda_error(eb);
+        return direct ? LSQ_OK : LSQ_ERR_CUDA;  // enqueued: as below
+    }
     std::optional<UncountedScope> uncounted;
     if (direct) uncounted.emplace();
     const lsq_status cap = enqueue_fanout(cs, order, stream_of, slots, slot_bytes, run);
@@ -258,8 +264,10 @@ void assign_streams(const std::vector<double>& work, std::vector<int>& order, st
 lsq_status batched(bool hpne, int32_t count, const lsq_batch_problem* probs, void* ws, size_t ws_bytes,
                    cudaStream_t st) {
     if (count <= 0 || !probs) return LSQ_ERR_ARG;
+    // everything that a single solve refuses, before any problem runs
     for (int i = 0; i < count; ++i) {
         lsq_status r = check_problem(probs[i]);
+        if (r == LSQ_OK) r = check_opts_ext(&probs[i].opts, probs[i].m, probs[i].n);
         if (r != LSQ_OK) return r;
     }
     std::lock_guard<std::mutex> lk(g_batch.mu);
@@ -303,6 +311,7 @@ lsq_status batched(bool hpne, int32_t count, const lsq_batch_problem* probs, voi
                 int p = host_ch[i];
                 q[i].opts.sketch_prec = (p >= LSQ_FP8_E4M3 && p <= LSQ_FP64) ? p : LSQ_FP64;
                 if (q[i].opts.sketch_prec == LSQ_FP64) q[i].opts.qr_prec = LSQ_FP64;
+                if ((r = check_opts_ext(&q[i].opts, q[i].m, q[i].n)) != LSQ_OK) return r;
             }
     }
 
@@ -324,7 +333,7 @@ size_t qr_slot_bytes(const lsq_qr_problem& p) { return lsq_workspace_size(LSQ_OP
 lsq_status check_sketch_problem(const lsq_sketch_problem& p) {
     if (!p.A || !p.As || !p.colexp || p.m <= 0 || p.n <= 0 || p.lda < p.m || p.ldas < p.opts.s) return LSQ_ERR_ARG;
     if (p.opts.sketch_prec < LSQ_FP8_E4M3 || p.opts.sketch_prec > LSQ_FP64) return LSQ_ERR_ARG;
-    return sketch_slot_bytes(p) ? LSQ_OK : LSQ_ERR_ARG;
+    return sketch_slot_bytes(p) ? check_opts_ext(&p.opts, p.m, p.n) : LSQ_ERR_ARG;
 }
 
 lsq_status check_qr_problem(const lsq_qr_problem& p) {

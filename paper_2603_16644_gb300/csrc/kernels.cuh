@@ -66,6 +66,8 @@ bool tensor_core_sketch_enabled();
 // srft_ws_bytes of scratch (the signed, padded, transformed columns).
 int64_t srft_order(int64_t m);
 size_t srft_ws_bytes(int64_t m, int64_t n, int prec);
+// Whether the transform takes m rows (launch_srft refuses more).
+bool srft_fits(int64_t m, int prec);
 lsq_status launch_srft(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp, int prec,
                        uint64_t seed, int64_t s, void* W, void* As, int64_t ldas, cudaStream_t st);
 // Columns [k0, k0 + kc) of -Omega (FP64), s x kc column-major, ld s.

@@ -741,12 +741,14 @@ size_t srft_ws_bytes(int64_t m, int64_t n, int prec) {
     return (prec == LSQ_FP64 ? 8 : 4) * (size_t)srft_order(m) * (size_t)n;
 }
 
+// Largest order: 2^10 blocks in FP32, 2^9 in FP64.
+bool srft_fits(int64_t m, int prec) { return srft_order(m) <= ((int64_t)FW_B << (prec == LSQ_FP64 ? 9 : 10)); }
+
 template <typename T, int PREC>
 static lsq_status srft_run(const double* A, int64_t m, int64_t n, int64_t lda, const int32_t* colexp, uint64_t seed,
                            int64_t s, T* W, void* As, int64_t ldas, cudaStream_t st) {
     const int64_t mp = srft_order(m);
-    // largest order: 2^10 blocks in FP32, 2^9 in FP64
-    if (mp > ((int64_t)FW_B << (sizeof(T) == 8 ? 9 : 10))) return LSQ_ERR_ARG;
+    if (!srft_fits(m, PREC)) return LSQ_ERR_ARG;
     k_srft_block<T, PREC><<<dim3((unsigned)ceil_div(mp, FW_B), (unsigned)n), 256, 0, st>>>(A, m, lda, colexp, seed, mp, W);
     LSQ_LAUNCH_CHECK();
     // the levels above: at most five at a time

@@ -191,6 +191,39 @@ def test_batched_launches_are_counted_once():
     assert lsq.launch_count() == n2
 
 
+@pytest.mark.parametrize("field,value", [("refine_steps", 2), ("qr_prec", lsq.BF16), ("row_offset", -1)])
+def test_batched_refuses_before_any_problem_runs(field, value):
+    """Options that a single call refuses, in a problem after heavier ones: the
+    batch is refused with nothing launched, and runs without that problem."""
+    probs, opts = make_batch(3, 23)
+    probs.append(P.make_problem(600, 2, 10.0, 0.0, 5))
+    opts.append(lsq.make_opts(kind=lsq.SPARSE_SIGN, s=20, zeta=4, seed=1, sketch_prec=lsq.FP32))
+    As, bs, xs, infos, desc, ws = batch_buffers(probs, opts)
+    setattr(desc[3].opts, field, value)
+    n0 = lsq.launch_count()
+    with pytest.raises(lsq.LsqError):
+        lsq.solve_batched(desc, ws)
+    assert lsq.launch_count() == n0
+    for x, info in zip(xs, infos):
+        assert np.isnan(to_np(x)).all() and int(to_np(info)[0]) == -9
+    three = lsq.batch_descriptors(As[:3], bs[:3], xs[:3], infos[:3], opts[:3])
+    lsq.solve_batched(three, ws)
+    for A, b, x, o in zip(As, bs, xs[:3], opts):
+        np.testing.assert_array_equal(to_np(x), to_np(lsq.pne(A, b, opts=o)[0]))
+
+
+def test_batched_sketch_refuses_the_transform_order_before_any_runs():
+    """An SRFT of more rows than the transform takes (2^22 in FP32)."""
+    big = torch.randn((1, 2**22 + 1), dtype=torch.float64, device="cuda").t()
+    small = dev_colmajor(np.random.default_rng(1).standard_normal((4000, 200)))
+    ob = lsq.make_opts(kind=lsq.SRFT, s=8, zeta=0, seed=1, sketch_prec=lsq.FP32)
+    os_ = lsq.make_opts(kind=lsq.GAUSSIAN, s=4000, zeta=0, seed=1, sketch_prec=lsq.FP32)
+    n0 = lsq.launch_count()
+    with pytest.raises(lsq.LsqError):
+        lsq.sketch_batched([small, big], [os_, ob])
+    assert lsq.launch_count() == n0
+
+
 def test_autotuner_picks_a_candidate(tmp_path):
     from paper_2603_16644_gb300.autotune import CANDIDATES, Autotuner
 
