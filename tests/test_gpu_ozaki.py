@@ -88,6 +88,37 @@ def test_nonfinite_columns_give_nan_rows_and_columns():
     np.testing.assert_array_equal(G[np.ix_(ok, ok)], (Xi.T @ Xi)[np.ix_(ok, ok)])
 
 
+@pytest.mark.parametrize("m,n,tn", [(600, 1025, False), (70000, 1100, False), (600, 769, True), (70000, 900, True)])
+def test_many_blocks_exact_on_integer_data(m, n, tn):
+    """Enough 128 x 128 blocks for the combination kernel of large n (n above
+    1024 for X^T X, 768 for X^T Y on 152 SMs), one K chunk and two: exact on
+    small integers; 26-bit integers (one chunk) rounded correctly; NaN exactly
+    in the rows and columns of a column with an infinite entry."""
+    g = torch.Generator(device="cuda").manual_seed(m + n)
+    X = torch.randint(-8, 9, (n, m), generator=g, device="cuda").double().t()
+    Y = torch.randint(-8, 9, (n, m), generator=g, device="cuda").double().t() if tn else X
+
+    def run(X, Y):
+        G, info = lsq.gemm_tn_tc(X, Y) if tn else lsq.gram_tc(X)
+        assert int(to_np(info)[0]) == 0
+        return to_np(G)
+
+    np.testing.assert_array_equal(run(X, Y), to_np(X.t() @ Y))  # sums below 2^53
+    if m == 600:
+        rng = np.random.default_rng(n)
+        W = [rng.integers(-(2**26), 2**26, (m, n)) for _ in range(2)]
+        Wx, Wy = W[0], W[1] if tn else W[0]
+        G = run(dev_colmajor(Wx.astype(np.float64)), dev_colmajor(Wy.astype(np.float64)))
+        np.testing.assert_array_equal(G, (Wx.T @ Wy).astype(np.float64))  # below 2^62: one rounding
+        Z = X.clone()
+        Z[7, n - 3] = float("inf")
+        G, want = run(Z, Y if tn else Z), to_np(X.t() @ Y)
+        want[n - 3, :] = np.nan
+        if not tn:
+            want[:, n - 3] = np.nan
+        np.testing.assert_array_equal(G, want)
+
+
 @pytest.mark.parametrize("m,n,spread", [(5000, 257, 0), (70000, 130, 0), (4000, 64, 30)])
 def test_within_fp64_error_order(m, n, spread):
     rng = np.random.default_rng(7 + n)
