@@ -248,6 +248,25 @@ def test_precond_qr_extreme_column_norms(prec, lo, hi, s, n):
     assert err.max() <= 20 * n * unit * O.kappa(Bs), err.max()
 
 
+@pytest.mark.parametrize("s,n", [(513, 257), (1024, 300), (1025, 513), (1537, 600), (2600, 260)])
+def test_precond_qr_fp64_block_products_over_chunks(s, n):
+    """More than 256 columns: the block's products V^T [V C] over one to six
+    chunks of 512 rows, the last one ragged, columns graded over 2^+-60: the bound
+    of test_precond_qr_fp64_rows_per_lane, and R times a power of two exactly."""
+    rng = np.random.default_rng(3 * s + n)
+    B = rng.standard_normal((s, n))
+    g = np.exp2(rng.integers(-60, 61, n))
+    R, info = lsq.precond_qr(dev_colmajor(B * g), None, O.FP64)
+    R = to_np(R)
+    assert int(to_np(info)[0]) == 0
+    Ro = np.linalg.qr(B, mode="r")
+    Ro *= np.sign(np.diag(Ro))[:, None]
+    err = np.linalg.norm(R / g - Ro, axis=0) / np.linalg.norm(Ro, axis=0)
+    assert err.max() <= 20 * n * U64 * O.kappa(B), err.max()
+    R2, _ = lsq.precond_qr(dev_colmajor(B * g * 2.0**-30), None, O.FP64)
+    np.testing.assert_array_equal(to_np(R2), R * 2.0**-30)
+
+
 def test_precond_qr_fp64_triangular_input():
     """Columns that are zero below the diagonal already (sigma = 0) with
     diagonal entries of either sign: R is the input with its rows' signs
