@@ -4,6 +4,7 @@ kernels, same inputs), replays reuse the graph and see new data, AUTO
 precisions are resolved per problem, and the results meet the solution
 tolerance against the oracle."""
 import ctypes as C
+import threading
 
 import numpy as np
 import pytest
@@ -222,6 +223,70 @@ def test_batched_sketch_refuses_the_transform_order_before_any_runs():
     with pytest.raises(lsq.LsqError):
         lsq.sketch_batched([small, big], [os_, ob])
     assert lsq.launch_count() == n0
+
+
+def test_new_batches_in_a_row_without_synchronisation():
+    """Batches never seen before, one after another on one stream and on two,
+    each enqueued while the ones before still run (and while their graphs are
+    captured), then all of them again as replays: the bits of single calls."""
+    sets = []
+    for k in range(4):
+        probs, opts = make_batch(5, 30 + k)
+        sets.append((opts, batch_buffers(probs, opts)))
+    want = [[to_np(lsq.pne(A, b, opts=o)[0]).copy() for A, b, o in zip(bufs[0], bufs[1], opts)] for opts, bufs in sets]
+    other = torch.cuda.Stream()
+    for streams in ([None] * 4, [None, other, None, other], [None] * 4):
+        for _, bufs in sets:
+            for x in bufs[2]:
+                x.fill_(float("nan"))
+        torch.cuda.synchronize()
+        for st, (_, bufs) in zip(streams, sets):
+            with torch.cuda.stream(st):
+                lsq.solve_batched(bufs[4], bufs[5])
+        torch.cuda.synchronize()
+        for (_, bufs), ws in zip(sets, want):
+            for x, w, info in zip(bufs[2], ws, bufs[3]):
+                assert int(to_np(info)[0]) == 0
+                np.testing.assert_array_equal(to_np(x), w)
+
+
+def test_new_batches_from_two_threads():
+    """Two threads, each with a stream and alternating between two batches of its
+    own, so that every call meets the other thread's graph in the cache."""
+    work = []
+    for t in range(2):
+        mine = []
+        for k in range(2):
+            probs, opts = make_batch(4, 40 + 2 * t + k)
+            bufs = batch_buffers(probs, opts)
+            mine.append((bufs, [to_np(lsq.pne(A, b, opts=o)[0]).copy() for A, b, o in zip(bufs[0], bufs[1], opts)]))
+        work.append(mine)
+    torch.cuda.synchronize()
+    bad = []
+
+    def run(mine):
+        try:
+            st = torch.cuda.Stream()
+            with torch.cuda.stream(st):
+                for _ in range(3):
+                    for bufs, want in mine:
+                        for x in bufs[2]:
+                            x.fill_(float("nan"))
+                        lsq.solve_batched(bufs[4], bufs[5])
+                        st.synchronize()
+                        for x, w in zip(bufs[2], want):
+                            if not np.array_equal(x.cpu().numpy(), w):
+                                bad.append("bits")
+        except Exception as e:
+            bad.append(repr(e))
+
+    threads = [threading.Thread(target=run, args=(m,)) for m in work]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join(120)
+        assert not th.is_alive()
+    assert not bad, bad
 
 
 def test_autotuner_picks_a_candidate(tmp_path):
