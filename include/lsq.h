@@ -583,7 +583,7 @@ lsq_status lsq_pne_solve_learned(const double* A, int64_t m, int64_t n, int64_t 
 
 /* ---- Instrumentation (no counterpart in the paper) --------------------- */
 
-/* Route Gaussian sketches in FP8-e4m3 / BF16 / FP16 to the tensor-core
+/* Route Gaussian sketches in FP8-e4m3 / BF16 / FP16 / FP32 to the tensor-core
  * kernel (enable = 1, the default) or to the CUDA-core GEMM (0); returns
  * the previous setting.  Process-wide; for tests and comparisons. */
 int32_t lsq_set_tensor_core_sketch(int32_t enable);
@@ -611,8 +611,9 @@ int64_t lsq_launch_count(void);
  * per stage (flops: 36 digit-pair products of 2 M N K each for the update
  * kernel, 21 for its three-digit form, the Householder panel flops for the
  * QR panel, 2 M N K of the
- * launch's K for the sketch GEMM, which is six times the product's for an
- * FP32 sketch of BF16 pieces; 0 for the steps).
+ * launch's K for the sketch GEMM, which is three times the product's for an
+ * FP32 sketch of FP16 pieces and six times for one of BF16 pieces; 0 for the
+ * steps).
  * Host-side state, not thread safe across concurrent solves on different
  * streams. */
 int32_t lsq_profile(int32_t enable);

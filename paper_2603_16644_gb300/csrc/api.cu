@@ -152,7 +152,7 @@ struct SketchLayout {
 constexpr int64_t kSketchChunk = 960;  // K chunk of the FP64 sketch (three-digit Omega; OT_KMAX3 in oz_trsm.cu)
 
 // The Gaussian sketch on the tensor cores: FP64 by digit slicing (switch
-// lsq_set_fp64_emulation), FP32 as BF16 pieces (lsq_set_tensor_core_sketch).
+// lsq_set_fp64_emulation), FP32 as FP16 or BF16 pieces (lsq_set_tensor_core_sketch).
 bool gauss_fp64_tc(int prec) { return prec == LSQ_FP64 && g_fp64_emulation && ot_trsm_supported(); }
 // FP32 Gaussian sketches of at least this many rows take two FP16 pieces per
 // value (three products), shorter ones three BF16 pieces (six).  Relative error

@@ -103,8 +103,8 @@ __device__ __forceinline__ uint32_t ot_digit_pair(unsigned long long W0, unsigne
 }
 
 // Rows of X (m x K, column-major): Ex[i] and digit planes Z[(t mp + i) Kp + k]
-// (K-contiguous; zero for rows m <= i < mp and for K <= k < Kp, so that every
-// TMA box lies inside the planes), with the row exponents from per-block
+// (K-contiguous; zero for rows m <= i < mp and for K <= k < Kp), with the row
+// exponents from per-block
 // exponents (Eblk[b m + i] for blocks b0 .. b0+nbk-1, INT32_MIN for an
 // all-zero block): a 2-D grid, one thread per row and 64-wide range of K
 // (blockIdx.y), so that many loads are in flight.  zdiv ranges form a K chunk
@@ -187,7 +187,7 @@ constexpr int OT_RS_THREADS = 256;  // 4 per row, 16 columns each
 // columns, zero outside) into shared memory [64 columns][64 rows]; otherwise
 // every thread loads its values (coalesced over rows, a column at a time).
 // own_exp (with tma_x, K <= 64): the row exponents are those of the rows'
-// largest values, formed here (the two threads of a row combine their maxima)
+// largest values, formed here (the four threads of a row combine their maxima)
 // instead of from the diagonal kernel's per-block exponents.
 template <bool tma_x, bool own_exp>
 __global__ void __launch_bounds__(OT_RS_THREADS, 3) k_ot_rowslice_s(const __grid_constant__ CUtensorMap tmZ,
@@ -1409,8 +1409,10 @@ size_t ot_trsm_ws_bytes(int64_t m, int64_t n) {
     return ot_eblk_offset(m, n) + align_up(sizeof(int32_t) * (size_t)m * ceil_div(n, OT_NB), 256) + 512;
 }
 
-// Digit planes as a 3-D tensor (k, row, digit); Kp and rows are multiples of
-// the box, so no box reaches outside.
+// Digit planes as a 3-D tensor (k, row, digit).  Kp and rows are multiples of the
+// box, so that a box lies inside or wholly outside: the second half of a 256-row
+// or 128-column tile, tiles of the lower-triangle list and the last K chunk of a
+// long product read outside, and count on the zeros that the TMA fills in.
 static bool ot_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t rows, int box_rows) {
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return false;
