@@ -205,10 +205,6 @@ __device__ __forceinline__ void load4(const double* p, double (&o)[4]) {
 }
 
 __device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) { *(float4*)p = make_float4(a, b, c, d); }
-__device__ __forceinline__ void store4(double* p, double a, double b, double c, double d) {
-    *(double2*)p = make_double2(a, b);
-    *(double2*)(p + 2) = make_double2(c, d);
-}
 
 // sum_{q < QCL} x[q * stride], pairwise (the same order in every CTA)
 template <typename T, int QCL>
@@ -267,8 +263,9 @@ __device__ __forceinline__ double qr_rcp(double d) {
     return ed < 1021 ? __longlong_as_double(__double_as_longlong(y) - ((long long)ed << 52)) : 1.0 / d;
 }
 
-// QCL: CTAs per cluster (1 to 16; 16 is non-portable, else 8).  Dynamic shared memory: the local panel (Rp x QNB) and, in the fused
-// form, the previous panel's reflector rows and the partial products behind it.
+// QCL: CTAs per cluster (1 to 16; 16 is non-portable, else 8).  Dynamic shared
+// memory: the local panel (Rp x QNB) and, in the fused form, the previous panel's
+// reflector rows and the partial products behind it.
 template <typename T, int QCL>
 __global__ void __launch_bounds__(QCT)
     k_qr_panel_cl(T* __restrict__ W, int64_t ld, int64_t s, int64_t k0, int nb, T* __restrict__ beta_out,
@@ -680,8 +677,8 @@ __global__ void __launch_bounds__(QCT)
         // from lane jj and, after the update, column jj + 1 from lane jj + 1 by
         // shuffles, and forms v, the update and the next dots itself (no
         // divergent single-lane phases, no shared-memory round trips).
-        // Measured: the FP64 path 6.2 -> 23.5 solves/s; for FP32 the
-        // shared-memory form below is faster (3.07 against 4.55 ms per solve).
+        // Measured: the FP64 path 6.2 -> 23.5 solves/s; FP32 broadcasts through
+        // shared memory below, which is faster there (3.07 against 4.55 ms per solve).
         // The loops run over QR = 4, 8, ... 32 rows per lane, the fewest that hold
         // the warp's rows: the FP64 pipe takes 16 cycles an instruction and SM, so
         // masked rows are not free (a panel's column costs ~11 thousand cycles
@@ -1393,10 +1390,11 @@ static bool qu_cluster16_ok() {
 }
 
 // C (rows x nt, ld s) <- (I - V T^T V^T) C.  A cluster per 32 columns; FP64
-// updates of few columns (the in-block updates of the blocked FP64 QR: at
-// most 7 column tiles, 56 CTAs with 8 per cluster) take 16 CTAs per cluster
-// when there are rows for 16 (2048 or more), so that twice the SMs share
-// them.
+// updates of few columns (at most 7 column tiles, 56 CTAs with 8 per cluster)
+// take 16 CTAs per cluster when there are rows for 16 (2048 or more), so that
+// twice the SMs share them.  That is the unblocked FP64 QR (n <= 256, or the
+// digit-sliced products off): the blocked one spreads such updates over the chip
+// (qr_apply_wide below), with scratch that the unblocked one does not have.
 template <typename T>
 static lsq_status qr_apply(const T* V, const T* Tm, int nb, int64_t rows, T* C, int64_t s, int64_t nt,
                            cudaStream_t st) {
