@@ -490,6 +490,7 @@ __global__ void __launch_bounds__(1024) k_lu_panel(T* __restrict__ H, int64_t ld
                 if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
             }
             if (lane == 0) {
+                if (bi >= rows) bi = j;  // NaN in every row: a pivot that is reported below
                 pivrow = bi;
                 piv[j] = (int32_t)bi;
             }

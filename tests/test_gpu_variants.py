@@ -123,3 +123,23 @@ def test_srft_solve_matches_oracle(hpne, m, n, kap, rho, prec):
     more = oracle_realizations(pr, hpne=hpne, **kw)
     assert_solution_parity(to_np(x), ref["x"], pr.x_star, kap, rho, "srft", refined=False, u_p=prec,
                            realizations=more)
+
+
+@pytest.mark.parametrize("prec", [lsq.FP32, lsq.FP64])
+@pytest.mark.parametrize("c", [0, 17, 32])
+def test_nne_reports_a_nan_column_of_a_tall_sketch(prec, c):
+    """A column that is NaN in every row of a sketch taller than the LU panel's
+    clusters hold (8192 rows): its index is reported, with the pivots in range."""
+    m, n, s = 8400, 33, 8300
+    g = torch.Generator(device="cuda").manual_seed(c)
+    A = torch.randn((n, m), generator=g, dtype=torch.float64, device="cuda").t()
+    A[5, c] = float("nan")
+    b = torch.randn(m, generator=g, dtype=torch.float64, device="cuda")
+    opts = lsq.make_opts(kind=lsq.GAUSSIAN, s=s, seed=1, sketch_prec=prec, qr_prec=prec)
+    x, info = lsq.solve(A, b, method="nne_lu", opts=opts)
+    assert int(to_np(info)[0]) == c + 1
+    A[5, c] = 1.0
+    x, info = lsq.solve(A, b, method="nne_lu", opts=opts)
+    assert int(to_np(info)[0]) == 0
+    ref = torch.linalg.lstsq(A.contiguous(), b[:, None]).solution[:, 0]
+    assert float((x - ref).norm() / ref.norm()) <= 1e-10
