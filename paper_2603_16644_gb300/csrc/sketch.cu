@@ -605,6 +605,10 @@ __device__ __forceinline__ float quant_f32(double a, int e) {
     else return __uint_as_float(q);
 }
 
+__device__ __forceinline__ double flip_sign(double v, int on) {
+    return __longlong_as_double(__double_as_longlong(v) ^ (on ? (long long)0x8000000000000000ull : 0ll));
+}
+
 // Rounding, signs, padding and the levels h = 1 .. B/2 for B = min(m', 4096)
 // consecutive rows of a column: one read of A and one write of W.  HBM bound
 // (8 bytes read and 4 written per element).  A thread holds 16 entries, all 16
@@ -613,6 +617,10 @@ __device__ __forceinline__ float quant_f32(double a, int e) {
 // shared memory).  A separate load that rounded one entry at a time with a
 // run-time precision, and a transform with a pass over shared memory and two
 // barriers per level, took 525 + 377 us for 100000 x 400 to FP32; this 120 us.
+// FP64 is bound by its additions (a warp instruction in 16 cycles an SM): a select of
+// a sum and a difference issues both, and idle warps add their zeros.  With the sign
+// flipped instead and no warps without entries a sketch of 200000 x 200 takes 2.13
+// ms (2.62 before; the separate load and transform 2.08), 2000 x 1000 97 us (179; 95).
 template <typename T, int PREC>
 __global__ void __launch_bounds__(256) k_srft_block(const double* __restrict__ A, int64_t m, int64_t lda,
                                                     const int32_t* __restrict__ colexp, uint64_t seed, int64_t mp,
@@ -643,21 +651,25 @@ __global__ void __launch_bounds__(256) k_srft_block(const double* __restrict__ A
         // the padding stays +0
         if (((w >> lane) & 1u) && b0 + i0 + 32 * k < m) v[k] = -v[k];
     }
+    // FP64: one addition an entry and level, none for the entries past B
+    constexpr bool F64 = PREC == LSQ_FP64;
 #pragma unroll
     for (int h = 1; h < 32; h <<= 1) {
         if (h >= B) break;
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const T o = __shfl_xor_sync(0xffffffffu, v[k], h);
-            v[k] = (lane & h) ? o - v[k] : v[k] + o;
-        }
+        for (int k = 0; k < 16; ++k)
+            if (!F64 || 32 * k < B) {
+                const T o = __shfl_xor_sync(0xffffffffu, v[k], h);
+                if constexpr (F64) v[k] = o + flip_sign(v[k], lane & h);
+                else v[k] = (lane & h) ? o - v[k] : v[k] + o;
+            }
     }
 #pragma unroll
     for (int h = 1; h < 16; h <<= 1) {
         if (32 * h >= B) break;
 #pragma unroll
         for (int k = 0; k < 16; ++k)
-            if (!(k & h)) {
+            if (!(k & h) && (!F64 || 32 * k < B)) {
                 const T p = v[k], q = v[k + h];
                 v[k] = p + q;
                 v[k + h] = p - q;
@@ -673,9 +685,8 @@ __global__ void __launch_bounds__(256) k_srft_block(const double* __restrict__ A
 #pragma unroll
     for (int k = 0; k < 16; ++k) x[i0 + 32 * k] = v[k];
     __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int l = t + 256 * r;
+#pragma unroll 2
+    for (int l = t; l < 512; l += F64 ? (int)blockDim.x : 256) {
         T u[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) u[k] = x[l + 512 * k];
@@ -684,7 +695,7 @@ __global__ void __launch_bounds__(256) k_srft_block(const double* __restrict__ A
             if (512 * h >= B) break;
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-                if (!(k & h)) {
+                if (!(k & h) && (!F64 || 512 * k < B)) {
                     const T p = u[k], q = u[k + h];
                     u[k] = p + q;
                     u[k + h] = p - q;
@@ -749,7 +760,9 @@ static lsq_status srft_run(const double* A, int64_t m, int64_t n, int64_t lda, c
                            int64_t s, T* W, void* As, int64_t ldas, cudaStream_t st) {
     const int64_t mp = srft_order(m);
     if (!srft_fits(m, PREC)) return LSQ_ERR_ARG;
-    k_srft_block<T, PREC><<<dim3((unsigned)ceil_div(mp, FW_B), (unsigned)n), 256, 0, st>>>(A, m, lda, colexp, seed, mp, W);
+    // FP64: the warps that have entries (16 a thread)
+    const int threads = PREC == LSQ_FP64 ? (int)std::min<int64_t>(256, std::max<int64_t>(32, mp / 16)) : 256;
+    k_srft_block<T, PREC><<<dim3((unsigned)ceil_div(mp, FW_B), (unsigned)n), threads, 0, st>>>(A, m, lda, colexp, seed, mp, W);
     LSQ_LAUNCH_CHECK();
     // the levels above: at most five at a time
     for (int64_t h = FW_B; h < mp;) {
