@@ -40,10 +40,14 @@ constexpr int OT_BM = 128, OT_BN = 64;      // output tile (rows x columns)
 constexpr int OT_BK = 64;                   // K per stage: 64 BF16 = 128 bytes
 constexpr int OT_XST = 6;                   // stages of X digit tiles
 constexpr int OT_KMAX = 512;                // exact FP32 group sums up to this K
-// With three X digits (at most 3 pairs per group) the FP32 sums would be exact
-// up to K = 1024; the 64-bit sums of k_ot_update2, K 2^53 (1 + 2/128 + ...) in
-// magnitude, bound K to 1003: 15 slabs of 64.
-constexpr int OT_KMAX3 = 960;
+// With three X digits (at most 3 pairs per group) the FP32 sums are exact up to K =
+// 1024.  So are the epilogue's 64-bit sums (floor(I / 2^8)): with X = -q 2^-17, |q| <=
+// 2^20 - 1, on the fixed exponent 3, |V_x| <= 2^55 - 2^35, |V_y| <= 2^55, and the
+// pairs left out (t + u > 7) add up to 65 a product, so that |I| <= K (2^61 - 2^41 + 65)
+// < 2^71, and the last step's partial value lies within 2^23 of floor(I / 2^8).
+// (960 from a bound digit by digit took a second chunk for up to 64 rows more: a
+// 1000 x 100 sketch 121 us, 97 with 1024.)
+constexpr int OT_KMAX3 = 1024;
 constexpr int OT_NB = 32;                   // diagonal block solved by substitution
 constexpr int OT_THREADS = 608;             // warp 0 TMA, warps 1-2 MMA, warps 3-18 epilogue
 constexpr int OT_XTILE = OT_BM * 128;       // bytes of one X digit tile
