@@ -462,7 +462,8 @@ size_t lsq_batched_workspace_size(int32_t hpne, int32_t count, const lsq_batch_p
  * the descriptors (pointers, shapes, options, workspace), the process-wide
  * switches and the reduction hook stay the same.  A
  * call with new descriptors enqueues the fan-out directly (forked from and
- * joined to `stream`) and captures the graph while the GPU works; a CUDA error
+ * joined to `stream`) and captures the graph while the GPU works, or, for many
+ * small problems, captures it first and launches it; a CUDA error
  * while it enqueues leaves the outputs undefined, and what a single solve
  * refuses is refused before any problem runs.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
  * batched condition-estimate pass (the same fan-out, in a cached graph of

@@ -176,8 +176,15 @@ lsq_status enqueue_fanout(cudaStream_t from, const std::vector<int>& order, cons
 
 // Whether a new fan-out is enqueued directly before it is captured: not when the
 // caller's own stream is being captured, nor while a reduction hook or the
-// stage timing would see every step twice.
-bool direct_ok(cudaStream_t st) {
+// stage timing would see every step twice, nor for many small problems (mean
+// work 2 m n^2 below 4e7).  Those finish before the host has enqueued them, so that
+// enqueuing them and then capturing them costs the host twice: alternating
+// batches of 64 problems, precision from the estimate on a sketch, 2000 x 32 38.4 ms
+// so and 30.6 captured first, 4000 x 48 38.8 and 34.5, 4000 x 100 about equal, and 8000
+// x 150 directly 49 to 53 against about 58; eight 2000 x 32 4.4 both ways, four 2.6
+// directly and 2.8 captured first.
+bool direct_ok(cudaStream_t st, size_t count, double mean_work) {
+    if (count > 8 && mean_work < 4e7) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
         cudaGetLastError();
@@ -188,8 +195,8 @@ bool direct_ok(cudaStream_t st) {
 
 // A fan-out of per-problem work over the internal streams, run(i, stream, slot)
 // enqueuing problem i: one graph (cached in `cache` under `key`) launched on st.
-// Under a new key the work is enqueued on the internal streams directly and
-// the graph captured while the GPU runs it: capturing and instantiating the
+// Under a new key the work is enqueued on the internal streams directly (direct_ok)
+// and the graph captured while the GPU runs it: capturing and instantiating the
 // thousands of launches of 64 solves takes ~46 ms of host time, which the GPU
 // waited for (145 ms a pass over ever new batches of 64 uneven problems, 113
 // now; 99 ms when the same batch is repeated).  No step of a problem forks onto
@@ -198,14 +205,15 @@ bool direct_ok(cudaStream_t st) {
 // kernels.  Caller holds g_batch.mu.
 template <typename F>
 lsq_status capture_fanout(GraphCache& cache, const std::vector<int>& order, const std::vector<int>& stream_of,
-                          char* slots, size_t slot_bytes, std::vector<unsigned char>& key, cudaStream_t st, F run) {
+                          char* slots, size_t slot_bytes, std::vector<unsigned char>& key, double mean_work,
+                          cudaStream_t st, F run) {
     if (cache.exec && key == cache.key) {
         LSQ_CUDA_TRY(cudaGraphLaunch(cache.exec, st));
         return LSQ_OK;
     }
     cache.drop();
     FanoutScope scope;
-    const bool direct = direct_ok(st);
+    const bool direct = direct_ok(st, order.size(), mean_work);
     if (direct) {
         lsq_status r = enqueue_fanout(st, order, stream_of, slots, slot_bytes, run);
         if (r != LSQ_OK) return r;
@@ -294,7 +302,9 @@ lsq_status batched(bool hpne, int32_t count, const lsq_batch_problem* probs, voi
         std::vector<unsigned char> ekey(sizeof(lsq_batch_problem) * count);
         std::memcpy(ekey.data(), probs, sizeof(lsq_batch_problem) * count);
         key_tail(ekey, ws, ws_bytes, 0);
-        r = capture_fanout(g_est, est_order, P.stream_of, slots, P.slot_bytes, ekey, st,
+        double ework = 0.0;
+        for (int i : est_order) ework += work_of(q[i]);
+        r = capture_fanout(g_est, est_order, P.stream_of, slots, P.slot_bytes, ekey, ework / (double)est_order.size(), st,
                            [&](int i, cudaStream_t sk, char* slot) {
                                if (q[i].opts.sketch_prec == LSQ_AUTO)
                                    return launch_condest(q[i].A, q[i].m, q[i].n, q[i].lda, k0 + i, ch + i, slot,
@@ -319,7 +329,9 @@ lsq_status batched(bool hpne, int32_t count, const lsq_batch_problem* probs, voi
     std::vector<unsigned char> key(sizeof(lsq_batch_problem) * count);
     std::memcpy(key.data(), q.data(), sizeof(lsq_batch_problem) * count);
     key_tail(key, ws, ws_bytes, hpne ? 1 : 0);
-    return capture_fanout(g_main, P.order, P.stream_of, slots, P.slot_bytes, key, st,
+    double work = 0.0;
+    for (int i = 0; i < count; ++i) work += work_of(q[i]);
+    return capture_fanout(g_main, P.order, P.stream_of, slots, P.slot_bytes, key, work / count, st,
                           [&](int i, cudaStream_t sk, char* slot) {
                               return solve_impl_ext(hpne, q[i].A, q[i].m, q[i].n, q[i].lda, q[i].b, &q[i].opts,
                                                     q[i].x, nullptr, q[i].info, slot, P.slot_bytes, sk, nullptr);
@@ -366,7 +378,9 @@ lsq_status batched_steps(int tag, int32_t count, const Prob* probs, void* ws, si
     std::vector<unsigned char> key(sizeof(Prob) * count);
     std::memcpy(key.data(), probs, sizeof(Prob) * count);
     key_tail(key, ws, ws_bytes, tag);
-    return capture_fanout(g_main, order, stream_of, base, slot, key, st,
+    double sum = 0.0;
+    for (double w : work) sum += w;
+    return capture_fanout(g_main, order, stream_of, base, slot, key, sum / count, st,
                           [&](int i, cudaStream_t sk, char* sl) { return run(probs[i], sl, slot, sk); });
 }
 

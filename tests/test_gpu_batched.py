@@ -227,11 +227,12 @@ def test_batched_sketch_refuses_the_transform_order_before_any_runs():
 
 def test_new_batches_in_a_row_without_synchronisation():
     """Batches never seen before, one after another on one stream and on two,
-    each enqueued while the ones before still run (and while their graphs are
-    captured), then all of them again as replays: the bits of single calls."""
+    each enqueued while the ones before still run (of three problems directly,
+    with the graph captured behind; of ten small ones as a graph), then all of
+    them again: the bits of single calls."""
     sets = []
     for k in range(4):
-        probs, opts = make_batch(5, 30 + k)
+        probs, opts = make_batch(3, 30 + k) if k < 3 else make_batch(10, 47)
         sets.append((opts, batch_buffers(probs, opts)))
     want = [[to_np(lsq.pne(A, b, opts=o)[0]).copy() for A, b, o in zip(bufs[0], bufs[1], opts)] for opts, bufs in sets]
     other = torch.cuda.Stream()
@@ -257,7 +258,7 @@ def test_new_batches_from_two_threads():
     for t in range(2):
         mine = []
         for k in range(2):
-            probs, opts = make_batch(4, 40 + 2 * t + k)
+            probs, opts = make_batch(3, 40 + 2 * t + k)
             bufs = batch_buffers(probs, opts)
             mine.append((bufs, [to_np(lsq.pne(A, b, opts=o)[0]).copy() for A, b, o in zip(bufs[0], bufs[1], opts)]))
         work.append(mine)
