@@ -456,16 +456,13 @@ size_t lsq_batched_workspace_size(int32_t hpne, int32_t count, const lsq_batch_p
 /* Alg. 1 with PNE (Eq. e_pne) or HPNE (Eq. e_hpne) on `count` independent
  * problems.  The problems are spread over 16 internal streams (or
  * $LSQ_BATCH_STREAMS, 1 to 64, read once per process; the workspace size
- * grows with it), heaviest first to the least-loaded stream, and the whole
- * fan-out is captured into one
- * CUDA graph; the executable graph is cached and replayed on `stream` while
- * the descriptors (pointers, shapes, options, workspace), the process-wide
- * switches and the reduction hook stay the same.  A
- * call with new descriptors enqueues the fan-out directly (forked from and
- * joined to `stream`) and captures the graph while the GPU works, or, for many
- * small problems, captures it first and launches it; a CUDA error
- * while it enqueues leaves the outputs undefined, and what a single solve
- * refuses is refused before any problem runs.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
+ * grows with it), heaviest first to the least-loaded stream, forked from and
+ * joined to `stream`.  When a call has the descriptors (pointers, shapes, options,
+ * workspace), process-wide switches and reduction hook of the call before it, the
+ * whole fan-out is captured into one CUDA graph, and the executable graph is
+ * replayed on `stream` in the calls after that.  A CUDA error while a call
+ * enqueues leaves the outputs undefined; what a single solve refuses is refused
+ * before any problem runs.  Problems with sketch_prec = AUTO or AUTO_SKETCH first get one
  * batched condition-estimate pass (the same fan-out, in a cached graph of
  * its own) and one readback of the chosen precisions (a stream
  * synchronisation).  Each problem's status goes to its own info.

@@ -465,8 +465,8 @@ def batched_workspace(desc, hpne=False, device=None):
 
 
 def solve_batched(desc, ws, hpne=False):
-    """Alg. 1 on every problem of `desc` (from batch_descriptors): one cached
-    CUDA-graph launch of all solves over 16 internal streams."""
+    """Alg. 1 on every problem of `desc` (from batch_descriptors), over 16
+    internal streams; a repeated batch is one cached CUDA-graph launch."""
     L = _batch_sigs()
     fn = L.lsq_hpne_solve_batched if hpne else L.lsq_pne_solve_batched
     _check(fn(len(desc), desc, _ptr(ws), ws.numel(), _stream()), "lsq_solve_batched")

@@ -1,18 +1,17 @@
 // Batched PNE / HPNE (Alg. 1 on many independent problems of uneven shape).
 //
 // The problems are spread over a fixed set of internal streams (heaviest
-// first, each to the least-loaded stream), and the whole fan-out -- every
-// kernel of every problem plus the fork/join events -- is captured into one
-// CUDA graph.  The executable graph is cached and replayed while the batch
-// description is unchanged, so a repeated batched call is one graph launch on
-// the caller's stream; a call with a new description enqueues the fan-out on
-// the internal streams and captures it while the GPU works.  Problems asking
-// for the AUTO
+// first, each to the least-loaded stream).  A batch seen for the first time is
+// enqueued there, forked from and joined to the caller's stream by events; when the
+// same batch (descriptors, workspace, settings) comes again the whole fan-out -- every
+// kernel of every problem plus the fork/join events -- is captured into one CUDA
+// graph, and from then on a call is one graph launch on the caller's stream.
+// Problems asking for the AUTO
 // precision first get one batched condition-estimate pass (Sec. 6.1; on A^T A
 // for AUTO, on a sketch for AUTO_SKETCH) and a single readback of the chosen
 // precisions, because kernel selection in the captured graph needs them on
 // the host.  The batched sketch and preconditioner QR (lsq_sketch_batched,
-// lsq_precond_qr_batched) use the same captured fan-out.
+// lsq_precond_qr_batched) use the same fan-out.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -63,6 +62,7 @@ BatchState g_batch;
 struct GraphCache {
     cudaGraphExec_t exec = nullptr;
     std::vector<unsigned char> key;
+    std::vector<unsigned char> seen;  // of the last batch that was enqueued without a graph
     void drop() {
         if (exec) cudaGraphExecDestroy(exec);
         exec = nullptr;
@@ -81,8 +81,10 @@ lsq_status ensure_streams() {
     LSQ_CUDA_TRY(cudaEventCreateWithFlags(&g_batch.fork, cudaEventDisableTiming));
     LSQ_CUDA_TRY(cudaStreamCreateWithFlags(&g_batch.cap, cudaStreamNonBlocking));
     g_batch.dev = dev;
-    g_main.drop();
-    g_est.drop();
+    for (GraphCache* c : {&g_main, &g_est}) {
+        c->drop();
+        c->seen.clear();
+    }
     return LSQ_OK;
 }
 
@@ -174,17 +176,10 @@ lsq_status enqueue_fanout(cudaStream_t from, const std::vector<int>& order, cons
     return r;
 }
 
-// Whether a new fan-out is enqueued directly before it is captured: not when the
-// caller's own stream is being captured, nor while a reduction hook or the
-// stage timing would see every step twice, nor for many small problems (mean
-// work 2 m n^2 below 4e7).  Those finish before the host has enqueued them, so that
-// enqueuing them and then capturing them costs the host twice: alternating
-// batches of 64 problems, precision from the estimate on a sketch, 2000 x 32 38.4 ms
-// so and 30.6 captured first, 4000 x 48 38.8 and 34.5, 4000 x 100 about equal, and 8000
-// x 150 directly 49 to 53 against about 58; eight 2000 x 32 4.4 both ways, four 2.6
-// directly and 2.8 captured first.
-bool direct_ok(cudaStream_t st, size_t count, double mean_work) {
-    if (count > 8 && mean_work < 4e7) return false;
+// Whether a fan-out may be enqueued without a graph: not when the caller's own
+// stream is being captured, nor while a reduction hook or the stage timing would
+// see every step twice when it is captured behind.
+bool direct_ok(cudaStream_t st) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
         cudaGetLastError();
@@ -194,15 +189,19 @@ bool direct_ok(cudaStream_t st, size_t count, double mean_work) {
 }
 
 // A fan-out of per-problem work over the internal streams, run(i, stream, slot)
-// enqueuing problem i: one graph (cached in `cache` under `key`) launched on st.
-// Under a new key the work is enqueued on the internal streams directly (direct_ok)
-// and the graph captured while the GPU runs it: capturing and instantiating the
-// thousands of launches of 64 solves takes ~46 ms of host time, which the GPU
-// waited for (145 ms a pass over ever new batches of 64 uneven problems, 113
-// now; 99 ms when the same batch is repeated).  No step of a problem forks onto
-// the library's shared look-ahead streams here (FanoutScope; captured or
-// not), so concurrent problems never share a stream and both ways run the same
-// kernels.  Caller holds g_batch.mu.
+// enqueuing problem i, cached as a graph in `cache` under `key`.  A batch that is not
+// the last call's is enqueued on the internal streams directly; when it comes again it
+// is captured (large problems, mean work 2 m n^2 from 1e9, directly once more and
+// captured while the GPU runs them); from then on the graph is launched on st.
+// Capturing and instantiating the thousands of launches of 64 solves takes ~46 ms of
+// host time, which the GPU waited for when every new batch was captured first, and which
+// came on top of enqueuing it when it was captured behind.  64 problems, another batch
+// each call, precision from the estimate on a sketch, captured first / behind / not:
+// 2000 x 32 33 / 43 / 16 ms, 16000 x 250 106 / 75 / 52 ms, the uneven ones 145 / 111 / 93
+// (94 when the same batch is repeated).
+// No step of a problem forks onto the library's shared look-ahead streams here
+// (FanoutScope; captured or not), so concurrent problems never share a stream and both
+// ways run the same kernels.  Caller holds g_batch.mu.
 template <typename F>
 lsq_status capture_fanout(GraphCache& cache, const std::vector<int>& order, const std::vector<int>& stream_of,
                           char* slots, size_t slot_bytes, std::vector<unsigned char>& key, double mean_work,
@@ -211,13 +210,18 @@ lsq_status capture_fanout(GraphCache& cache, const std::vector<int>& order, cons
         LSQ_CUDA_TRY(cudaGraphLaunch(cache.exec, st));
         return LSQ_OK;
     }
-    cache.drop();
     FanoutScope scope;
-    const bool direct = direct_ok(st, order.size(), mean_work);
+    const bool first = key != cache.seen;
+    const bool direct = direct_ok(st) && (first || mean_work >= 1e9);
     if (direct) {
         lsq_status r = enqueue_fanout(st, order, stream_of, slots, slot_bytes, run);
         if (r != LSQ_OK) return r;
+        if (first) {
+            cache.seen.swap(key);
+            return LSQ_OK;
+        }
     }
+    cache.drop();
     cudaGraph_t graph = nullptr;
     // Capture on an internal stream (the caller may use the legacy default
     // stream, which cannot be captured); the graph is then launched on st.

@@ -134,7 +134,8 @@ def test_batched_follows_the_switches(switch, auto):
     for o in opts:
         o.kind, o.sketch_prec, o.qr_prec = lsq.GAUSSIAN, lsq.AUTO if auto else lsq.FP32, lsq.FP32
     As, bs, xs, infos, desc, ws = batch_buffers(probs, opts)
-    lsq.solve_batched(desc, ws)
+    for _ in range(3):  # enqueued, captured, replayed
+        lsq.solve_batched(desc, ws)
     first = [to_np(x).copy() for x in xs]
     prev = switch(False)
     try:
@@ -156,7 +157,8 @@ def test_batched_follows_the_reduction_hook():
     no more once it is removed."""
     probs, opts = make_batch(3, 22)
     As, bs, xs, infos, desc, ws = batch_buffers(probs, opts)
-    lsq.solve_batched(desc, ws)
+    for _ in range(3):  # enqueued, captured, replayed
+        lsq.solve_batched(desc, ws)
     first = [to_np(x).copy() for x in xs]
     calls = []
     lsq.set_reduce_hook(lambda buf, count, kind, stream: calls.append(count) or 0)
@@ -175,7 +177,8 @@ def test_batched_follows_the_reduction_hook():
 
 def test_batched_launches_are_counted_once():
     """lsq_launch_count over a new batch is the sum over single calls (problems
-    of one QR panel, where both run the same kernels), and a replay adds none."""
+    of one QR panel, where both run the same kernels), as over the call that captures
+    it, also where it is enqueued and captured behind; a replay adds none."""
     probs, opts = [], []
     for i in range(3):
         probs.append(P.make_problem(900 + 100 * i, 30, 1e3, 1e-6, 77 + i))
@@ -189,7 +192,21 @@ def test_batched_launches_are_counted_once():
     n2 = lsq.launch_count()
     assert n2 - n1 == n1 - n0 > 0
     lsq.solve_batched(desc, ws)
+    assert lsq.launch_count() - n2 == n1 - n0
+    n2 = lsq.launch_count()
+    lsq.solve_batched(desc, ws)
     assert lsq.launch_count() == n2
+    big = P.make_problem_torch(600000, 32, 1e3, 1e-6, 78)  # mean work above 1e9
+    A, b = big[0], big[1]
+    x, info = torch.zeros(32, dtype=torch.float64, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    desc = lsq.batch_descriptors([A], [b], [x], [info], [lsq.make_opts(kind=lsq.SPARSE_SIGN, s=128, zeta=8, seed=1)])
+    ws = lsq.batched_workspace(desc)
+    count = []
+    for _ in range(3):
+        n0 = lsq.launch_count()
+        lsq.solve_batched(desc, ws)
+        count.append(lsq.launch_count() - n0)
+    assert count[0] == count[1] > 0 == count[2]
 
 
 @pytest.mark.parametrize("field,value", [("refine_steps", 2), ("qr_prec", lsq.BF16), ("row_offset", -1)])
@@ -227,23 +244,24 @@ def test_batched_sketch_refuses_the_transform_order_before_any_runs():
 
 def test_new_batches_in_a_row_without_synchronisation():
     """Batches never seen before, one after another on one stream and on two,
-    each enqueued while the ones before still run (of three problems directly,
-    with the graph captured behind; of ten small ones as a graph), then all of
-    them again: the bits of single calls."""
+    each enqueued while the ones before still run; then each three times in a row
+    (enqueued, captured, replayed), again without waiting, and in turn once more:
+    the bits of single calls."""
     sets = []
     for k in range(4):
-        probs, opts = make_batch(3, 30 + k) if k < 3 else make_batch(10, 47)
+        probs, opts = make_batch(5, 30 + k)
         sets.append((opts, batch_buffers(probs, opts)))
     want = [[to_np(lsq.pne(A, b, opts=o)[0]).copy() for A, b, o in zip(bufs[0], bufs[1], opts)] for opts, bufs in sets]
     other = torch.cuda.Stream()
-    for streams in ([None] * 4, [None, other, None, other], [None] * 4):
+    for streams, calls in [([None] * 4, 1), ([None, other] * 2, 1), ([None] * 4, 3), ([None, other] * 2, 3), ([None] * 4, 1)]:
         for _, bufs in sets:
             for x in bufs[2]:
                 x.fill_(float("nan"))
         torch.cuda.synchronize()
         for st, (_, bufs) in zip(streams, sets):
             with torch.cuda.stream(st):
-                lsq.solve_batched(bufs[4], bufs[5])
+                for _ in range(calls):
+                    lsq.solve_batched(bufs[4], bufs[5])
         torch.cuda.synchronize()
         for (_, bufs), ws in zip(sets, want):
             for x, w, info in zip(bufs[2], ws, bufs[3]):
@@ -252,8 +270,8 @@ def test_new_batches_in_a_row_without_synchronisation():
 
 
 def test_new_batches_from_two_threads():
-    """Two threads, each with a stream and alternating between two batches of its
-    own, so that every call meets the other thread's graph in the cache."""
+    """Two threads, each with a stream and two batches of its own, one of them
+    three times in a row, so that calls meet the other thread's graph in the cache."""
     work = []
     for t in range(2):
         mine = []
@@ -270,7 +288,7 @@ def test_new_batches_from_two_threads():
             st = torch.cuda.Stream()
             with torch.cuda.stream(st):
                 for _ in range(3):
-                    for bufs, want in mine:
+                    for bufs, want in [mine[0]] * 3 + [mine[1]]:
                         for x in bufs[2]:
                             x.fill_(float("nan"))
                         lsq.solve_batched(bufs[4], bufs[5])
