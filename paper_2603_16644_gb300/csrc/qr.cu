@@ -725,8 +725,9 @@ __global__ void __launch_bounds__(QCT)
                 for (int q = 0; q < QR; ++q) s4[q & 3] = fma(xn[q], a[q], s4[q & 3]);
                 acc = lane < nb ? (s4[0] + s4[1]) + (s4[2] + s4[3]) : (T)0;
             }
-            for (int jj = 0; jj < nb; ++jj) {
-                const Scal sc = exchange(jj, acc, rowbuf, 1);
+            // column jj after its exchange; FAR: u scaled by 1 / v1 where needed
+            auto column = [&](int jj, const Scal& sc, auto far_tag) {
+                constexpr bool FAR = decltype(far_tag)::value;
                 if (jj > 0) scale_y(jj - 1);
                 // u_jj on this warp's rows: 0 above row jj, v1 on it, x below
                 T u[QR];
@@ -736,7 +737,7 @@ __global__ void __launch_bounds__(QCT)
                     const int gr = gr0 + q;
                     u[q] = (gr < jj || q >= nv) ? (T)0 : (gr == jj ? sc.v1 : x);
                 }
-                if (sc.far) {
+                if (FAR && sc.far) {
 #pragma unroll
                     for (int q = 0; q < QR; ++q) u[q] *= sc.rv1;
                 }
@@ -744,7 +745,7 @@ __global__ void __launch_bounds__(QCT)
                     myscale = sc.rv1;
                     myR = sc.mu;
                 }
-                rprev = sc.far ? (T)1 : sc.rv1;
+                rprev = FAR && sc.far ? (T)1 : sc.rv1;
                 // later columns: a_c -= w_c v = (w_c / v1) u
                 const bool upd = lane > jj && lane < nb && sc.b != (T)0;
                 const T f = sc.f;
@@ -763,6 +764,19 @@ __global__ void __launch_bounds__(QCT)
 #pragma unroll
                 for (int q = 0; q < QR; ++q) s4[q & 3] = fma(ylane ? u[q] : xn[q], a[q], s4[q & 3]);
                 acc = (ylane || dlane) ? (s4[0] + s4[1]) + (s4[2] + s4[3]) : (T)0;
+            };
+            // from the first far column on in a loop of its own: the branch alone
+            // cost a panel of few rows 5 %
+            int jj = 0;
+            Scal sc;
+            for (; jj < nb; ++jj) {
+                sc = exchange(jj, acc, rowbuf, 1);
+                if (sc.far) break;
+                column(jj, sc, std::false_type{});
+            }
+            while (jj < nb) {
+                column(jj, sc, std::true_type{});
+                if (++jj < nb) sc = exchange(jj, acc, rowbuf, 1);
             }
             ysc0 = myscale * rprev;  // of Y's last column, formed below
             // R on and above the diagonal, v below it
